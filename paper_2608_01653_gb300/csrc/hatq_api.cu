@@ -924,6 +924,10 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     const bool drains = a.num_kb > a.chunk_kb;
     a.buf_cols = a.n_t;
     a.nbuf = (drains || g.G == 128) ? 1 : 2;
+    const bool general = L->act == HATQ_ACT_SILU || L->act == HATQ_ACT_GELU;
+    // the lean kernels: INT8 codes of one exact chunk per tile, no further option
+    a.lean = !drains && !general && !L->out_f32 && !a.affine && !a.a_f16 && !a.out_f16 && !a.d2s;
+    a.group = g.G;
     a.tmem_cols = 512;
     a.a_col = 2 * a.n_t;
     a.seg = g.seg;
@@ -931,6 +935,7 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     const int esz = L->out_f32 ? 4 : 1;
     a.row_stride = a.n_t * esz + 16;                 // padded rows: 8 consecutive rows hit 8 bank groups
     a.staging_bytes = L->out_f32 ? 0 : a.nbuf * kTileRows * a.row_stride;   // float32 output is stored directly
+    if (a.lean) a.staging_bytes = 8 * 4096;          // two 32-row buffers of 64 columns per epilogue warp
     a.win_h = (a.th - 1) * d->stride + d->kh;
     a.win_w = (a.tw - 1) * d->stride + d->kw;
     a.win_pitch = a.win_tma ? window_box_bytes(a.tw, d->stride, d->kw, d->c_in) : (a.win_w * d->c_in + 15) & ~15;
@@ -939,7 +944,6 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     // + 16 bytes: the gather reads up to 11 bytes past a row segment
     const int win_bytes = g.gather ? a.win_buf * (a.win_tma ? 2 : 1) : 0;
     const int table_bytes = g.gather ? a.num_kb * 8 * 4 : 0;
-    const bool general = L->act == HATQ_ACT_SILU || L->act == HATQ_ACT_GELU;
     const int const_bytes = ((4 * d->c_out * 4 + 127) & ~127) + (general ? 256 : 0);
     const int fixed = 1024 /* align */ + 8 * (3 * 8 + 13) + 16 + 128 + table_bytes + const_bytes + win_bytes;
     const int budget = 227 * 1024 - 1024 /* static */ - fixed - a.staging_bytes;
@@ -968,7 +972,7 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     a.win_off = a.const_off + const_bytes;
     const int smem_bytes = a.stages * a.stage_bytes + a.staging_bytes + 1024 + a.win_off + win_bytes;
     // the exchange of a 128-wide next-layer transform uses the output tile: 2 x 128 rows x 64 bytes
-    if (g.G == 128 && L->hb_next == 128 && a.staging_bytes < 2 * kTileRows * 64)
+    if (!a.lean && g.G == 128 && L->hb_next == 128 && a.staging_bytes < 2 * kTileRows * 64)
         return fail(HATQ_ERR_UNSUPPORTED, "output tile too small for the 128-wide transition exchange");
     if (smem_bytes > 227 * 1024 - 1024) return fail(HATQ_ERR_UNSUPPORTED, "shared memory budget exceeded (%d bytes)", smem_bytes);
     if (a.affine && g.gather) return fail(HATQ_ERR_UNSUPPORTED, "affine activations need c_in % 16 == 0");
@@ -993,8 +997,27 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     a.err = err_word();
     if (!a.err) return fail(HATQ_ERR_CUDA, "no CUDA device");
 
-    CUtensorMap tmB, tmA;
+    CUtensorMap tmB, tmA, tmY;
     std::memcpy(&tmB, L->opaque, sizeof tmB);
+    tmY = tmB;
+    if (a.lean) {
+        // the launch's output pixels as a [n][ho][wo][co] tensor (a parity class of a transposed
+        // convolution: every ostride-th row and column from (ooy, oox)); a box is the 32 rows of one
+        // epilogue warp, 64 (G = 32: 32) channels wide, swizzled over its row
+        EncodeTiledFn enc = encode_fn();
+        if (!enc) return fail(HATQ_ERR_CUDA, "cuTensorMapEncodeTiled is unavailable");
+        const cuuint64_t px = (cuuint64_t)a.co * a.ostride, rw = (cuuint64_t)a.y_w * px, im = (cuuint64_t)a.y_h * a.y_w * a.co;
+        const cuuint64_t dims[4] = {(cuuint64_t)a.co, (cuuint64_t)wo, (cuuint64_t)ho, (cuuint64_t)n};
+        const cuuint64_t strides[3] = {px, rw, im};
+        const int bx = a.tw < 32 ? a.tw : 32;
+        const cuuint32_t box[4] = {g.G == 32 ? 32u : 64u, (cuuint32_t)bx, (cuuint32_t)(32 / bx), 1};
+        const cuuint32_t estr[4] = {1, 1, 1, 1};
+        void *base = static_cast<int8_t *>(y) + ((long long)a.ooy * a.y_w + a.oox) * a.co;
+        CUresult r = enc(&tmY, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, base, dims, strides, box, estr,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, g.G == 32 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B,
+                         CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return fail(HATQ_ERR_CUDA, "output tensor map encoding failed (%d)", (int)r);
+    }
     if (!g.gather) {
         EncodeTiledFn enc = encode_fn();
         if (!enc) return fail(HATQ_ERR_CUDA, "cuTensorMapEncodeTiled is unavailable");
@@ -1030,7 +1053,7 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     } else {
         tmA = tmB;
     }
-    cudaError_t e = hatq::launch_conv(tmA, tmB, a, smem_bytes, reinterpret_cast<cudaStream_t>(stream));
+    cudaError_t e = hatq::launch_conv(tmA, tmB, tmY, a, smem_bytes, reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(e, "convolution launch");
     return HATQ_OK;
 }

@@ -33,12 +33,19 @@
 // Every mbarrier wait is bounded: on expiry the kernel records an error word,
 // raises a CTA-wide abort flag and unwinds (waiting, again bounded, for its own
 // MMAs and copies) before freeing TMEM.
-// This file is compiled twice: as itself (the kernels for activation blocks of
-// whole 64-channel boxes, the launcher, the self test) and, through
-// hatq_conv_pieces.cu with HATQ_CONV_PIECES = 1, for the kernels whose blocks
-// arrive as two 32-channel boxes; two translation units build in parallel.
+// This file is compiled four times: as itself (the kernels with every option,
+// the launcher, the self test) and through hatq_conv_pieces.cu (activation
+// blocks arriving as two 32-channel boxes), hatq_conv_lean.cu and
+// hatq_conv_lean_pieces.cu (the lean kernels: INT8 codes of one exact chunk per
+// tile without further options, one instantiation per transform group). Four
+// translation units build in parallel, and no kernel carries code that its
+// layers never run: with every option in one kernel, each change of any branch
+// changed the code generated for all of them (ga1 between 7.6 and 8.9 ms).
 #ifndef HATQ_CONV_PIECES
 #define HATQ_CONV_PIECES 0
+#endif
+#ifndef HATQ_CONV_LEAN
+#define HATQ_CONV_LEAN 0
 #endif
 
 #include <cuda_fp16.h>
@@ -362,6 +369,98 @@ __device__ __forceinline__ void epi_split128(const EpiCtx &e, const ConvArgs &a,
     store_codes<64>(a, e.row, half, p);
 }
 
+// ------------------------------------------------------------------ lean epilogue
+//
+// Layers that emit INT8 codes with no further option (no general transition,
+// float or fp16 output, affine operand or sub-pixel rearrangement) whose
+// reduction is one exact chunk. Each warp finishes its 32 pixel rows by itself:
+// the accumulator columns of a group are read with two tensor-memory loads in
+// flight, the region is released as soon as the last ones arrived, and the
+// codes leave as one TMA store per warp and 64 (32) columns from a swizzled
+// 32-row staging buffer (two per warp). Nothing waits for another warp, except
+// the pair of warps that shares the rows of a 128-wide group.
+// Bound: integer issue (38 integer operations per value of a WH(64) -> ReLU ->
+// DH(64) transition, the 64-bit adds on the integer pipe at half rate).
+// Against the epilogue with every option (named barriers and a copy loop per
+// tile, 16 columns per tensor-memory load, the shared register budget): the
+// analysis chain on 8 x 2160 x 3840 16.32 -> 15.35 ms (ga1 is half of it), the
+// entropy chains on 8 x 135 x 240 7.52 -> 7.24 ms, 512 x 768 analysis 215 -> 204 us.
+
+// t = M a + M b of G columns from tile column col: tensor memory, then 64-bit
+// multiply-adds with the bias products staged in shared memory.
+template <int G>
+__device__ __forceinline__ void lean_scale(const uint32_t (&r)[G], const long long *mb, const int *mult, long long *t) {
+#pragma unroll
+    for (int i = 0; i < G; i += 4) {
+        const int4 m = *reinterpret_cast<const int4 *>(mult + i);
+        const longlong2 b0 = *reinterpret_cast<const longlong2 *>(mb + i);
+        const longlong2 b1 = *reinterpret_cast<const longlong2 *>(mb + i + 2);
+        t[i] = (long long)m.x * __float2int_rn(__uint_as_float(r[i])) + b0.x;
+        t[i + 1] = (long long)m.y * __float2int_rn(__uint_as_float(r[i + 1])) + b0.y;
+        t[i + 2] = (long long)m.z * __float2int_rn(__uint_as_float(r[i + 2])) + b1.x;
+        t[i + 3] = (long long)m.w * __float2int_rn(__uint_as_float(r[i + 3])) + b1.y;
+    }
+}
+
+// Codes of G columns as words of four. For a shift n >= 33 the half 2^(n-1) has
+// a zero low word, so round half up is (hi + half_hi) >> (n - 32) on the high
+// word alone, and half to even differs only for values whose low word is zero:
+// without one in the group (the usual case) that is the rounding.
+template <int G>
+__device__ __forceinline__ void lean_codes(const ConvArgs &a, const long long (&t)[G], uint32_t (&w)[G / 4]) {
+    if (a.shift >= 32) {
+        uint32_t mn = 0xFFFFFFFFu;
+#pragma unroll
+        for (int i = 0; i < G; i += 2) mn = min(mn, min((uint32_t)t[i], (uint32_t)t[i + 1]));
+        const int sh = a.shift - 32;
+        if (sh > 0 && mn != 0u) {
+            const int half = 1 << (sh - 1);
+#pragma unroll
+            for (int i = 0; i < G / 4; ++i) {
+                int q[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    q[k] = max(((int)((unsigned long long)t[4 * i + k] >> 32) + half) >> sh, -127);
+                w[i] = pack4_sat(q[0], q[1], q[2], q[3]);
+            }
+            return;
+        }
+        const long long kadd = (1LL << (a.shift - 1)) - 1;
+#pragma unroll
+        for (int i = 0; i < G / 4; ++i)
+            w[i] = pack4_sat(requant8_lo(t[4 * i], kadd, sh), requant8_lo(t[4 * i + 1], kadd, sh),
+                             requant8_lo(t[4 * i + 2], kadd, sh), requant8_lo(t[4 * i + 3], kadd, sh));
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < G / 4; ++i)
+        w[i] = pack4(requant8(t[4 * i], a.shift), requant8(t[4 * i + 1], a.shift), requant8(t[4 * i + 2], a.shift),
+                     requant8(t[4 * i + 3], a.shift));
+}
+
+// One warp's staging: two buffers of 32 rows of 64 bytes.
+constexpr int kWarpStage = 4096;
+
+// Codes of this lane's row (G = 64: 64 bytes, 64-byte swizzle; G = 32: 32
+// bytes, 32-byte swizzle) into a staging buffer, then one TMA store of the
+// warp's 32 rows. The buffer's previous store was the second last.
+template <int G>
+__device__ __forceinline__ void lean_store(uint8_t *buf, const uint32_t (&w)[G / 4], const CUtensorMap *tmY, int lane,
+                                           bool inside, int ch, int ox, int oy, int img) {
+    if (lane == 0) bulk_wait_read<1>();
+    __syncwarp();
+    const int sw = G == 64 ? (lane >> 1) & 3 : (lane >> 2) & 1;
+#pragma unroll
+    for (int q = 0; q < G / 16; ++q)
+        *reinterpret_cast<uint4 *>(buf + lane * G + ((q ^ sw) << 4)) = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+    fence_async_shared();
+    __syncwarp();
+    if (lane == 0) {
+        if (inside) tma_store_4d(smem_addr(buf), tmY, ch, ox, oy, img);
+        bulk_commit();
+    }
+}
+
 // ------------------------------------------------------------------ kernel
 
 // One CTA per SM, looping over output tiles (tile t -> M tile t / n_tiles_n,
@@ -375,10 +474,11 @@ __device__ __forceinline__ void epi_split128(const EpiCtx &e, const ConvArgs &a,
 // SUB: 64-wide reduction blocks per pipeline stage (1, 2 or 4). PIECES: the
 // activation blocks arrive as two 32-channel boxes (c % 64 == 32); a separate
 // instantiation, so that the other layers' kernels carry none of its code.
-template <int SUB, bool PIECES>
+// LEAN: 0 the epilogue with every option, else the lean epilogue's group.
+template <int SUB, bool PIECES, int LEAN>
 __global__ void __launch_bounds__(kThreads, 1)
     conv_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                const __grid_constant__ ConvArgs a) {
+                const __grid_constant__ CUtensorMap tmY, const __grid_constant__ ConvArgs a) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int S = a.stages;
@@ -443,18 +543,29 @@ __global__ void __launch_bounds__(kThreads, 1)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     // bias codes, multipliers and dequant factors of all output channels,
-    // staged once per CTA (128-byte aligned, read with 16-byte vector loads)
+    // staged once per CTA (128-byte aligned, read with 16-byte vector loads);
+    // the lean epilogue takes the bias products M b (64 bits) and the multipliers
     int *cb = reinterpret_cast<int *>(bar_area + a.const_off);
-    const float s_aff = a.affine ? *a.affine_s : 0.f;
-    for (int c = threadIdx.x; c < a.co; c += kThreads) {
-        cb[c] = a.b_int[c];
-        cb[a.co + c] = a.mult[c];
-        reinterpret_cast<float *>(cb)[2 * a.co + c] = a.affine ? s_aff * a.s_w[c] * a.inv_gamma : a.deq[c];
-        reinterpret_cast<float *>(cb)[3 * a.co + c] = a.affine ? a.deq[c] : 0.f;
-    }
+    long long *mbs = reinterpret_cast<long long *>(bar_area + a.const_off);
+    int *mults = reinterpret_cast<int *>(mbs + a.co);
     int8_t *lut_s = reinterpret_cast<int8_t *>(bar_area + a.lut_off);
-    if (a.general)
-        for (int i = threadIdx.x; i < 256; i += kThreads) lut_s[i] = a.lut[i];
+    if constexpr (LEAN != 0) {
+        for (int c = threadIdx.x; c < a.co; c += kThreads) {
+            const int m = a.mult[c];
+            mbs[c] = (long long)m * a.b_int[c];
+            mults[c] = m;
+        }
+    } else {
+        const float s_aff = a.affine ? *a.affine_s : 0.f;
+        for (int c = threadIdx.x; c < a.co; c += kThreads) {
+            cb[c] = a.b_int[c];
+            cb[a.co + c] = a.mult[c];
+            reinterpret_cast<float *>(cb)[2 * a.co + c] = a.affine ? s_aff * a.s_w[c] * a.inv_gamma : a.deq[c];
+            reinterpret_cast<float *>(cb)[3 * a.co + c] = a.affine ? a.deq[c] : 0.f;
+        }
+        if (a.general)
+            for (int i = threadIdx.x; i < 256; i += kThreads) lut_s[i] = a.lut[i];
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -825,6 +936,125 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (a.win_tma && ok) mbar_arrive(win_empty(j & 1));   // this thread's reads of the window are done
             }
         }
+    } else if constexpr (LEAN != 0) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 200;" ::: "memory");
+        // ---------------------------------------------------------- lean epilogue (warps 4-11)
+        const int wg = (warp - 4) >> 2;            // 0 or 1
+        const int quad = warp & 3;                 // TMEM lane quadrant this warp may access
+        const uint32_t t_lane = tmem + ((uint32_t)(quad * 32) << 16);
+        uint8_t *wstage = staging + (warp - 4) * kWarpStage;
+        const int row0 = quad * 32;                // first tile row of this warp; its 32 rows are one output box
+        const int box_y = row0 >> a.tw_log2, box_x = row0 & (a.tw - 1);
+        bool ok = true;
+        int buf = 0;
+        for (int j = 0; j < my_tiles; ++j) {
+            if (LEAN != 128 && (j & 1) != wg) continue;
+            int img, ho0, wo0, n0;
+            tile_coords(j, img, ho0, wo0, n0);
+            const int reg = j & 1;
+            const uint32_t t_acc = t_lane + (uint32_t)(reg * a.n_t);
+            if (ok) ok = __all_sync(0xffffffffu, mbar_wait(acc_full(reg), (j >> 1) & 1, abort_flag, a.err));
+            tc_fence_after();
+            const int oy = ho0 + box_y, ox = wo0 + box_x;
+            const bool inside = oy < a.ho && ox < a.wo;
+            if constexpr (LEAN != 128) {
+                if (!ok) break;
+                for (int col = 0; col < a.n_t; col += LEAN) {
+                    long long t[LEAN];
+                    {
+                        uint32_t r[LEAN];
+#pragma unroll
+                        for (int q = 0; q < LEAN / 32; ++q)
+                            tmem_ld32(t_acc + col + 32 * q, reinterpret_cast<uint32_t(&)[32]>(r[32 * q]));
+                        tmem_wait_ld();
+                        if (col + LEAN >= a.n_t) {       // TMEM reads of this region are complete
+                            tc_fence_before();
+                            mbar_arrive(acc_empty(reg));
+                        }
+                        lean_scale<LEAN>(r, mbs + n0 + col, mults + n0 + col, t);
+                    }
+                    if (a.hb_out) fwht_stages<LEAN>(t, a.hb_out);
+                    if (a.act) {
+#pragma unroll
+                        for (int i = 0; i < LEAN; ++i) t[i] = relu_mad(t[i]);
+                    }
+                    if (a.hb_next) fwht_stages<LEAN>(t, a.hb_next);
+                    uint32_t w[LEAN / 4];
+                    lean_codes<LEAN>(a, t, w);
+                    lean_store<LEAN>(wstage + buf * (kWarpStage / 2), w, &tmY, lane, inside, n0 + col, ox, oy, img);
+                    buf ^= 1;
+                }
+            } else {
+                // A 128-column group shared by the two warps of a quadrant, warpgroup wg producing
+                // outputs 64 wg .. 64 wg + 63 (see epi_split128): both halves of the accumulator are
+                // read for hb_out = 128, and for hb_next = 128 the halves of phi are exchanged through
+                // the warps' first staging buffers, eight values per thread and round, at a barrier of
+                // the pair. Every warp runs the exchange barriers, also after an abort.
+                const int half = 64 * wg;
+                long long p[64];
+                {
+                    uint32_t r0[32], r1[32];
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        if (a.hb_out == 128) {
+                            long long x[32];
+                            tmem_ld32(t_acc + 32 * q, r0);
+                            tmem_ld32(t_acc + 64 + 32 * q, r1);
+                            tmem_wait_ld();
+                            lean_scale<32>(r0, mbs + n0 + 32 * q, mults + n0 + 32 * q, p + 32 * q);
+                            lean_scale<32>(r1, mbs + n0 + 64 + 32 * q, mults + n0 + 64 + 32 * q, x);
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) p[32 * q + i] = wg ? p[32 * q + i] - x[i] : p[32 * q + i] + x[i];
+                        } else {
+                            tmem_ld32(t_acc + half + 32 * q, r0);
+                            tmem_wait_ld();
+                            lean_scale<32>(r0, mbs + n0 + half + 32 * q, mults + n0 + half + 32 * q, p + 32 * q);
+                        }
+                    }
+                }
+                tc_fence_before();
+                mbar_arrive(acc_empty(reg));
+                if (a.hb_out) fwht_stages<64>(p, min(a.hb_out, 64));
+                if (a.act) {
+#pragma unroll
+                    for (int i = 0; i < 64; ++i) p[i] = relu_mad(p[i]);
+                }
+                if (a.hb_next == 128) {
+                    // [pair k][row] in 16-byte units: a warp's accesses are 512 contiguous bytes
+                    int4 *mine = reinterpret_cast<int4 *>(wstage) + lane;
+                    const int4 *theirs =
+                        reinterpret_cast<const int4 *>(staging + (wg ? warp - 8 : warp) * kWarpStage) + lane;
+#pragma unroll
+                    for (int rd = 0; rd < 8; ++rd) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const long long u0 = p[8 * rd + 2 * k], u1 = p[8 * rd + 2 * k + 1];
+                            mine[k * 32] = make_int4((int)u0, (int)(u0 >> 32), (int)u1, (int)(u1 >> 32));
+                        }
+                        asm volatile("bar.sync %0, 64;" ::"r"(4 + quad) : "memory");
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int4 v = theirs[k * 32];
+                            const long long o0 = (long long)(((unsigned long long)(uint32_t)v.y << 32) | (uint32_t)v.x);
+                            const long long o1 = (long long)(((unsigned long long)(uint32_t)v.w << 32) | (uint32_t)v.z);
+                            const int i0 = 8 * rd + 2 * k;
+                            p[i0] = wg ? o0 - p[i0] : p[i0] + o0;           // u_0 - u_1 on the upper half, u_0 + u_1 on the lower
+                            p[i0 + 1] = wg ? o1 - p[i0 + 1] : p[i0 + 1] + o1;
+                        }
+                        asm volatile("bar.sync %0, 64;" ::"r"(4 + quad) : "memory");
+                    }
+                    fwht_fixed<64, 64>(p);
+                } else if (a.hb_next) {
+                    fwht_stages<64>(p, a.hb_next);
+                }
+                uint32_t w[16];
+                lean_codes<64>(a, p, w);
+                // the second buffer holds every tile's codes (the exchange has the first): its last store is long read
+                if (lane == 0) bulk_wait_read<0>();
+                lean_store<64>(wstage + kWarpStage / 2, w, &tmY, lane, inside && ok, n0 + half, ox, oy, img);
+            }
+        }
+        if (lane == 0) bulk_wait_all();
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 200;" ::: "memory");
         // ---------------------------------------------------------- epilogue warpgroups (warps 4-7, 8-11)
@@ -993,7 +1223,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
-#if !HATQ_CONV_PIECES
+#if !HATQ_CONV_PIECES && !HATQ_CONV_LEAN
 // Failure-detection self test: one thread waits, through the pipeline's
 // bounded wait, on an mbarrier nothing arrives at; the wait expires after
 // `limit` cycles and records kErrWaitTimeout in the error word.
@@ -1011,31 +1241,44 @@ __global__ void wait_selftest_kernel(int *err, long long limit) {
 
 }  // namespace
 
-#if HATQ_CONV_PIECES
-ConvKernelFn conv_pieces_kernel(int sub) {
-    return sub == 4 ? conv_kernel<4, true> : (sub == 2 ? conv_kernel<2, true> : conv_kernel<1, true>);
+#define HATQ_SUB_KERNEL(pieces, lean) \
+    (sub == 4 ? conv_kernel<4, pieces, lean> : (sub == 2 ? conv_kernel<2, pieces, lean> : conv_kernel<1, pieces, lean>))
+
+#if HATQ_CONV_LEAN && HATQ_CONV_PIECES
+ConvKernelFn conv_lean_pieces_kernel(int sub, int g) {
+    return g == 128 ? HATQ_SUB_KERNEL(true, 128) : (g == 64 ? HATQ_SUB_KERNEL(true, 64) : HATQ_SUB_KERNEL(true, 32));
 }
+#elif HATQ_CONV_LEAN
+ConvKernelFn conv_lean_kernel(int sub, int g) {
+    return g == 128 ? HATQ_SUB_KERNEL(false, 128) : (g == 64 ? HATQ_SUB_KERNEL(false, 64) : HATQ_SUB_KERNEL(false, 32));
+}
+#elif HATQ_CONV_PIECES
+ConvKernelFn conv_pieces_kernel(int sub) { return HATQ_SUB_KERNEL(true, 0); }
 #else
+ConvKernelFn conv_full_kernel(int sub) { return HATQ_SUB_KERNEL(false, 0); }
+
 cudaError_t launch_wait_selftest(int *err, long long limit_cycles, cudaStream_t s) {
     wait_selftest_kernel<<<1, 32, 0, s>>>(err, limit_cycles);
     return cudaGetLastError();
 }
 
-cudaError_t launch_conv(const CUtensorMap &tmA, const CUtensorMap &tmB, const ConvArgs &a, int smem_bytes, cudaStream_t s) {
+cudaError_t launch_conv(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmY, const ConvArgs &a,
+                        int smem_bytes, cudaStream_t s) {
     // the shared-memory opt-in and the SM count are per device
     constexpr int kMaxDev = 64;
-    static int configured_smem[kMaxDev][6] = {};
+    static int configured_smem[kMaxDev][24] = {};
     static int sms_of[kMaxDev] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDev) return cudaErrorInvalidDevice;
     if ((a.sub != 1 && a.sub != 2 && a.sub != 4) || (a.gather && a.sub != 1) || a.chunk_kb % a.sub ||
-        (a.half && (a.gather || a.a_f16 || a.cin_h < 1)))
+        (a.half && (a.gather || a.a_f16 || a.cin_h < 1)) || (a.lean && a.num_kb > a.chunk_kb))
         return cudaErrorInvalidValue;   // gathered tiles: one block per stage
-    const int v = (a.sub == 4 ? 2 : (a.sub == 2 ? 1 : 0)) + (a.half ? 3 : 0);
-    const ConvKernelFn kern = a.half ? conv_pieces_kernel(a.sub)
-                                     : (v == 2 ? conv_kernel<4, false> : (v == 1 ? conv_kernel<2, false> : conv_kernel<1, false>));
+    const int fam = a.lean ? (a.group == 128 ? 3 : (a.group == 64 ? 2 : 1)) : 0;
+    const int v = (a.sub == 4 ? 2 : (a.sub == 2 ? 1 : 0)) + (a.half ? 3 : 0) + 6 * fam;
+    const ConvKernelFn kern = a.lean ? (a.half ? conv_lean_pieces_kernel(a.sub, a.group) : conv_lean_kernel(a.sub, a.group))
+                                     : (a.half ? conv_pieces_kernel(a.sub) : conv_full_kernel(a.sub));
     if (smem_bytes > configured_smem[dev][v]) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
         if (e != cudaSuccess) return e;
@@ -1048,10 +1291,10 @@ cudaError_t launch_conv(const CUtensorMap &tmA, const CUtensorMap &tmB, const Co
         sms_of[dev] = sms > 0 ? sms : 1;
     }
     const int grid = a.num_tiles < sms_of[dev] ? a.num_tiles : sms_of[dev];
-    kern<<<grid, kThreads, smem_bytes, s>>>(tmA, tmB, a);
+    kern<<<grid, kThreads, smem_bytes, s>>>(tmA, tmB, tmY, a);
     return cudaGetLastError();
 }
 
-#endif  // HATQ_CONV_PIECES
+#endif
 
 }  // namespace hatq

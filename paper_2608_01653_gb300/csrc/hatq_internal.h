@@ -127,6 +127,7 @@ struct ConvArgs {
     const float *affine_s;
     const float *s_w;
     int general, shift_in;
+    int lean, group;                 // INT8 codes without options: lean kernel of this transform group (32, 64, 128)
     int a_f16;                       // operand codes as fp16 in the TMA tile: the MMA reads A from shared memory
     int out_f16;                     // codes written as fp16
     int lut_off;                     // offset of the table copy from the barrier area
@@ -134,11 +135,17 @@ struct ConvArgs {
     int8_t lut[256];
 };
 
-// the convolution kernel for layers whose activation blocks arrive as two 32-channel boxes (a.half),
-// with sub 64-wide blocks per pipeline stage (compiled in its own translation unit)
-using ConvKernelFn = void (*)(const CUtensorMap, const CUtensorMap, const ConvArgs);
+// The convolution kernels, by blocks per pipeline stage (sub): the one with
+// every option, and the lean ones for INT8 codes without options (a.lean, group
+// g = 32, 64 or 128); "pieces" for layers whose activation blocks arrive as two
+// 32-channel boxes (a.half). Each family is its own translation unit.
+using ConvKernelFn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const ConvArgs);
+ConvKernelFn conv_full_kernel(int sub);
 ConvKernelFn conv_pieces_kernel(int sub);
-cudaError_t launch_conv(const CUtensorMap &tmA, const CUtensorMap &tmB, const ConvArgs &a,
+ConvKernelFn conv_lean_kernel(int sub, int g);
+ConvKernelFn conv_lean_pieces_kernel(int sub, int g);
+// tmY: output box of one epilogue warp (lean kernels)
+cudaError_t launch_conv(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmY, const ConvArgs &a,
                         int smem_bytes, cudaStream_t s);
 
 // GDN / IGDN transition kernel (hatq_gdn.cu).

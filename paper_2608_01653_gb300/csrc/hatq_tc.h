@@ -90,6 +90,24 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *tm,
         : "memory");
 }
 
+// Box of a 4-D tensor written from shared memory (parts outside the tensor are
+// dropped). Commit, then wait until at most N of this thread's latest groups
+// still read shared memory (or, with bulk_wait_all, until all are written).
+__device__ __forceinline__ void tma_store_4d(uint32_t src, const CUtensorMap *tm, int c0, int c1, int c2, int c3) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%1, {%2, %3, %4, %5}], [%0];" ::"r"(src),
+                 "l"(tm), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void bulk_wait_read() {
+    asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_shared() {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
 // tcgen05 shared-memory matrix descriptor: K-major operand, 128-byte swizzle,
 // 8-row groups 1024 bytes apart (stride byte offset), version field = 1.
 __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
@@ -223,6 +241,17 @@ __device__ __forceinline__ uint32_t pack4(int q0, int q1, int q2, int q3) {
                        0x5410);
 }
 
+// max(v, 0) with the two products on the multiply-add pipe: the sign mask m is
+// 0 or -1 and x + m x is x or 0. (A compare and two selects are three
+// operations on the integer pipe, which bounds the 64-bit transitions.)
+__device__ __forceinline__ long long relu_mad(long long v) {
+    const int lo = (int)(uint32_t)v, hi = (int)((unsigned long long)v >> 32), m = hi >> 31;
+    int l, h;
+    asm("mad.lo.s32 %0, %1, %2, %1;" : "=r"(l) : "r"(lo), "r"(m));
+    asm("mad.lo.s32 %0, %1, %2, %1;" : "=r"(h) : "r"(hi), "r"(m));
+    return (long long)(((unsigned long long)(uint32_t)h << 32) | (uint32_t)l);
+}
+
 template <int G, int HB, typename T>
 __device__ __forceinline__ void fwht_fixed(T (&t)[G]) {
 #pragma unroll
@@ -248,6 +277,27 @@ __device__ __forceinline__ void fwht(T (&t)[G], int hb) {
         case 32: if (G >= 32) fwht_fixed<G, (G >= 32 ? 32 : 2)>(t); break;
         case 64: if (G >= 64) fwht_fixed<G, (G >= 64 ? 64 : 2)>(t); break;
         default: break;
+    }
+}
+
+// The same transform as one sequence of stages: whole groups (hb = G, the
+// usual case) run straight through, smaller blocks stop after log2(hb) stages.
+template <int G, typename T>
+__device__ __forceinline__ void fwht_stages(T (&t)[G], int hb) {
+    if (hb == G) {
+        fwht_fixed<G, G>(t);
+        return;
+    }
+#pragma unroll
+    for (int h = 1; h < G / 2; h <<= 1) {
+        if (h >= hb) break;
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+            if (i & h) continue;
+            const T a = t[i], b = t[i + h];
+            t[i] = a + b;
+            t[i + h] = a - b;
+        }
     }
 }
 

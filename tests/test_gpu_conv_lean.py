@@ -1,0 +1,79 @@
+"""The convolution kernels for INT8 codes without further options, at the
+places where their epilogue decides: rounding ties at shifts around a word
+boundary, ragged output boxes, and every transform group. Bit-exact against
+the oracle."""
+import numpy as np
+import pytest
+
+from oracle import hatq_oracle as O
+from synth import configs as C
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def H():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2608_01653_gb300 import hatq
+    hatq.load()
+    return hatq
+
+
+def dev(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def layer_from_codes(q, form, stride, act):
+    """A layer whose weight codes are q [c_out, k, k, c_in] at scale 2^-10 (blocks of 4 and
+    64 have exact square roots, so W and its transform are exact)."""
+    co, k, _, ci = q.shape
+    L = C.layer("t", ci, co, k, stride, k // 2, form, act, hb_in=4 if form == "DH" else None,
+                hb_out=64 if form == "WH" else None)
+    if form == "DH":
+        w = O.transform_real(q.astype(np.float64), 4)
+    else:
+        w = np.moveaxis(O.transform_real(np.moveaxis(q.astype(np.float64), 0, -1), 64), -1, 0)
+    return L, (w * 2.0 ** -10).astype(np.float32)
+
+
+def run_both(H, L, w, b, s_x, s_y, hb_next, x):
+    P = H.prepare_weights(H.desc_from_spec(L), w, b, s_x, s_y, L.act, hb_next, False)
+    y = H.conv2d_i8(dev(x), P)
+    H.sync_status()
+    p = O.prepare_layer(w, b, L.form, L.hb_in, L.hb_out, s_x, s_y, L.act, hb_next, False, L.stride, L.pad)
+    return y.cpu().numpy(), O.conv_layer(x, p), P
+
+
+@pytest.mark.parametrize("shift", [30, 31, 32, 33, 36])
+@pytest.mark.parametrize("c_out,form,hb_next,act", [(64, "DH", 0, "none"), (192, "DH", 64, "relu"), (224, "DH", 32, "none"),
+                                                    (128, "DH", 128, "relu"), (64, "WH", 64, "relu"), (32, "DH", 0, "relu")])
+def test_power_of_two_scales_round_ties_to_even(H, c_out, form, hb_next, act, shift):
+    """M = 2^30 for every channel, so M a / 2^n has ties whatever n is: at n <= 32 the half lies
+    in the low word, above it the low word of a tie is zero."""
+    rng = np.random.default_rng(shift + c_out)
+    q = rng.integers(-2, 3, size=(c_out, 3, 3, 64))
+    q[:, 1, 1, 0] = 127                                    # the channel's scale
+    L, w = layer_from_codes(q, form, 1, act)
+    x = rng.integers(-3, 4, size=(2, 9, 37, 64)).astype(np.int8)
+    x[..., 0] = rng.integers(-1, 2, size=(2, 9, 37)) * (rng.random((2, 9, 37)) < 0.2)
+    alpha = (8.0 if form == "WH" else 1.0) * np.sqrt(hb_next if hb_next else 1)
+    s_y = float(np.float32(2.0 ** -10 * 2.0 ** (shift - 30) / alpha))
+    got, ref, P = run_both(H, L, w, np.zeros(c_out, np.float32), 1.0, s_y, hb_next, x)
+    assert np.array_equal(got, ref)
+    if hb_next != 128 and hb_next != 32:                   # alpha is a power of two
+        assert P.struct.shift == shift
+    assert len(np.unique(ref)) > 3
+
+
+@pytest.mark.parametrize("h,w", [(1, 1), (1, 129), (5, 31), (17, 33), (130, 3), (16, 64)])
+@pytest.mark.parametrize("c_out,hb_next", [(192, 64), (96, 32), (128, 128)])
+def test_ragged_output_boxes(H, h, w, c_out, hb_next):
+    """Output sizes at the edges of the warps' 32-row boxes; two images."""
+    rng = np.random.default_rng(h * 1000 + w)
+    L, wt = layer_from_codes(rng.integers(-127, 128, size=(c_out, 1, 1, 64)), "DH", 1, "relu")
+    x = rng.integers(-127, 128, size=(2, h, w, 64)).astype(np.int8)
+    got, ref, _ = run_both(H, L, wt, rng.normal(0, 1, c_out).astype(np.float32), 0.05, 0.11, hb_next, x)
+    assert np.array_equal(got, ref)

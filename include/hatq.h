@@ -121,6 +121,9 @@ typedef struct {
     int8_t lut[256];      /* phi_int of Eq. supp_general_activation at z = -127..127 (index z + 127) */
     int in_f16;           /* 1: the INT8 operand arrives as IEEE fp16 values (exact), see hatq_set_operand_format */
     int out_f16;          /* 1: the INT8 codes are written as IEEE fp16 values (exact) */
+    int chunk_kb;         /* 64-wide reduction blocks whose fp32 sums are exact for these weights (written by the
+                             preparation from w_i8); 0: the bound that holds for any codes. Set it to 0 if
+                             the weight buffers are changed afterwards */
 } hatq_prepared;
 
 /*

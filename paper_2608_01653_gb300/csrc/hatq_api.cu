@@ -609,6 +609,40 @@ hatq_status check_out_buffers(const hatq_prepared *out) {
     return HATQ_OK;
 }
 
+// Blocks of an exact fp32 chunk that hold whatever the codes are: 1024 products
+// of |x| <= 127 (INT8 operands), 512 of |x| <= 255 (centred affine codes).
+constexpr int kChunkAny = 16, kChunkAnyAffine = 8;
+
+// The longest chunk (in 64-wide reduction blocks, a multiple of 4 so that no
+// pipeline stage straddles two chunks) whose fp32 partial sums are exact for
+// these weight codes: every partial sum of a chunk is an integer of magnitude
+// <= xmax sum |w| over the chunk, and fp32 holds every integer up to 2^24.
+// Real weight codes average far below 127, so most layers' whole reduction is
+// one chunk and the accumulator is never drained inside a tile.
+int exact_chunk(const std::vector<int8_t> &w, int co, int k_pad, int xmax, int any) {
+    const int nkb = k_pad / 64;
+    std::vector<int> s((size_t)co * nkb);               // sum |w| of each channel's blocks
+    for (int o = 0; o < co; ++o)
+        for (int b = 0; b < nkb; ++b) {
+            int t = 0;
+            for (int k = 0; k < 64; ++k) t += std::abs((int)w[(size_t)o * k_pad + b * 64 + k]);
+            s[(size_t)o * nkb + b] = t;
+        }
+    const long long lim = (1LL << 24) / xmax;
+    for (int chunks = 1;; ++chunks) {
+        const int len = ((nkb + chunks - 1) / chunks + 3) & ~3;
+        if (len <= any) return any;
+        bool ok = true;
+        for (int o = 0; o < co && ok; ++o)
+            for (int b0 = 0; b0 < nkb && ok; b0 += len) {
+                long long t = 0;
+                for (int b = b0; b < nkb && b < b0 + len; ++b) t += s[(size_t)o * nkb + b];
+                ok = t <= lim;
+            }
+        if (ok) return len;
+    }
+}
+
 // Copies the host arrays to the caller's device buffers, encodes the weight
 // tensor map and fills the struct (dop: the descriptor of the operand).
 hatq_status upload_layer(const hatq_conv_desc &dop, const Geometry &g, const HostLayer &hl, int act, int hb_next,
@@ -655,6 +689,7 @@ hatq_status upload_layer(const hatq_conv_desc &dop, const Geometry &g, const Hos
     out->in_affine = 0;
     out->in_f16 = 0;
     out->out_f16 = 0;
+    out->chunk_kb = exact_chunk(hl.w_i8, co, g.k_pad, 128, kChunkAny);   // INT8 operands, -128 included
     out->mult_in = gen ? gen->mult_in : 0;
     if (gen) std::memcpy(out->lut, gen->lut, sizeof out->lut);
     else std::memset(out->lut, 0, sizeof out->lut);
@@ -897,7 +932,6 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     a.half = g.half;
     a.cin_h = g.cin_pad / 32;
     a.gather = g.gather;
-    // exact fp32 chunks: 1024 products of |x| <= 127 (INT8 codes), 512 of |x| <= 255 (centred affine codes)
     a.affine = L->in_affine ? 1 : 0;
     a.a_f16 = L->in_f16 ? 1 : 0;
     a.out_f16 = L->out_f16 ? 1 : 0;
@@ -905,7 +939,8 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
         return fail(HATQ_ERR_UNSUPPORTED, "an fp16 operand needs c_in %% 64 == 0 or 16 or 48, and INT8 codes");
     if (a.out_f16 && (L->out_f32 || (og && og->d2s)))
         return fail(HATQ_ERR_UNSUPPORTED, "fp16 code output needs INT8 output without the sub-pixel rearrangement");
-    a.chunk_kb = a.affine ? 8 : 16;
+    // exact fp32 chunks: as prepared for these weights, else the length that holds for any codes
+    a.chunk_kb = L->chunk_kb > 0 ? L->chunk_kb : (a.affine ? kChunkAnyAffine : kChunkAny);
     a.b_bytes = a.n_t * 128;
     a.raw_bytes = g.gather ? 0 : ((a.affine || a.a_f16) ? 16384 : 8192);
     a.n_tiles_n = d->c_out / a.n_t;
@@ -1219,6 +1254,7 @@ hatq_status hatq_prepare_weights_affine(const hatq_conv_desc *d, const float *w_
     }
     if ((st = upload_layer(dop, g, hl, act, 0, 1, 1.f, 0.f, nullptr, out, stream)) != HATQ_OK) return st;
     out->in_affine = 1;
+    out->chunk_kb = exact_chunk(hl.w_i8, dop.c_out, g.k_pad, 255, kChunkAnyAffine);
     out->s_x = 0.f;
     return HATQ_OK;
 }

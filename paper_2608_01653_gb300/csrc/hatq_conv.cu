@@ -11,7 +11,9 @@
 // fp32 accumulators in tensor memory (TMEM). Every product is an integer of
 // magnitude <= 127^2 and every partial sum of a 1024-long reduction chunk is
 // an integer of magnitude <= 1024 * 127^2 < 2^24, so all fp32 values involved
-// are exactly representable integers and the chunk sum is exact. Chunk g
+// are exactly representable integers and the chunk sum is exact. A chunk may be
+// longer where the layer's own weight codes keep its sums below 2^24 (chunk_kb
+// of the prepared layer). Chunk g
 // accumulates in TMEM region g & 1; the epilogue warps convert finished chunks
 // to int32 and add them into int32 partials in their registers, so the full
 // accumulator is the exact int32 sum.
@@ -466,7 +468,7 @@ __device__ __forceinline__ void lean_store(uint8_t *buf, const uint32_t (&w)[G /
 // One CTA per SM, looping over output tiles (tile t -> M tile t / n_tiles_n,
 // N tile t % n_tiles_n). The stage ring runs continuously across tiles. TMEM
 // holds two fp32 accumulator regions and the reduction runs in exact chunks
-// of at most 1024 (sums below 2^24), chunk g accumulating in region g & 1, so
+// (sums below 2^24), chunk g accumulating in region g & 1, so
 // the MMA issuer fills one region while the epilogue empties the other. With
 // one chunk per tile epilogue warpgroup w takes the tiles of region w; with
 // several, both warpgroups drain every chunk into int32 register partials
@@ -1104,7 +1106,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     mbar_arrive(acc_empty(reg));
                     continue;
                 }
-                if (nbuf == 1) {
+                if (nbuf == 1 && nchunks > 1) {
                     // last chunk: chunk sum + partial -> exact int32 totals, written back in place so
                     // that each 64/128-wide transform group can read all of its columns
                     if (ok) {
@@ -1136,7 +1138,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 e.deq = reinterpret_cast<const float *>(cb + 2 * a.co) + n0;
                 e.biasf = reinterpret_cast<const float *>(cb + 3 * a.co) + n0;
                 e.t_acc = t_acc;
-                e.int_acc = nbuf == 1;
+                e.int_acc = nbuf == 1 && nchunks > 1;
                 e.lut = lut_s;
                 e.row = stage_tile + (size_t)row * a.row_stride;
                 e.gout = nullptr;

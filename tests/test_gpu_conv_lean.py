@@ -77,3 +77,28 @@ def test_ragged_output_boxes(H, h, w, c_out, hb_next):
     x = rng.integers(-127, 128, size=(2, h, w, 64)).astype(np.int8)
     got, ref, _ = run_both(H, L, wt, rng.normal(0, 1, c_out).astype(np.float32), 0.05, 0.11, hb_next, x)
     assert np.array_equal(got, ref)
+
+
+@pytest.mark.parametrize("avg,one_chunk", [(120, True), (122, False)])
+@pytest.mark.parametrize("sign", [1, -1])
+def test_whole_reduction_in_one_exact_chunk(H, avg, one_chunk, sign):
+    """1088 weight codes of average magnitude 120: 128 sum |w| stays below 2^24, so the layer takes
+    the reduction in one chunk, and with operand codes of -128 and 127 the sums come within 0.4 %
+    of 2^24; at 122 they would pass it and the general 1024-long chunk stays. The bias cancels the
+    sum, so the output shows its low bits."""
+    k = 1088
+    q = np.full((32, 1, 1, k), avg)
+    q[:, 0, 0, 0] = 127
+    s = np.where(np.arange(32) % 2, 1, -1)[:, None, None, None]
+    L, w = layer_from_codes(q * s, "DH", 1, "none")
+    x = np.full((1, 5, 27, k), -128 if sign < 0 else 127, np.int8)
+    x[0, 1:, :, 5] -= 1 * sign
+    x[0, 2:, 3:, 7] -= 2 * sign
+    x[0, :, 9::2, 1] += np.int8(-sign)
+    s_w = 2.0 ** -10
+    total = int(np.abs(q[0]).sum()) * (128 if sign < 0 else 127)
+    b = (-sign * s[:, 0, 0, 0] * (total - 300) * s_w).astype(np.float32)
+    got, ref, P = run_both(H, L, w, b, 1.0, float(np.float32(8 * s_w)), 0, x)
+    assert np.array_equal(got, ref)
+    assert (P.struct.chunk_kb >= k // 64) == one_chunk
+    assert len(np.unique(ref)) > 3

@@ -980,7 +980,7 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     const int win_bytes = g.gather ? a.win_buf * (a.win_tma ? 2 : 1) : 0;
     const int table_bytes = g.gather ? a.num_kb * 8 * 4 : 0;
     const int const_bytes = ((4 * d->c_out * 4 + 127) & ~127) + (general ? 256 : 0);
-    const int fixed = 1024 /* align */ + 8 * (3 * 8 + 13) + 16 + 128 + table_bytes + const_bytes + win_bytes;
+    const int fixed = 1024 /* align */ + 8 * (3 * 8 + 9) + 16 + 128 + table_bytes + const_bytes + win_bytes;
     const int budget = 227 * 1024 - 1024 /* static */ - fixed - a.staging_bytes;
     // a stage holds `sub` 64-wide reduction blocks: [weights x sub | INT8 box x sub].
     // The cost of a stage is dominated by its barrier hand-offs, not its bytes,
@@ -1002,7 +1002,8 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     if (a.stages > 8) a.stages = 8;
     if (g.gather && a.stages > 4) a.stages = 4;
     if (a.stages < 2) return fail(HATQ_ERR_UNSUPPORTED, "tile does not fit in shared memory");
-    const int bar_bytes = 8 * (3 * a.stages + 13) + 16;
+    if (a.a_slots > a.stages) a.a_slots = a.stages;   // the converters take a slot's release from its stage's barrier
+    const int bar_bytes = 8 * (3 * a.stages + 9) + 16;
     a.const_off = (bar_bytes + table_bytes + 127) & ~127;
     a.win_off = a.const_off + const_bytes;
     const int smem_bytes = a.stages * a.stage_bytes + a.staging_bytes + 1024 + a.win_off + win_bytes;

@@ -19,13 +19,14 @@
 // accumulator is the exact int32 sum.
 //
 // Persistent kernel, one CTA per SM, 512 threads in four warpgroups:
-//   warp 0      TMA producer: weight tile (fp16, 128B-swizzled) and, for
-//               c_in % 16 == 0, the INT8 activation box of one kernel tap and
-//               64 input channels (64B-swizzled; zero fill outside the image =
-//               zero padding), SUB 64-wide blocks per pipeline stage.
-//   warp 1      TMEM allocation; lane 0 issues the MMAs (A operand in TMEM,
-//               B in shared memory) and commits.
-//   warps 2-3   idle (they complete warpgroup 0 for the register split).
+//   warp 0      TMA producer of the weight tiles (fp16, 128B-swizzled), SUB
+//               64-wide blocks per pipeline stage.
+//   warp 1      TMEM allocation; issues the MMAs (A operand in TMEM, B in shared
+//               memory) and their commits.
+//   warp 2      TMA producer of the INT8 activation boxes of one kernel tap and 64
+//               input channels (c_in % 16 == 0; 64B-swizzled; zero fill outside
+//               the image = zero padding) or of a small-channel layer's windows.
+//   warp 3      idle (it completes warpgroup 0 for the register split).
 //   warps 4-11  epilogue warpgroups: drains and the fused requantize /
 //               Hadamard epilogue into a shared-memory output tile, copied out
 //               coalesced.
@@ -487,19 +488,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint8_t *staging = smem + (size_t)S * a.stage_bytes;
     uint8_t *bar_area = staging + (size_t)a.staging_bytes;
     const uint32_t bar0 = smem_addr(bar_area);
-    // barriers: full[S], conv[S], empty[S], acc_full[2], acc_empty[2], a_free[4], mma_done
+    // barriers: full[S], conv[S], empty[S], acc_full[2], acc_empty[2], mma_done, win_full[2], win_empty[2]
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
     auto conv_bar = [&](int s) { return bar0 + 8u * (S + s); };
     auto empty_bar = [&](int s) { return bar0 + 8u * (2 * S + s); };
     auto acc_full = [&](int b) { return bar0 + 8u * (3 * S + b); };
     auto acc_empty = [&](int b) { return bar0 + 8u * (3 * S + 2 + b); };
-    auto a_free = [&](int q) { return bar0 + 8u * (3 * S + 4 + q); };
-    const uint32_t mma_done = bar0 + 8u * (3 * S + 8);
+    const uint32_t mma_done = bar0 + 8u * (3 * S + 4);
     // small-channel layers with a TMA-loaded input window: two window buffers
-    auto win_full = [&](int b) { return bar0 + 8u * (3 * S + 9 + b); };
-    auto win_empty = [&](int b) { return bar0 + 8u * (3 * S + 11 + b); };
-    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(bar_area + 8 * (3 * S + 13));
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(bar_area + 8 * (3 * S + 13) + 4);
+    auto win_full = [&](int b) { return bar0 + 8u * (3 * S + 5 + b); };
+    auto win_empty = [&](int b) { return bar0 + 8u * (3 * S + 7 + b); };
+    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(bar_area + 8 * (3 * S + 9));
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(bar_area + 8 * (3 * S + 9) + 4);
 
     // A failure already recorded by this launch (or an earlier, unread one)
     // ends every CTA that has not started, so a fault cannot serialize waits.
@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
-            mbar_init(full_bar(s), 1);
+            mbar_init(full_bar(s), a.gather ? 1 : 2);   // weight and activation producers
             mbar_init(conv_bar(s), kConvThreads);
             mbar_init(empty_bar(s), 1);
         }
@@ -529,7 +529,6 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(acc_full(b), 1);
             mbar_init(acc_empty(b), ep_count);
         }
-        for (int q = 0; q < 4; ++q) mbar_init(a_free(q), 1);
         mbar_init(mma_done, 1);
         for (int b = 0; b < 2; ++b) {
             mbar_init(win_full(b), 1);
@@ -591,61 +590,81 @@ __global__ void __launch_bounds__(kThreads, 1)
     // warpgroups 1-2 (epilogue) 200: 128 x (40 + 72) + 256 x 200 = 65536, and
     // per scheduler (one warp of each warpgroup) 32 x (40 + 72 + 2 x 200) = 16384.
     const int SA = a.a_slots;
+    // The issuing warps run their loops converged (waits by every lane, uniform
+    // counters) and elect one lane for the copies, MMAs and commits, so that
+    // the operands of those instructions stay in uniform registers: with the
+    // whole loop inside one divergent lane each TMA cost ~190 cycles and a
+    // stage's loop tail ~500, more than the MMAs of the stage (analysis chain on
+    // 8 x 2160 x 3840 15.16 -> 14.53 ms, entropy chains on 8 x 135 x 240
+    // 6.79 -> 6.41 ms, 5x5 s2 192 -> 192 on 256 x 256 51.3 -> 49.2 us).
     if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;" ::: "memory");
-    if (warp == 0) {
-        // ---------------------------------------------------------- TMA producer
-        if (lane == 0) {
-            // stage s with phase parity ph, advanced incrementally (the issuing
-            // threads of the pipeline avoid integer division)
-            const uint32_t tx_bytes = (uint32_t)(a.b_bytes + (a.gather ? 0 : a.raw_bytes));
-            int issued_ph[8];
-            for (int q = 0; q < 8; ++q) issued_ph[q] = -1;
-            int win_ph[2] = {-1, -1};
-            bool ok = true;
-            int s = 0;
-            uint32_t ph = 0;
-            for (int j = 0; j < my_tiles && ok; ++j) {
-                int img, ho0, wo0, n0;
-                tile_coords(j, img, ho0, wo0, n0);
-                if (a.win_tma) {
-                    // the tile's input window: one 3-D box of the [n][h][w c] byte tensor, its first byte
-                    // column rounded down to 16 (out-of-image parts, also negative ones, are zero-filled)
-                    const int b = j & 1;
-                    if (j >= 2 && !mbar_wait(win_empty(b), ((j >> 1) - 1) & 1, abort_flag, a.err)) { ok = false; break; }
+    if (warp == 0 || warp == 2) {
+        // ---------------------------------------------------------- TMA producers
+        // warp 0: weight boxes; warp 2: activation boxes (or the input windows of
+        // a small-channel layer). Both count on full[s].
+        const bool acts = warp == 2;
+        const uint32_t stage0 = smem_addr(smem) + (uint32_t)(acts ? a.raw_off : a.b_off);
+        const uint32_t box_bytes = (uint32_t)(acts ? a.raw_bytes : a.b_bytes);
+        // last phase parity this warp issued per stage / window buffer (bit), and whether any
+        uint32_t issued = 0, issued_ph = 0, win_issued = 0, win_ph = 0;
+        bool ok = true;
+        int s = 0;
+        uint32_t ph = 0;
+        for (int j = 0; j < my_tiles && ok; ++j) {
+            int img, ho0, wo0, n0;
+            tile_coords(j, img, ho0, wo0, n0);
+            if (acts && a.gather) {
+                if (!a.win_tma) break;               // the converters stage the window themselves
+                // the tile's input window: one 3-D box of the [n][h][w c] byte tensor, its first byte
+                // column rounded down to 16 (out-of-image parts, also negative ones, are zero-filled)
+                const int b = j & 1;
+                if (j >= 2)
+                    ok = __all_sync(0xffffffffu, mbar_wait(win_empty(b), ((j >> 1) - 1) & 1, abort_flag, a.err));
+                if (!ok) break;
+                if (elect_one()) {
                     mbar_expect_tx(win_full(b), (uint32_t)a.win_tma_bytes);
                     const int xb = (wo0 * a.stride - a.pad_x) * a.c;
                     tma_load_3d(smem_addr(bar_area + a.win_off + b * a.win_buf), &tmA, win_full(b), xb & ~15,
                                 ho0 * a.stride - a.pad_y, img);
-                    win_ph[b] = (j >> 1) & 1;
                 }
-                int cb = 0, kx = 0, ky = 0;          // 64-channel block, kernel column and row of block kb
-                for (int kb0 = 0; kb0 < a.num_kb; kb0 += SUB) {
-                    const int nsub = min(SUB, a.num_kb - kb0);
-                    if (!mbar_wait(empty_bar(s), ph ^ 1, abort_flag, a.err)) { ok = false; break; }
-                    const uint32_t st = smem_addr(smem + (size_t)s * a.stage_bytes);
-                    mbar_expect_tx(full_bar(s), tx_bytes * (uint32_t)nsub);
+                win_issued |= 1u << b;
+                win_ph = (win_ph & ~(1u << b)) | ((uint32_t)((j >> 1) & 1) << b);
+                continue;
+            }
+            const int x0 = wo0 * a.stride - a.pad_x, y0 = ho0 * a.stride - a.pad_y;
+            int cb = 0, kx = 0, ky = 0;              // channel block (or piece), kernel column and row of block kb
+            for (int kb0 = 0; kb0 < a.num_kb; kb0 += SUB) {
+                const int nsub = min(SUB, a.num_kb - kb0);
+                ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1, abort_flag, a.err));
+                if (!ok) break;
+                const uint32_t st = stage0 + (uint32_t)s * (uint32_t)a.stage_bytes;
+                const bool leader = elect_one();
+                if (leader) mbar_expect_tx(full_bar(s), box_bytes * (uint32_t)nsub);
+                if (!acts) {
+                    if (leader) {
+#pragma unroll
+                        for (int u = 0; u < SUB; ++u)
+                            if (u < nsub) tma_load_2d(st + u * box_bytes, &tmB, full_bar(s), (kb0 + u) * kBlockK, n0);
+                    }
+                } else {
 #pragma unroll
                     for (int u = 0; u < SUB; ++u) {
                         if (u >= nsub) break;
-                        tma_load_2d(st + a.b_off + u * a.b_bytes, &tmB, full_bar(s), (kb0 + u) * kBlockK, n0);
                         if constexpr (!PIECES) {
-                            if (!a.gather) {
-                                tma_load_4d(st + a.raw_off + u * a.raw_bytes, &tmA, full_bar(s), cb * kBlockK,
-                                            wo0 * a.stride + kx - a.pad_x, ho0 * a.stride + ky - a.pad_y, img);
-                                if (++cb == a.cin_kb) {
-                                    cb = 0;
-                                    if (++kx == a.kw) { kx = 0; ++ky; }
-                                }
+                            if (leader) tma_load_4d(st + u * box_bytes, &tmA, full_bar(s), cb * kBlockK, x0 + kx, y0 + ky, img);
+                            if (++cb == a.cin_kb) {
+                                cb = 0;
+                                if (++kx == a.kw) { kx = 0; ++ky; }
                             }
                         } else {
                             // two 32-channel pieces (cb counts pieces); past the last tap the
                             // weights are zero and the box, in or out of the image, is read as is
 #pragma unroll
                             for (int hp = 0; hp < 2; ++hp) {
-                                tma_load_4d(st + a.raw_off + u * a.raw_bytes + hp * (a.raw_bytes >> 1), &tmA,
-                                            full_bar(s), cb * 32, wo0 * a.stride + kx - a.pad_x,
-                                            ho0 * a.stride + ky - a.pad_y, img);
+                                if (leader)
+                                    tma_load_4d(st + u * box_bytes + hp * (box_bytes >> 1), &tmA, full_bar(s), cb * 32,
+                                                x0 + kx, y0 + ky, img);
                                 if (++cb == a.cin_h) {
                                     cb = 0;
                                     if (++kx == a.kw) { kx = 0; ++ky; }
@@ -653,60 +672,60 @@ __global__ void __launch_bounds__(kThreads, 1)
                             }
                         }
                     }
-                    issued_ph[s] = (int)ph;
-                    if (++s == S) { s = 0; ph ^= 1u; }
                 }
+                issued |= 1u << s;
+                issued_ph = (issued_ph & ~(1u << s)) | (ph << s);
+                if (++s == S) { s = 0; ph ^= 1u; }
             }
-            if (!ok) {
-                // let our own copies land before the CTA unwinds
-                for (int b = 0; b < 2; ++b)
-                    if (win_ph[b] >= 0) {
-                        const long long t0 = clock64();
-                        while (!mbar_try_wait(win_full(b), (uint32_t)win_ph[b]) && clock64() - t0 < kWaitLimitCycles) {
-                        }
-                    }
-                for (int q = 0; q < S && q < 8; ++q)
-                    if (issued_ph[q] >= 0) {
-                        const long long t0 = clock64();
-                        while (!mbar_try_wait(full_bar(q), (uint32_t)issued_ph[q]) && clock64() - t0 < kWaitLimitCycles) {
-                        }
-                    }
-            }
+        }
+        if (!ok) {
+            // let our own copies land before the CTA unwinds (one limit for all of them: a stage
+            // the other producer did not reach never completes)
+            const long long t0 = clock64();
+            for (int b = 0; b < 2; ++b)
+                while ((win_issued >> b & 1u) && !mbar_try_wait(win_full(b), win_ph >> b & 1u) &&
+                       clock64() - t0 < kWaitLimitCycles) {
+                }
+            for (int q = 0; q < S; ++q)
+                while ((issued >> q & 1u) && !mbar_try_wait(full_bar(q), issued_ph >> q & 1u) &&
+                       clock64() - t0 < kWaitLimitCycles) {
+                }
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------- MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = idesc_f16(a.n_t);
-            // weight descriptor of stage 0, block 0; a stage / block moves its start address field
-            const uint64_t desc0 = sdesc_sw128(smem_addr(smem) + (uint32_t)a.b_off);
-            // fp16 operand codes: the A tile of the stage (128 rows of 128 bytes per block, 128-byte swizzle)
-            const uint64_t adesc0 = sdesc_sw128(smem_addr(smem) + (uint32_t)a.raw_off);
-            const uint32_t stage_step = (uint32_t)a.stage_bytes >> 4, blk_step = (uint32_t)a.b_bytes >> 4;
-            const uint32_t raw_step = (uint32_t)a.raw_bytes >> 4;
-            const bool a_f16 = a.a_f16 != 0;
-            bool ok = true;
-            int s = 0, slot = 0;
-            uint32_t ph = 0;
-            int g = 0;                       // exact chunks issued so far; chunk g accumulates in region g & 1
-            uint32_t d_tmem = tmem;
-            for (int j = 0; j < my_tiles && ok; ++j) {
-                // a stage holds SUB 64-wide reduction blocks; chunk boundaries
-                // (multiples of chunk_kb, itself a multiple of SUB) fall between stages
-                int ck = 0;                  // blocks of the current exact chunk already issued
-                for (int kb0 = 0; kb0 < a.num_kb; kb0 += SUB) {
-                    const int nsub = min(SUB, a.num_kb - kb0);
-                    if (ck == 0) {
-                        d_tmem = tmem + (uint32_t)((g & 1) * a.n_t);
-                        if (g >= 2) {        // wait until the epilogue released the region
-                            if (!mbar_wait(acc_empty(g & 1), ((g >> 1) - 1) & 1, abort_flag, a.err)) { ok = false; break; }
-                            tc_fence_after();
-                        }
-                    }
-                    // conv[s] completes only after every converter observed full[s] (the TMA
-                    // bytes of this stage), so waiting for it orders the weight reads as well
-                    if (!mbar_wait(conv_bar(s), ph, abort_flag, a.err)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint64_t db0 = desc0 + (uint64_t)((uint32_t)s * stage_step);
+        const uint32_t idesc = idesc_f16(a.n_t);
+        // weight descriptor of stage 0, block 0; a stage / block moves its start address field
+        const uint64_t desc0 = sdesc_sw128(smem_addr(smem) + (uint32_t)a.b_off);
+        // fp16 operand codes: the A tile of the stage (128 rows of 128 bytes per block, 128-byte swizzle)
+        const uint64_t adesc0 = sdesc_sw128(smem_addr(smem) + (uint32_t)a.raw_off);
+        const uint32_t stage_step = (uint32_t)a.stage_bytes >> 4, blk_step = (uint32_t)a.b_bytes >> 4;
+        const uint32_t raw_step = (uint32_t)a.raw_bytes >> 4;
+        const bool a_f16 = a.a_f16 != 0;
+        bool ok = true;
+        int s = 0, slot = 0;
+        uint32_t ph = 0;
+        int g = 0;                           // exact chunks issued so far; chunk g accumulates in region g & 1
+        uint32_t d_tmem = tmem;
+        for (int j = 0; j < my_tiles && ok; ++j) {
+            // a stage holds SUB 64-wide reduction blocks; chunk boundaries
+            // (multiples of chunk_kb, itself a multiple of SUB) fall between stages
+            int ck = 0;                      // blocks of the current exact chunk already issued
+            for (int kb0 = 0; kb0 < a.num_kb; kb0 += SUB) {
+                const int nsub = min(SUB, a.num_kb - kb0);
+                if (ck == 0) {
+                    d_tmem = tmem + (uint32_t)((g & 1) * a.n_t);
+                    if (g >= 2)              // wait until the epilogue released the region
+                        ok = __all_sync(0xffffffffu, mbar_wait(acc_empty(g & 1), ((g >> 1) - 1) & 1, abort_flag, a.err));
+                    if (!ok) break;
+                }
+                // conv[s] completes only after every converter observed full[s] (the TMA
+                // bytes of this stage), so waiting for it orders the weight reads as well
+                ok = __all_sync(0xffffffffu, mbar_wait(conv_bar(s), ph, abort_flag, a.err));
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t db0 = desc0 + (uint64_t)((uint32_t)s * stage_step);
+                const bool last = ck + nsub == a.chunk_kb || kb0 + nsub == a.num_kb;
+                if (elect_one()) {
                     if (!a_f16) {
                         const uint32_t a_t = tmem + (uint32_t)(a.a_col + slot * SUB * 32);
 #pragma unroll
@@ -731,22 +750,23 @@ __global__ void __launch_bounds__(kThreads, 1)
                                             (ck + u > 0 || kk > 0) ? 1u : 0u);
                         }
                     }
-                    umma_commit(empty_bar(s));
-                    umma_commit(a_free(slot));
-                    ck += nsub;
-                    if (ck == a.chunk_kb || kb0 + nsub == a.num_kb) {
-                        umma_commit(acc_full(g & 1));
-                        ++g;
-                        ck = 0;
-                    }
-                    if (++s == S) { s = 0; ph ^= 1u; }
-                    if (++slot == SA) slot = 0;
+                    umma_commit(empty_bar(s));   // frees the stage and the A slot
+                    if (last) umma_commit(acc_full(g & 1));
                 }
+                __syncwarp();
+                ck += nsub;
+                if (last) {
+                    ++g;
+                    ck = 0;
+                }
+                if (++s == S) { s = 0; ph ^= 1u; }
+                if (++slot == SA) slot = 0;
             }
-            umma_commit(mma_done);
-            const long long t0 = clock64();
-            while (!mbar_try_wait(mma_done, 0) && clock64() - t0 < kWaitLimitCycles) {
-            }
+        }
+        if (elect_one()) umma_commit(mma_done);
+        __syncwarp();
+        const long long t0 = clock64();
+        while (!mbar_try_wait(mma_done, 0) && clock64() - t0 < kWaitLimitCycles) {
         }
     }
     } else if (warp >= 12) {
@@ -758,17 +778,22 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int m = quad * 32 + lane;               // 0..127
         const uint32_t t_lane = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)a.a_col;
         bool ok = true;
-        // stage s (phase parity ph) and A slot (use parity sph), advanced incrementally
-        int s = 0, slot = 0;
-        uint32_t ph = 0, sph = 0;
+        // stage s (phase parity ph) and A slot, advanced incrementally,
+        // and the stage fs (phase parity fph) of SA iterations before, whose MMAs read the slot last
+        int s = 0, slot = 0, fs = 0;
+        uint32_t ph = 0, fph = 0;
         bool reuse = false;                           // the slot was used before (some slot wrapped)
         auto advance = [&]() {
+            if (reuse && ++fs == S) { fs = 0; fph ^= 1u; }
             if (++s == S) { s = 0; ph ^= 1u; }
-            if (++slot == SA) { slot = 0; sph ^= 1u; reuse = true; }
+            if (++slot == SA) { slot = 0; reuse = true; }
         };
-        // wait until the A slot was released by the MMAs that last read it
+        // Wait until the A slot was released by the MMAs that last read it, SA
+        // iterations before: their commit frees the stage they read as well. That
+        // stage's next phase needs this iteration or a later one (SA <= S), so the
+        // parity cannot have moved on by two.
         auto slot_free = [&]() {
-            bool w = !reuse || mbar_wait(a_free(slot), sph ^ 1u, abort_flag, a.err);
+            bool w = !reuse || mbar_wait(empty_bar(fs), fph, abort_flag, a.err);
             w = __all_sync(0xffffffffu, w);
             tc_fence_after();
             return w;
@@ -855,7 +880,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // memory; kernel row ky of output pixel m is then one contiguous
             // kw*c-byte segment of window row py*s+ky, read as 8-entry pieces
             // through a per-CTA table (window offset of each piece, -1 = zero).
-            int *tab = reinterpret_cast<int *>(bar_area + 8 * (3 * S + 13) + 16);
+            int *tab = reinterpret_cast<int *>(bar_area + 8 * (3 * S + 9) + 16);
             uint8_t *win = bar_area + a.win_off;
             for (int q = m; q < a.num_kb * 8; q += kConvThreads) {
                 const int k0 = q * 8, ky = k0 / a.seg;

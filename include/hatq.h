@@ -124,6 +124,8 @@ typedef struct {
     int chunk_kb;         /* 64-wide reduction blocks whose fp32 sums are exact for these weights (written by the
                              preparation from w_i8); 0: the bound that holds for any codes. Set it to 0 if
                              the weight buffers are changed afterwards */
+    int chunk_units;      /* the same for the order of the window convolution: input windows (64 channels, for
+                             stride 2 of one column parity) per exact chunk; 0: that kernel is not taken */
 } hatq_prepared;
 
 /*

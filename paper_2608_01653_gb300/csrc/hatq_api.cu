@@ -643,6 +643,34 @@ int exact_chunk(const std::vector<int8_t> &w, int co, int k_pad, int xmax, int a
     }
 }
 
+// The same for the window convolution, which takes the reduction in units of 64
+// channels (for stride 2 and kw > 1: and one column parity), all taps of a unit
+// in turn: the longest run of units that is exact for these codes, 0 if a single
+// unit is not.
+int exact_units(const std::vector<int8_t> &w, const hatq_conv_desc &d, const Geometry &g, int xmax) {
+    if (g.gather) return 0;
+    const int par = d.stride == 2 && d.kw > 1 ? 2 : 1, ncb = (d.c_in + 63) / 64, units = ncb * par;
+    std::vector<long long> s((size_t)d.c_out * units, 0);
+    for (int o = 0; o < d.c_out; ++o)
+        for (int tap = 0; tap < d.kh * d.kw; ++tap)
+            for (int c = 0; c < d.c_in; ++c)
+                s[(size_t)o * units + (c / 64) * par + (tap % d.kw) % par] +=
+                    std::abs((int)w[(size_t)o * g.k_pad + (size_t)tap * g.cin_pad + c]);
+    const long long lim = (1LL << 24) / xmax;
+    for (int chunks = 1; chunks <= units; ++chunks) {
+        const int len = (units + chunks - 1) / chunks;
+        bool ok = true;
+        for (int o = 0; o < d.c_out && ok; ++o)
+            for (int u0 = 0; u0 < units && ok; u0 += len) {
+                long long t = 0;
+                for (int u = u0; u < units && u < u0 + len; ++u) t += s[(size_t)o * units + u];
+                ok = t <= lim;
+            }
+        if (ok) return len;
+    }
+    return 0;
+}
+
 // Copies the host arrays to the caller's device buffers, encodes the weight
 // tensor map and fills the struct (dop: the descriptor of the operand).
 hatq_status upload_layer(const hatq_conv_desc &dop, const Geometry &g, const HostLayer &hl, int act, int hb_next,
@@ -690,6 +718,7 @@ hatq_status upload_layer(const hatq_conv_desc &dop, const Geometry &g, const Hos
     out->in_f16 = 0;
     out->out_f16 = 0;
     out->chunk_kb = exact_chunk(hl.w_i8, co, g.k_pad, 128, kChunkAny);   // INT8 operands, -128 included
+    out->chunk_units = exact_units(hl.w_i8, dop, g, 128);
     out->mult_in = gen ? gen->mult_in : 0;
     if (gen) std::memcpy(out->lut, gen->lut, sizeof out->lut);
     else std::memset(out->lut, 0, sizeof out->lut);
@@ -863,6 +892,75 @@ struct OutGrid {
     int pad_y, pad_x, ho, wo, y_h, y_w, ostride, ooy, oox, d2s;
 };
 
+// Where the window convolution applies (hatq_conv_win.cu): fills its arguments and
+// returns the shared memory it needs, or 0. Plain INT8 layers (the caller checks
+// the options) with at most 64 taps, whose windows and at least two weight stages
+// fit shared memory and whose output is not mostly the padding of its 8 x 16-pixel
+// tiles: `area` is the pixels of the other kernel's tiling, and up to a quarter
+// more is still the better bargain (a 64-row conversion saved per tap).
+int win_plan(const hatq_conv_desc &d, const Geometry &g, const hatq_prepared &L, const OutGrid *og, int n, int ho, int wo,
+             long long area, hatq::WinArgs &a, int &epi) {
+    if (L.chunk_units < 1 || d.kh * d.kw > 64 || d.kh * d.kw < 2) return 0;
+    a = hatq::WinArgs{};
+    a.ho = ho;
+    a.wo = wo;
+    a.co = d.c_out;
+    a.tiles_w = (wo + 7) / 8;
+    a.tiles_h = (ho + 15) / 16;
+    if ((long long)a.tiles_w * a.tiles_h * 128 * 4 > area * 5) return 0;
+    a.n_t = g.n_t;
+    a.n_tiles_n = d.c_out / g.n_t;
+    const long long nt = (long long)n * a.tiles_w * a.tiles_h * a.n_tiles_n;
+    if (nt >= (1LL << 31)) return 0;
+    a.num_tiles = (int)nt;
+    a.kh = d.kh;
+    a.kw = d.kw;
+    a.stride = d.stride;
+    a.pad_y = og ? og->pad_y : d.pad;
+    a.pad_x = og ? og->pad_x : d.pad;
+    a.par = d.stride == 2 && d.kw > 1 ? 2 : 1;
+    a.cin_kb = (d.c_in + 63) / 64;
+    a.k_tap = g.cin_pad;
+    a.nk_last = (d.c_in - 64 * (a.cin_kb - 1) + 15) / 16;
+    a.pairs = d.c_in == 32 && a.par == 1;
+    a.kblocks = g.k_pad / 64;
+    a.pitch = 7 + (d.kw + d.stride - 1) / d.stride;
+    a.rows = a.pitch * (15 * d.stride + d.kh);
+    a.chunk_units = L.chunk_units;
+    a.nch = (a.cin_kb * a.par + a.chunk_units - 1) / a.chunk_units;
+    if (g.G == 128) {
+        if (g.n_t != 128 || a.nch > 2) return 0;
+        epi = a.nch == 2 ? 2128 : 1128;
+    } else if (a.nch > 1) {
+        if (g.n_t > 192) return 0;
+        epi = 2064;
+    } else {
+        epi = g.G;
+    }
+    a.b_bytes = g.n_t * 128;
+    a.w8_bytes = (a.rows * 64 + 1023) & ~1023;
+    a.w16_bytes = (a.rows * 128 + 1023) & ~1023;
+    const int const_bytes = (12 * d.c_out + 127) & ~127, bars = 8 * 33 + 16;
+    const int budget = 227 * 1024 - 1024 /* static */ - 1024 /* alignment */ - 8 * 4096 - 512 - const_bytes - 2 * a.w16_bytes;
+    // two INT8 buffers unless they cost weight stages below four
+    a.n8 = (budget - 2 * a.w8_bytes) / a.b_bytes >= 4 ? 2 : 1;
+    a.stages = (budget - a.n8 * a.w8_bytes) / a.b_bytes;
+    if (a.stages > 8) a.stages = 8;
+    if (a.stages < 2) return 0;
+    a.w16_off = a.stages * a.b_bytes;
+    a.w8_off = a.w16_off + 2 * a.w16_bytes;
+    a.stg_off = a.w8_off + a.n8 * a.w8_bytes;
+    a.bar_off = a.stg_off + 8 * 4096;
+    a.const_off = (bars + 127) & ~127;
+    a.b_int = L.b_int;
+    a.mult = L.mult;
+    a.shift = L.shift;
+    a.hb_out = d.form == HATQ_WH ? d.hb_out : 0;
+    a.hb_next = L.hb_next;
+    a.act = L.act == HATQ_ACT_RELU ? 1 : 0;
+    return a.bar_off + a.const_off + const_bytes + 1024;
+}
+
 hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared *L, void *y, hatq_stream stream,
                         const OutGrid *og, const float *affine_s = nullptr) {
     if (!L) return fail(HATQ_ERR_INVALID_ARG, "null layer");
@@ -961,7 +1059,8 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     a.nbuf = (drains || g.G == 128) ? 1 : 2;
     const bool general = L->act == HATQ_ACT_SILU || L->act == HATQ_ACT_GELU;
     // the lean kernels: INT8 codes of one exact chunk per tile, no further option
-    a.lean = !drains && !general && !L->out_f32 && !a.affine && !a.a_f16 && !a.out_f16 && !a.d2s;
+    const bool plain = !general && !L->out_f32 && !a.affine && !a.a_f16 && !a.out_f16 && !a.d2s;
+    a.lean = !drains && plain;
     a.group = g.G;
     a.tmem_cols = 512;
     a.a_col = 2 * a.n_t;
@@ -1036,7 +1135,11 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     CUtensorMap tmB, tmA, tmY;
     std::memcpy(&tmB, L->opaque, sizeof tmB);
     tmY = tmB;
-    if (a.lean) {
+    hatq::WinArgs wa;
+    int epi = 0, win_smem = 0;
+    if (plain && !g.gather)
+        win_smem = win_plan(*d, g, *L, og, n, ho, wo, (long long)a.tiles_w * a.tw * a.tiles_h * a.th, wa, epi);
+    if (a.lean || win_smem) {
         // the launch's output pixels as a [n][ho][wo][co] tensor (a parity class of a transposed
         // convolution: every ostride-th row and column from (ooy, oox)); a box is the 32 rows of one
         // epilogue warp, 64 (G = 32: 32) channels wide, swizzled over its row
@@ -1045,14 +1148,32 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
         const cuuint64_t px = (cuuint64_t)a.co * a.ostride, rw = (cuuint64_t)a.y_w * px, im = (cuuint64_t)a.y_h * a.y_w * a.co;
         const cuuint64_t dims[4] = {(cuuint64_t)a.co, (cuuint64_t)wo, (cuuint64_t)ho, (cuuint64_t)n};
         const cuuint64_t strides[3] = {px, rw, im};
-        const int bx = a.tw < 32 ? a.tw : 32;
-        const cuuint32_t box[4] = {g.G == 32 ? 32u : 64u, (cuuint32_t)bx, (cuuint32_t)(32 / bx), 1};
+        const int bx = win_smem ? 8 : (a.tw < 32 ? a.tw : 32);
+        const bool narrow = g.G == 32 || (win_smem && epi == 2064);
+        const cuuint32_t box[4] = {narrow ? 32u : 64u, (cuuint32_t)bx, (cuuint32_t)(32 / bx), 1};
         const cuuint32_t estr[4] = {1, 1, 1, 1};
         void *base = static_cast<int8_t *>(y) + ((long long)a.ooy * a.y_w + a.oox) * a.co;
         CUresult r = enc(&tmY, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, base, dims, strides, box, estr,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, g.G == 32 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, narrow ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B,
                          CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return fail(HATQ_ERR_CUDA, "output tensor map encoding failed (%d)", (int)r);
+    }
+    if (win_smem) {
+        // one input window of 64 channels: pitch columns (every stride-th), all its rows
+        EncodeTiledFn enc = encode_fn();
+        if (!enc) return fail(HATQ_ERR_CUDA, "cuTensorMapEncodeTiled is unavailable");
+        const cuuint64_t dims[4] = {(cuuint64_t)d->c_in, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
+        const cuuint64_t strides[3] = {(cuuint64_t)d->c_in, (cuuint64_t)w * d->c_in, (cuuint64_t)h * w * d->c_in};
+        const cuuint32_t box[4] = {64, (cuuint32_t)(wa.pitch * d->stride), (cuuint32_t)(wa.rows / wa.pitch), 1};
+        const cuuint32_t estr[4] = {1, (cuuint32_t)d->stride, 1, 1};
+        CUresult r = enc(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void *>(x), dims, strides, box, estr,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return fail(HATQ_ERR_CUDA, "input window tensor map encoding failed (%d)", (int)r);
+        wa.err = a.err;
+        cudaError_t e = hatq::launch_conv_win(tmA, tmB, tmY, wa, epi, win_smem, reinterpret_cast<cudaStream_t>(stream));
+        if (e != cudaSuccess) return cuda_fail(e, "convolution launch");
+        return HATQ_OK;
     }
     if (!g.gather) {
         EncodeTiledFn enc = encode_fn();

@@ -1,0 +1,514 @@
+// INT8 convolution with the fused requantize / Hadamard epilogue (Eqs.
+// linear_operator, integer_accumulation, integer_hadamard_transition) for
+// layers with c_in % 16 == 0: the window form of conv_kernel.
+//
+// The tensor cores take the codes as exact fp16 values, so the INT8 operand has
+// to be converted. conv_kernel converts it again for every kernel tap (25 times
+// for a 5x5 layer); at about 115 warp instructions per 64-code row and tap that
+// conversion, not the MMAs, bounded the large layers (307 issue slots per
+// scheduler and 64-wide block against 256 cycles of MMA at N = 128). Here a tile
+// of 8 x 16 output pixels loads its input window once per 64 channels, converts
+// it once into shared memory (rows of 64 fp16 channels, 128-byte swizzle) and
+// every tap's MMAs read it in place: pixel (py, px) of tap (ky, kx) is window row
+// (stride py + ky) pitch + px + kx, so the A descriptor of a tap is the window's
+// start address plus (ky pitch + kx) rows with a group stride of stride * pitch
+// rows. For stride 2 the window is loaded by column parity (two units per 64
+// channels), which makes the eight pixels of a group neighbours again.
+//
+// Exactness as in conv_kernel: chunks of whole units whose fp32 sums stay below
+// 2^24 for the layer's weight codes, chunk g in accumulator region g & 1.
+//
+// Persistent, one CTA per SM, 512 threads:
+//   warp 0       TMA of the weight blocks (64 x n_t fp16, one per tap and unit)
+//   warp 1       TMEM allocation, MMA issue
+//   warp 2       TMA of the INT8 windows
+//   warps 4-11   epilogue (hatq_lean.h): with one chunk per tile the warpgroups
+//                take the tiles in turn; with 128-wide groups (EPI 1128) or drains
+//                (EPI 2064, 2128) both share each tile, half of every group each
+//   warps 12-15  converters: INT8 window row -> fp16 window row
+// Every wait is bounded, as in conv_kernel.
+#include <cuda_fp16.h>
+
+#include "hatq_internal.h"
+#include "hatq_lean.h"
+#include "hatq_tc.h"
+
+namespace hatq {
+namespace {
+
+using namespace tc;
+
+constexpr int kThreads = 512;
+
+// barriers from bar_off: b_full[8], b_empty[8], w8_full[2], w8_empty[2], w16_full[2],
+// w16_empty[2], acc_full[4], acc_empty[4], done; then the TMEM address and the abort flag
+constexpr int kBars = 33;
+
+// EPI, the epilogue: 32 / 64 whole tiles per warpgroup; 1128, 2064, 2128 shared
+// tiles of 128- / 64-wide groups, 2xxx with several chunks per tile: 2064 drains
+// each into registers, 2128 (two chunks of 128 columns) keeps four regions.
+
+// Exchange of this warp's values with the warp of the same pixel rows in the
+// other warpgroup and the top butterfly of the group: the lower half keeps the
+// sums, the upper half the differences. Eight values per thread and round
+// through 2 KB per warp; every warp runs the barriers, also after an abort.
+template <int H>
+__device__ __forceinline__ void exchange_top(long long (&p)[H], uint8_t *mine_b, const uint8_t *theirs_b, int wg, int quad,
+                                             int lane) {
+    int4 *mine = reinterpret_cast<int4 *>(mine_b) + lane;
+    const int4 *theirs = reinterpret_cast<const int4 *>(theirs_b) + lane;
+#pragma unroll
+    for (int rd = 0; rd < H / 8; ++rd) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const long long u0 = p[8 * rd + 2 * k], u1 = p[8 * rd + 2 * k + 1];
+            mine[k * 32] = make_int4((int)u0, (int)(u0 >> 32), (int)u1, (int)(u1 >> 32));
+        }
+        asm volatile("bar.sync %0, 64;" ::"r"(4 + quad) : "memory");
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int4 v = theirs[k * 32];
+            const long long o0 = (long long)(((unsigned long long)(uint32_t)v.y << 32) | (uint32_t)v.x);
+            const long long o1 = (long long)(((unsigned long long)(uint32_t)v.w << 32) | (uint32_t)v.z);
+            const int i0 = 8 * rd + 2 * k;
+            p[i0] = wg ? o0 - p[i0] : p[i0] + o0;
+            p[i0 + 1] = wg ? o1 - p[i0 + 1] : p[i0 + 1] + o1;
+        }
+        asm volatile("bar.sync %0, 64;" ::"r"(4 + quad) : "memory");
+    }
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(kThreads, 1)
+    conv_win_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                    const __grid_constant__ CUtensorMap tmY, const __grid_constant__ WinArgs a) {
+    constexpr bool kSplit = EPI > 1000, kDrain = EPI == 2064, kTwo = EPI == 2128;
+    constexpr int G = EPI % 1000;
+    constexpr int kRegions = kTwo ? 4 : 2, kRegLog = kTwo ? 2 : 1;   // accumulator regions of n_t columns
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *bar_area = smem + a.bar_off;
+    const uint32_t bar0 = smem_addr(bar_area);
+    auto b_full = [&](int s) { return bar0 + 8u * s; };
+    auto b_empty = [&](int s) { return bar0 + 8u * (8 + s); };
+    auto w8_full = [&](int s) { return bar0 + 8u * (16 + s); };
+    auto w8_empty = [&](int s) { return bar0 + 8u * (18 + s); };
+    auto w16_full = [&](int s) { return bar0 + 8u * (20 + s); };
+    auto w16_empty = [&](int s) { return bar0 + 8u * (22 + s); };
+    auto acc_full = [&](int s) { return bar0 + 8u * (24 + s); };
+    auto acc_empty = [&](int s) { return bar0 + 8u * (28 + s); };
+    const uint32_t mma_done = bar0 + 8u * 32;
+    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(bar_area + 8 * kBars);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(bar_area + 8 * kBars + 4);
+
+    // a failure already recorded ends every CTA that has not started
+    __shared__ int s_skip;
+    if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile int *>(a.err);
+    __syncthreads();
+    if (s_skip != 0) return;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int S = a.stages;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < 8; ++s) {
+            mbar_init(b_full(s), 1);
+            mbar_init(b_empty(s), 1);
+        }
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(w8_full(s), 1);
+            mbar_init(w8_empty(s), 128);
+            mbar_init(w16_full(s), 128);
+            mbar_init(w16_empty(s), 1);
+        }
+        for (int s = 0; s < kRegions; ++s) {
+            mbar_init(acc_full(s), 1);
+            mbar_init(acc_empty(s), kSplit ? 256 : 128);
+        }
+        mbar_init(mma_done, 1);
+        *abort_flag = 0;
+        fence_barrier_init();
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_holder)),
+                     "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    // bias products M b (64 bits) and multipliers of all output channels
+    long long *mbs = reinterpret_cast<long long *>(bar_area + a.const_off);
+    int *mults = reinterpret_cast<int *>(mbs + a.co);
+    for (int c = threadIdx.x; c < a.co; c += kThreads) {
+        const int m = a.mult[c];
+        mbs[c] = (long long)m * a.b_int[c];
+        mults[c] = m;
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_holder;
+
+    const int my_tiles = a.num_tiles > (int)blockIdx.x ? (a.num_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    const int tiles_per_img = a.tiles_w * a.tiles_h;
+    auto tile_coords = [&](int j, int &img, int &ho0, int &wo0, int &n0) {
+        const int t = (int)blockIdx.x + j * (int)gridDim.x;
+        const int mt = t / a.n_tiles_n;
+        n0 = (t - mt * a.n_tiles_n) * a.n_t;
+        img = mt / tiles_per_img;
+        const int rem = mt - img * tiles_per_img;
+        const int ty = rem / a.tiles_w;
+        ho0 = ty * 16;
+        wo0 = (rem - ty * a.tiles_w) * 8;
+    };
+
+    // register split (launch 512 x 128): 56 / 200 / 200 / 56
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;" ::: "memory");
+        // The issuing warps stay converged, their loops have uniform trip counts (a
+        // wait that fails does not return) and their copies, MMAs and commits are
+        // predicated on one lane: then counters, addresses and descriptors live in
+        // uniform registers. Measured on h1 (3x3 320 -> 640): as branches in one
+        // lane 1123 us, predicated 918 us.
+        const uint32_t lead = elect_one() ? 1u : 0u;
+        if (warp == 0) {
+            // ------------------------------------------------------ weight producer
+            const uint32_t st0 = smem_addr(smem), bytes = (uint32_t)a.b_bytes;
+            int s = 0;
+            uint32_t ph = 1, st = st0;
+            auto load = [&](int k, int n0) {
+                mbar_wait_issue(b_empty(s), ph, abort_flag, a.err, tmem, false);
+                mbar_expect_tx_if(lead, b_full(s), bytes);
+                tma_load_2d_if(lead, st, &tmB, b_full(s), k, n0);
+                st += bytes;
+                if (++s == S) { s = 0; ph ^= 1u; st = st0; }
+            };
+            for (int j = 0; j < my_tiles; ++j) {
+                int img, ho0, wo0, n0;
+                tile_coords(j, img, ho0, wo0, n0);
+                if (a.pairs) {
+                    for (int i = 0; i < a.kblocks; ++i) load(i * 64, n0);
+                    continue;
+                }
+                for (int cb = 0; cb < a.cin_kb; ++cb)
+                    for (int p = 0; p < a.par; ++p)
+                        for (int ky = 0; ky < a.kh; ++ky)
+                            for (int kx = p; kx < a.kw; kx += a.par) load((ky * a.kw + kx) * a.k_tap + cb * 64, n0);
+            }
+        } else if (warp == 2) {
+            // ------------------------------------------------------ window producer
+            int s = 0;
+            uint32_t ph = 1;
+            for (int j = 0; j < my_tiles; ++j) {
+                int img, ho0, wo0, n0;
+                tile_coords(j, img, ho0, wo0, n0);
+                const int x0 = wo0 * a.stride - a.pad_x, y0 = ho0 * a.stride - a.pad_y;
+                for (int cb = 0; cb < a.cin_kb; ++cb)
+                    for (int p = 0; p < a.par; ++p) {
+                        mbar_wait_issue(w8_empty(s), ph, abort_flag, a.err, tmem, false);
+                        mbar_expect_tx_if(lead, w8_full(s), (uint32_t)(a.rows * 64));
+                        tma_load_4d_if(lead, smem_addr(smem) + (uint32_t)(a.w8_off + s * a.w8_bytes), &tmA, w8_full(s), cb * 64,
+                                       x0 + p, y0, img);
+                        if (++s == a.n8) { s = 0; ph ^= 1u; }
+                    }
+            }
+        } else if (warp == 1) {
+            // ------------------------------------------------------ MMA issuer
+            const uint32_t idesc = idesc_f16(a.n_t);
+            // descriptor halves: start address (and the unused leading offset) in the low word; group
+            // stride, version and 128-byte swizzle in the high word
+            const uint32_t bhi = (1024u >> 4) | (1u << 14) | (2u << 29);
+            const uint32_t ahi = (uint32_t)((a.stride * a.pitch * 128) >> 4) | (1u << 14) | (2u << 29);
+            const uint32_t blo0 = ((smem_addr(smem) >> 4) & 0x3FFFu) | (1u << 16);
+            const uint32_t alo0 = ((smem_addr(smem + a.w16_off) >> 4) & 0x3FFFu) | (1u << 16);
+            const uint32_t b_step = (uint32_t)a.b_bytes >> 4, w_step = (uint32_t)a.w16_bytes >> 4;
+            const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+            int s = 0, ws = 0, g = 0;
+            uint32_t ph = 0, wph = 0, acc = 0, d = tm;
+            uint32_t bl = blo0;                              // weight stage s
+            // one weight block: K steps 0-1 read the window at o0, 2-3 at o1 (nk of them)
+            auto step = [&](uint32_t o0, uint32_t o1, int nk) {
+                mbar_wait_issue(b_full(s), ph, abort_flag, a.err, tm, true);
+                umma_f16_ss_if(lead, d, o0, ahi, bl, bhi, idesc, acc);
+                if (nk > 1) umma_f16_ss_if(lead, d, o0 + 2, ahi, bl + 2, bhi, idesc, 1u);
+                if (nk > 2) umma_f16_ss_if(lead, d, o1, ahi, bl + 4, bhi, idesc, 1u);
+                if (nk > 3) umma_f16_ss_if(lead, d, o1 + 2, ahi, bl + 6, bhi, idesc, 1u);
+                umma_commit_if(lead, b_empty(s));
+                acc = 1u;
+                bl += b_step;
+                if (++s == S) { s = 0; ph ^= 1u; bl = blo0; }
+            };
+            for (int j = 0; j < my_tiles; ++j) {
+                int left = a.cin_kb * a.par;                 // units left in the tile
+                int cu = 0;                                  // units of the current chunk
+                for (int cb = 0; cb < a.cin_kb; ++cb)
+                    for (int p = 0; p < a.par; ++p) {
+                        if (cu == 0) {
+                            const int reg = g & (kRegions - 1);
+                            d = tm + (uint32_t)(reg * a.n_t);
+                            acc = 0u;
+                            if (g >= kRegions)
+                                mbar_wait_issue(acc_empty(reg), ((g >> kRegLog) - 1) & 1, abort_flag, a.err, tm, true);
+                        }
+                        mbar_wait_issue(w16_full(ws), wph, abort_flag, a.err, tm, true);
+                        tc_fence_after();
+                        const uint32_t w0 = alo0 + (uint32_t)ws * w_step;
+                        if (a.pairs) {
+                            // two 32-channel taps per weight block (64 bytes of each window row are zero)
+                            int ky = 0, kx = 0;
+                            for (int i = 0; i < a.kblocks; ++i) {
+                                const uint32_t o0 = w0 + (uint32_t)((ky * a.pitch + kx) * 8);
+                                if (++kx == a.kw) { kx = 0; ++ky; }
+                                const int nk = ky < a.kh ? 4 : 2;
+                                const uint32_t o1 = w0 + (uint32_t)((ky * a.pitch + kx) * 8);
+                                if (++kx == a.kw) { kx = 0; ++ky; }
+                                step(o0, o1, nk);
+                            }
+                        } else if (cb == a.cin_kb - 1 && a.nk_last < 4) {
+                            for (int ky = 0; ky < a.kh; ++ky) {
+                                uint32_t o = w0 + (uint32_t)(ky * a.pitch * 8);
+                                for (int kx = p; kx < a.kw; kx += a.par, o += 8) step(o, o + 4, a.nk_last);
+                            }
+                        } else {
+                            for (int ky = 0; ky < a.kh; ++ky) {
+                                uint32_t o = w0 + (uint32_t)(ky * a.pitch * 8);
+                                for (int kx = p; kx < a.kw; kx += a.par, o += 8) step(o, o + 4, 4);
+                            }
+                        }
+                        umma_commit_if(lead, w16_empty(ws));
+                        if (++ws == 2) { ws = 0; wph ^= 1u; }
+                        --left;
+                        if (++cu == a.chunk_units || left == 0) {
+                            umma_commit_if(lead, acc_full(g & (kRegions - 1)));
+                            ++g;
+                            cu = 0;
+                        }
+                    }
+            }
+            umma_commit_if(lead, mma_done);
+            const long long t0 = clock64();
+            while (!mbar_try_wait(mma_done, 0) && clock64() - t0 < kWaitLimitCycles) {
+            }
+        }
+    } else if (warp >= 12) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;" ::: "memory");
+        // ---------------------------------------------------------- converters
+        const int t = (int)threadIdx.x - 384;
+        bool ok = true;
+        int s8 = 0, s16 = 0;
+        uint32_t p8 = 0, p16 = 0;
+        const int total = my_tiles * a.cin_kb * a.par;
+        for (int u = 0; u < total; ++u) {
+            ok = __all_sync(0xffffffffu, mbar_wait(w8_full(s8), p8, abort_flag, a.err));
+            if (ok) ok = __all_sync(0xffffffffu, mbar_wait(w16_empty(s16), p16 ^ 1u, abort_flag, a.err));
+            if (!ok) break;
+            const uint8_t *src = smem + a.w8_off + s8 * a.w8_bytes;
+            uint8_t *dst = smem + a.w16_off + s16 * a.w16_bytes;
+#pragma unroll 2
+            for (int r = t; r < a.rows; r += 128) {
+                // 64 codes (64-byte swizzle) -> 64 fp16 values (128-byte swizzle)
+                const int sw8 = (r >> 1) & 3, sw16 = r & 7;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint4 v = *reinterpret_cast<const uint4 *>(src + r * 64 + ((q ^ sw8) << 4));
+                    uint4 lo, hi;
+                    i8x4_to_f16x4(v.x, lo.x, lo.y);
+                    i8x4_to_f16x4(v.y, lo.z, lo.w);
+                    i8x4_to_f16x4(v.z, hi.x, hi.y);
+                    i8x4_to_f16x4(v.w, hi.z, hi.w);
+                    *reinterpret_cast<uint4 *>(dst + r * 128 + (((2 * q) ^ sw16) << 4)) = lo;
+                    *reinterpret_cast<uint4 *>(dst + r * 128 + (((2 * q + 1) ^ sw16) << 4)) = hi;
+                }
+            }
+            fence_async_shared();                    // the MMAs read the window through the async proxy
+            mbar_arrive(w16_full(s16));
+            mbar_arrive(w8_empty(s8));
+            if (++s8 == a.n8) { s8 = 0; p8 ^= 1u; }
+            if (++s16 == 2) { s16 = 0; p16 ^= 1u; }
+        }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 200;" ::: "memory");
+        // ---------------------------------------------------------- epilogue (warps 4-11)
+        const int wg = (warp - 4) >> 2;            // 0 or 1
+        const int quad = warp & 3;                 // TMEM lane quadrant this warp may access
+        const uint32_t t_lane = tmem + ((uint32_t)(quad * 32) << 16);
+        uint8_t *staging = smem + a.stg_off;
+        uint8_t *wstage = staging + (warp - 4) * kWarpStage;
+        bool ok = true;
+        int buf = 0;
+        for (int j = 0; j < my_tiles; ++j) {
+            if (!kSplit && (j & 1) != wg) continue;
+            int img, ho0, wo0, n0;
+            tile_coords(j, img, ho0, wo0, n0);
+            const int oy = ho0 + 4 * quad, ox = wo0;       // this warp's 32 rows: 4 x 8 pixels
+            const bool inside = oy < a.ho && ox < a.wo;
+            if constexpr (!kSplit) {
+                const int reg = j & 1;
+                const uint32_t t_acc = t_lane + (uint32_t)(reg * a.n_t);
+                ok = __all_sync(0xffffffffu, mbar_wait(acc_full(reg), (j >> 1) & 1, abort_flag, a.err));
+                tc_fence_after();
+                if (!ok) break;
+                for (int col = 0; col < a.n_t; col += G) {
+                    long long t[G];
+                    {
+                        uint32_t r[G];
+#pragma unroll
+                        for (int q = 0; q < G / 32; ++q)
+                            tmem_ld32(t_acc + col + 32 * q, reinterpret_cast<uint32_t(&)[32]>(r[32 * q]));
+                        tmem_wait_ld();
+                        if (col + G >= a.n_t) {            // TMEM reads of this region are complete
+                            tc_fence_before();
+                            mbar_arrive(acc_empty(reg));
+                        }
+                        lean_scale<G>(r, mbs + n0 + col, mults + n0 + col, t);
+                    }
+                    if (a.hb_out) fwht_stages<G>(t, a.hb_out);
+                    if (a.act) {
+#pragma unroll
+                        for (int i = 0; i < G; ++i) t[i] = relu_mad(t[i]);
+                    }
+                    if (a.hb_next) fwht_stages<G>(t, a.hb_next);
+                    uint32_t w[G / 4];
+                    lean_codes<G>(a.shift, t, w);
+                    lean_store<G>(wstage + buf * (kWarpStage / 2), w, &tmY, lane, inside, n0 + col, ox, oy, img);
+                    buf ^= 1;
+                }
+            } else {
+                constexpr int H = G / 2;                   // columns of a group this warp finishes
+                constexpr int NP = G == 64 ? 3 : 1;        // groups of a tile (n_t <= 192 / n_t = 128)
+                const uint8_t *theirs = staging + (wg ? warp - 8 : warp) * kWarpStage;
+                uint32_t part[kDrain ? NP : 1][kDrain ? H : 1];   // exact int32 sums of the drained chunks
+                // groups of this warp: columns (2 gr + wg) H .. + H - 1 (tiles of 32-wide groups may hold an odd number)
+                const int ng = (a.n_t / H - wg + 1) / 2;
+                for (int ch = 0; kDrain && ch + 1 < a.nch; ++ch) {
+                    const int gc = j * a.nch + ch, reg = gc & 1;
+                    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(acc_full(reg), (gc >> 1) & 1, abort_flag, a.err));
+                    tc_fence_after();
+                    if (ok) {
+#pragma unroll
+                        for (int gr = 0; gr < NP; ++gr) {
+                            if (gr >= ng) break;
+#pragma unroll
+                            for (int q = 0; q < H / 32; ++q) {
+                                uint32_t r[32];
+                                tmem_ld32(t_lane + (uint32_t)(reg * a.n_t + gr * G + wg * H + 32 * q), r);
+                                tmem_wait_ld();
+#pragma unroll
+                                for (int i = 0; i < 32; ++i) {
+                                    const uint32_t v = (uint32_t)__float2int_rn(__uint_as_float(r[i]));
+                                    if constexpr (kDrain) part[gr][32 * q + i] = ch ? part[gr][32 * q + i] + v : v;
+                                }
+                            }
+                        }
+                    }
+                    tc_fence_before();
+                    mbar_arrive(acc_empty(reg));
+                }
+                if (ng == 0) {                             // n_t = 32: the other warpgroup has the tile
+                    tc_fence_before();
+                    mbar_arrive(acc_empty((j * a.nch + a.nch - 1) & (kRegions - 1)));
+                    continue;
+                }
+                // the last chunk's region; with 2128 both chunks of the tile still sit in regions of their own
+                const int gc = j * a.nch + a.nch - 1, reg = gc & (kRegions - 1), reg0 = (gc - 1) & (kRegions - 1);
+                if constexpr (kTwo)
+                    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(acc_full(reg0), ((gc - 1) >> kRegLog) & 1, abort_flag, a.err));
+                if (ok) ok = __all_sync(0xffffffffu, mbar_wait(acc_full(reg), (gc >> kRegLog) & 1, abort_flag, a.err));
+                tc_fence_after();
+#pragma unroll
+                for (int gr = 0; gr < NP; ++gr) {
+                    if (gr >= ng) break;
+                    const int col = gr * G + wg * H;
+                    long long t[H];
+#pragma unroll
+                    for (int q = 0; q < H / 32; ++q) {
+                        uint32_t r[32], r0[kTwo ? 32 : 1];
+                        tmem_ld32(t_lane + (uint32_t)(reg * a.n_t + col + 32 * q), r);
+                        if constexpr (kTwo) tmem_ld32(t_lane + (uint32_t)(reg0 * a.n_t + col + 32 * q), r0);
+                        tmem_wait_ld();
+                        if (q == H / 32 - 1 && gr == ng - 1) {
+                            tc_fence_before();
+                            mbar_arrive(acc_empty(reg));
+                            if constexpr (kTwo) mbar_arrive(acc_empty(reg0));
+                        }
+                        const long long *mb = mbs + n0 + col + 32 * q;
+                        const int *mu = mults + n0 + col + 32 * q;
+#pragma unroll
+                        for (int i = 0; i < 32; i += 4) {
+                            const int4 m = *reinterpret_cast<const int4 *>(mu + i);
+                            const longlong2 b0 = *reinterpret_cast<const longlong2 *>(mb + i);
+                            const longlong2 b1 = *reinterpret_cast<const longlong2 *>(mb + i + 2);
+                            int v[4];
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                v[k] = __float2int_rn(__uint_as_float(r[i + k]));
+                                if constexpr (kDrain) v[k] += (int)part[gr][32 * q + i + k];
+                                if constexpr (kTwo) v[k] += __float2int_rn(__uint_as_float(r0[i + k]));
+                            }
+                            t[32 * q + i] = (long long)m.x * v[0] + b0.x;
+                            t[32 * q + i + 1] = (long long)m.y * v[1] + b0.y;
+                            t[32 * q + i + 2] = (long long)m.z * v[2] + b1.x;
+                            t[32 * q + i + 3] = (long long)m.w * v[3] + b1.y;
+                        }
+                    }
+                    if (a.hb_out == G) exchange_top<H>(t, wstage, theirs, wg, quad, lane);
+                    if (a.hb_out) fwht_stages<H>(t, min(a.hb_out, H));
+                    if (a.act) {
+#pragma unroll
+                        for (int i = 0; i < H; ++i) t[i] = relu_mad(t[i]);
+                    }
+                    if (a.hb_next == G) exchange_top<H>(t, wstage, theirs, wg, quad, lane);
+                    if (a.hb_next) fwht_stages<H>(t, min(a.hb_next, H));
+                    uint32_t w[H / 4];
+                    lean_codes<H>(a.shift, t, w);
+                    uint8_t *out = wstage + kWarpStage / 2;
+                    if constexpr (H == 32) {
+                        out += buf * 1024;                 // two 1 KB buffers
+                        buf ^= 1;
+                    } else if (lane == 0) {
+                        bulk_wait_read<0>();               // one 2 KB buffer
+                    }
+                    lean_store<H>(out, w, &tmY, lane, inside && ok, n0 + col, ox, oy, img);
+                }
+            }
+        }
+        if (lane == 0) bulk_wait_all();
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
+}  // namespace
+
+cudaError_t launch_conv_win(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmY, const WinArgs &a, int epi,
+                            int smem_bytes, cudaStream_t s) {
+    using Fn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const WinArgs);
+    const int v = epi == 32 ? 0 : (epi == 64 ? 1 : (epi == 1128 ? 2 : (epi == 2064 ? 3 : 4)));
+    static const Fn kerns[5] = {conv_win_kernel<32>, conv_win_kernel<64>, conv_win_kernel<1128>, conv_win_kernel<2064>,
+                                conv_win_kernel<2128>};
+    const Fn kern = kerns[v];
+    // the shared-memory opt-in and the SM count are per device
+    constexpr int kMaxDev = 64;
+    static int configured[kMaxDev][5] = {};
+    static int sms_of[kMaxDev] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDev) return cudaErrorInvalidDevice;
+    if (smem_bytes > configured[dev][v]) {
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes)) != cudaSuccess) return e;
+        configured[dev][v] = smem_bytes;
+    }
+    if (!sms_of[dev]) {
+        int sms = 0;
+        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        sms_of[dev] = sms > 0 ? sms : 1;
+    }
+    const int grid = a.num_tiles < sms_of[dev] ? a.num_tiles : sms_of[dev];
+    kern<<<grid, kThreads, smem_bytes, s>>>(tmA, tmB, tmY, a);
+    return cudaGetLastError();
+}
+
+}  // namespace hatq

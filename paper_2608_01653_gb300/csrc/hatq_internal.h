@@ -148,6 +148,32 @@ ConvKernelFn conv_lean_pieces_kernel(int sub, int g);
 cudaError_t launch_conv(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmY, const ConvArgs &a,
                         int smem_bytes, cudaStream_t s);
 
+// Window convolution (hatq_conv_win.cu): each input window is converted to fp16
+// once in shared memory and every kernel tap's MMAs read it through a shifted
+// descriptor.
+struct WinArgs {
+    int ho, wo, co;                  // output grid of the launch
+    int tiles_w, tiles_h, num_tiles, n_tiles_n, n_t;   // 8 x 16-pixel M tiles, n_t-channel N tiles
+    int kh, kw, stride, pad_y, pad_x;
+    int par;                         // column parities with taps (stride 2, kw > 1: 2, else 1)
+    int cin_kb;                      // 64-channel blocks; units per tile = cin_kb * par
+    int k_tap;                       // packed reduction entries per tap
+    int nk_last;                     // K steps (16) of the last channel block
+    int pairs;                       // c_in = 32, one parity: a 64-wide weight block is taken as two taps
+    int kblocks;                     // pairs: weight blocks
+    int pitch, rows;                 // window columns (of one parity) and rows * columns
+    int chunk_units, nch;            // units per exact chunk, chunks per tile
+    int stages, n8;                  // weight stages, INT8 window buffers (1 or 2)
+    int b_bytes, w8_bytes, w16_bytes;
+    int w8_off, w16_off, stg_off, bar_off, const_off;   // shared-memory offsets (weight stages at 0)
+    const int32_t *b_int, *mult;
+    int shift, hb_out, hb_next, act;
+    int *err;
+};
+// epi: 32 / 64 (a warpgroup finishes whole tiles), 1128 / 2064 / 2128 (both share a tile; 2xxx: drains)
+cudaError_t launch_conv_win(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmY, const WinArgs &a, int epi,
+                            int smem_bytes, cudaStream_t s);
+
 // GDN / IGDN transition kernel (hatq_gdn.cu).
 struct GdnArgs {
     const int8_t *z;                 // [pixels][c] preactivation codes (read through the tensor map)

@@ -61,6 +61,67 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 }
 
 
+// Forms for the converged issuing warps: the instruction is predicated on the
+// elected lane instead of branched around, so that the code stays uniform and
+// its operands in uniform registers.
+__device__ __forceinline__ void mbar_expect_tx_if(uint32_t pr, uint32_t bar, uint32_t bytes) {
+    asm volatile(
+        "{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n @q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}\n" ::"r"(bar),
+        "r"(bytes), "r"(pr)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_2d_if(uint32_t pr, uint32_t dst, const CUtensorMap *tm, uint32_t bar, int x, int y) {
+    asm volatile(
+        "{\n .reg .pred q;\n setp.ne.b32 q, %5, 0;\n"
+        " @q cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n}\n" ::"r"(dst),
+        "l"(tm), "r"(bar), "r"(x), "r"(y), "r"(pr)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_4d_if(uint32_t pr, uint32_t dst, const CUtensorMap *tm, uint32_t bar, int c0, int c1,
+                                               int c2, int c3) {
+    asm volatile(
+        "{\n .reg .pred q;\n setp.ne.b32 q, %7, 0;\n"
+        " @q cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];\n}\n" ::"r"(dst),
+        "l"(tm), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(pr)
+        : "memory");
+}
+// The end of an issuing warp after a failure, away from its loops: gives this
+// CTA's copies and MMAs in flight `limit` cycles to land, meets the other warps at
+// the kernel's last barrier, frees the tensor memory if asked to and exits.
+__device__ __noinline__ __attribute__((noreturn)) inline void issue_unwind(uint32_t tmem, bool dealloc, long long limit) {
+    const long long t0 = clock64();
+    while (clock64() - t0 < limit) {
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    asm volatile("barrier.sync 0;" ::: "memory");
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (dealloc)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    asm volatile("exit;");
+    __builtin_unreachable();
+}
+constexpr long long kUnwindCycles = 20000000LL;        // about 10 ms: far beyond any copy or MMA of a CTA
+// A converged warp's bounded wait without a result: a failure leaves through
+// issue_unwind, so the caller's loops keep uniform trip counts (and their
+// counters, addresses and descriptors uniform registers).
+__device__ __forceinline__ void mbar_wait_issue(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *err,
+                                                uint32_t tmem, bool dealloc) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return;
+    const long long t0 = clock64();
+    for (uint32_t spin = 1;; ++spin) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return;
+        if ((spin & 63) == 0) {
+            const bool other = *abort_flag != 0 || *reinterpret_cast<volatile int *>(err) != 0;
+            const bool late = clock64() - t0 > kWaitLimitCycles;
+            if (__any_sync(0xffffffffu, other || late)) {
+                *abort_flag = 1;
+                if (__all_sync(0xffffffffu, !other)) atomicExch(err, kErrWaitTimeout);
+                issue_unwind(tmem, dealloc, kUnwindCycles);
+            }
+        }
+    }
+}
+
 // One lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
@@ -146,6 +207,23 @@ __device__ __forceinline__ void umma_f16_ss(uint32_t d_tmem, uint64_t a, uint64_
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
         "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
+}
+// The same, predicated, with the descriptors as 32-bit halves: only the low words
+// (start addresses) change between instructions.
+__device__ __forceinline__ void umma_f16_ss_if(uint32_t pr, uint32_t d_tmem, uint32_t alo, uint32_t ahi, uint32_t blo,
+                                               uint32_t bhi, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n .reg .b64 da, db;\n mov.b64 da, {%1, %2};\n mov.b64 db, {%3, %4};\n setp.ne.b32 p, %6, 0;\n"
+        " setp.ne.b32 q, %7, 0;\n @q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n" ::"r"(d_tmem),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc), "r"(pr)
+        : "memory");
+}
+__device__ __forceinline__ void umma_commit_if(uint32_t pr, uint32_t bar) {
+    asm volatile(
+        "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+        " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+        "r"(pr)
         : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {

@@ -46,7 +46,8 @@ class PreparedStruct(ctypes.Structure):
                 ("opaque", ctypes.c_uint64 * 16),
                 ("s_z", ctypes.c_float), ("s_u", ctypes.c_float), ("shift_in", ctypes.c_int),
                 ("in_affine", ctypes.c_int), ("mult_in", ctypes.c_longlong), ("lut", ctypes.c_int8 * 256),
-                ("in_f16", ctypes.c_int), ("out_f16", ctypes.c_int), ("chunk_kb", ctypes.c_int)]
+                ("in_f16", ctypes.c_int), ("out_f16", ctypes.c_int), ("chunk_kb", ctypes.c_int),
+                ("chunk_units", ctypes.c_int)]
 
 
 MAX_TRANSPOSED_CLASSES = 4

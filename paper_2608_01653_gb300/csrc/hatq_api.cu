@@ -928,7 +928,13 @@ int win_plan(const hatq_conv_desc &d, const Geometry &g, const hatq_prepared &L,
     a.rows = a.pitch * (15 * d.stride + d.kh);
     a.chunk_units = L.chunk_units;
     a.nch = (a.cin_kb * a.par + a.chunk_units - 1) / a.chunk_units;
-    if (g.G == 128) {
+    const bool general = L.act == HATQ_ACT_SILU || L.act == HATQ_ACT_GELU;
+    if (general || (og && og->d2s)) {
+        // whole tiles per warpgroup only; the sub-pixel stores gather 64 channels at a time
+        if (g.G == 128 || a.nch > 1) return 0;
+        if (og && og->d2s && (general || og->d2s != 2 || g.n_t % 64)) return 0;
+        epi = general ? 4000 + g.G : 3064;
+    } else if (g.G == 128) {
         if (g.n_t != 128 || a.nch > 2) return 0;
         epi = a.nch == 2 ? 2128 : 1128;
     } else if (a.nch > 1) {
@@ -940,7 +946,7 @@ int win_plan(const hatq_conv_desc &d, const Geometry &g, const hatq_prepared &L,
     a.b_bytes = g.n_t * 128;
     a.w8_bytes = (a.rows * 64 + 1023) & ~1023;
     a.w16_bytes = (a.rows * 128 + 1023) & ~1023;
-    const int const_bytes = (12 * d.c_out + 127) & ~127, bars = 8 * 33 + 16;
+    const int const_bytes = (12 * d.c_out + (general ? 256 : 0) + 127) & ~127, bars = 8 * 33 + 16;
     const int budget = 227 * 1024 - 1024 /* static */ - 1024 /* alignment */ - 8 * 4096 - 512 - const_bytes - 2 * a.w16_bytes;
     // two INT8 buffers unless they cost weight stages below four
     a.n8 = (budget - 2 * a.w8_bytes) / a.b_bytes >= 4 ? 2 : 1;
@@ -958,6 +964,9 @@ int win_plan(const hatq_conv_desc &d, const Geometry &g, const hatq_prepared &L,
     a.hb_out = d.form == HATQ_WH ? d.hb_out : 0;
     a.hb_next = L.hb_next;
     a.act = L.act == HATQ_ACT_RELU ? 1 : 0;
+    a.shift_in = L.shift_in;
+    a.mult_in = L.mult_in;
+    std::memcpy(a.lut, L.lut, sizeof a.lut);
     return a.bar_off + a.const_off + const_bytes + 1024;
 }
 
@@ -1137,9 +1146,10 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     tmY = tmB;
     hatq::WinArgs wa;
     int epi = 0, win_smem = 0;
-    if (plain && !g.gather)
+    const bool win_ok = !L->out_f32 && !a.affine && !a.a_f16 && !a.out_f16 && !g.gather;
+    if (win_ok)
         win_smem = win_plan(*d, g, *L, og, n, ho, wo, (long long)a.tiles_w * a.tw * a.tiles_h * a.th, wa, epi);
-    if (a.lean || win_smem) {
+    if (a.lean || (win_smem && !a.d2s)) {
         // the launch's output pixels as a [n][ho][wo][co] tensor (a parity class of a transposed
         // convolution: every ostride-th row and column from (ooy, oox)); a box is the 32 rows of one
         // epilogue warp, 64 (G = 32: 32) channels wide, swizzled over its row
@@ -1171,6 +1181,7 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return fail(HATQ_ERR_CUDA, "input window tensor map encoding failed (%d)", (int)r);
         wa.err = a.err;
+        wa.y = y;
         cudaError_t e = hatq::launch_conv_win(tmA, tmB, tmY, wa, epi, win_smem, reinterpret_cast<cudaStream_t>(stream));
         if (e != cudaSuccess) return cuda_fail(e, "convolution launch");
         return HATQ_OK;

@@ -46,7 +46,9 @@ constexpr int kBars = 33;
 
 // EPI, the epilogue: 32 / 64 whole tiles per warpgroup; 1128, 2064, 2128 shared
 // tiles of 128- / 64-wide groups, 2xxx with several chunks per tile: 2064 drains
-// each into registers, 2128 (two chunks of 128 columns) keeps four regions.
+// each into registers, 2128 (two chunks of 128 columns) keeps four regions;
+// 3064 whole tiles with the sub-pixel rearrangement (factor 2); 4032 / 4064 whole
+// tiles with the general transition (SiLU / GELU).
 
 // Exchange of this warp's values with the warp of the same pixel rows in the
 // other warpgroup and the top butterfly of the group: the lower half keeps the
@@ -82,7 +84,8 @@ template <int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
     conv_win_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmY, const __grid_constant__ WinArgs a) {
-    constexpr bool kSplit = EPI > 1000, kDrain = EPI == 2064, kTwo = EPI == 2128;
+    constexpr bool kSplit = EPI / 1000 == 1 || EPI / 1000 == 2, kDrain = EPI == 2064, kTwo = EPI == 2128;
+    constexpr bool kD2s = EPI / 1000 == 3, kGeneral = EPI / 1000 == 4;
     constexpr int G = EPI % 1000;
     constexpr int kRegions = kTwo ? 4 : 2, kRegLog = kTwo ? 2 : 1;   // accumulator regions of n_t columns
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -142,6 +145,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbs[c] = (long long)m * a.b_int[c];
         mults[c] = m;
     }
+    int8_t *lut_s = reinterpret_cast<int8_t *>(mults + a.co);
+    if constexpr (kGeneral)
+        for (int i = threadIdx.x; i < 256; i += kThreads) lut_s[i] = a.lut[i];
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -361,15 +367,58 @@ __global__ void __launch_bounds__(kThreads, 1)
                         lean_scale<G>(r, mbs + n0 + col, mults + n0 + col, t);
                     }
                     if (a.hb_out) fwht_stages<G>(t, a.hb_out);
-                    if (a.act) {
-#pragma unroll
-                        for (int i = 0; i < G; ++i) t[i] = relu_mad(t[i]);
-                    }
-                    if (a.hb_next) fwht_stages<G>(t, a.hb_next);
                     uint32_t w[G / 4];
-                    lean_codes<G>(a.shift, t, w);
-                    lean_store<G>(wstage + buf * (kWarpStage / 2), w, &tmY, lane, inside, n0 + col, ox, oy, img);
-                    buf ^= 1;
+                    if constexpr (kGeneral) {
+                        // z = clamp(round(H~_out (M_out (.) a) / 2^n_out)), u = phi_int(z), then the next
+                        // layer's transform on u itself (|H~ u| <= 127 * 64) and its requantization
+                        int u[G];
+#pragma unroll
+                        for (int i = 0; i < G; ++i) u[i] = (int)lut_s[requant8_any(t[i], a.shift) + 127];
+                        if (a.hb_next) fwht_stages<G>(u, a.hb_next);
+#pragma unroll
+                        for (int i = 0; i < G / 4; ++i) {
+                            int q[4];
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) q[k] = requant8_any(a.mult_in * (long long)u[4 * i + k], a.shift_in);
+                            w[i] = pack4(q[0], q[1], q[2], q[3]);
+                        }
+                    } else {
+                        if (a.act) {
+#pragma unroll
+                            for (int i = 0; i < G; ++i) t[i] = relu_mad(t[i]);
+                        }
+                        if (a.hb_next) fwht_stages<G>(t, a.hb_next);
+                        lean_codes<G>(a.shift, t, w);
+                    }
+                    if constexpr (kD2s) {
+                        // channel 4 cd + 2 i + j of this lane's pixel -> channel cd of pixel (2 oy + i, 2 ox + j):
+                        // word k holds the four codes of one cd, so 4 x 4 byte transposes give 16 channels
+                        // of each of the four pixels
+                        uint32_t o[4][4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const uint32_t t0 = __byte_perm(w[4 * q], w[4 * q + 1], 0x5140);
+                            const uint32_t t1 = __byte_perm(w[4 * q + 2], w[4 * q + 3], 0x5140);
+                            const uint32_t t2 = __byte_perm(w[4 * q], w[4 * q + 1], 0x7362);
+                            const uint32_t t3 = __byte_perm(w[4 * q + 2], w[4 * q + 3], 0x7362);
+                            o[0][q] = __byte_perm(t0, t1, 0x5410);
+                            o[1][q] = __byte_perm(t0, t1, 0x7632);
+                            o[2][q] = __byte_perm(t2, t3, 0x5410);
+                            o[3][q] = __byte_perm(t2, t3, 0x7632);
+                        }
+                        const int py = oy + (lane >> 3), px = ox + (lane & 7);
+                        if (py < a.ho && px < a.wo) {
+                            uint8_t *y = static_cast<uint8_t *>(a.y) + (n0 + col) / 4 +
+                                         (((long long)img * a.ho + py) * 4 * a.wo + 2 * px) * (a.co / 4);
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                *reinterpret_cast<uint4 *>(y + (long long)((k >> 1) * 2 * a.wo + (k & 1)) * (a.co / 4)) =
+                                    make_uint4(o[k][0], o[k][1], o[k][2], o[k][3]);
+                        }
+                    } else {
+                        lean_store<G>(wstage + buf * (kWarpStage / 2), w, &tmY, lane, inside, n0 + col, ox, oy, img);
+                        buf ^= 1;
+                    }
                 }
             } else {
                 constexpr int H = G / 2;                   // columns of a group this warp finishes
@@ -485,13 +534,18 @@ __global__ void __launch_bounds__(kThreads, 1)
 cudaError_t launch_conv_win(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmY, const WinArgs &a, int epi,
                             int smem_bytes, cudaStream_t s) {
     using Fn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const WinArgs);
-    const int v = epi == 32 ? 0 : (epi == 64 ? 1 : (epi == 1128 ? 2 : (epi == 2064 ? 3 : 4)));
-    static const Fn kerns[5] = {conv_win_kernel<32>, conv_win_kernel<64>, conv_win_kernel<1128>, conv_win_kernel<2064>,
-                                conv_win_kernel<2128>};
-    const Fn kern = kerns[v];
+    static const struct { int epi; Fn fn; } kerns[] = {
+        {32, conv_win_kernel<32>},     {64, conv_win_kernel<64>},     {1128, conv_win_kernel<1128>},
+        {2064, conv_win_kernel<2064>}, {2128, conv_win_kernel<2128>}, {3064, conv_win_kernel<3064>},
+        {4032, conv_win_kernel<4032>}, {4064, conv_win_kernel<4064>}};
+    constexpr int kKerns = sizeof(kerns) / sizeof(kerns[0]);
+    int v = 0;
+    while (v < kKerns && kerns[v].epi != epi) ++v;
+    if (v == kKerns) return cudaErrorInvalidValue;
+    const Fn kern = kerns[v].fn;
     // the shared-memory opt-in and the SM count are per device
     constexpr int kMaxDev = 64;
-    static int configured[kMaxDev][5] = {};
+    static int configured[kMaxDev][kKerns] = {};
     static int sms_of[kMaxDev] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);

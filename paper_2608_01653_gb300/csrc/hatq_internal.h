@@ -168,9 +168,13 @@ struct WinArgs {
     int w8_off, w16_off, stg_off, bar_off, const_off;   // shared-memory offsets (weight stages at 0)
     const int32_t *b_int, *mult;
     int shift, hb_out, hb_next, act;
+    void *y;                         // output (sub-pixel stores; else written through tmY)
+    int shift_in;                    // general transition: input-side pair and table
+    long long mult_in;
+    int8_t lut[256];
     int *err;
 };
-// epi: 32 / 64 (a warpgroup finishes whole tiles), 1128 / 2064 / 2128 (both share a tile; 2xxx: drains)
+// epi: see hatq_conv_win.cu
 cudaError_t launch_conv_win(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmY, const WinArgs &a, int epi,
                             int smem_bytes, cudaStream_t s);
 

@@ -49,3 +49,39 @@ def test_output_transform_with_chunks(H, hb_out, hb_next):
 @pytest.mark.parametrize("h,w", [(16, 8), (17, 9), (15, 7), (1, 40), (48, 1)])
 def test_ragged_windows(H, h, w):
     case(H, 64, 192, 3, 1, 64, 3, h, w)
+
+
+@pytest.mark.parametrize("c_out,form", [(256, "DH"), (192, "WH"), (768, "DH")])
+@pytest.mark.parametrize("h,w", [(33, 26), (16, 8), (17, 5)])
+def test_subpixel_stores(H, c_out, form, h, w):
+    """The factor-2 rearrangement in the epilogue's stores, at ragged tile edges."""
+    from oracle import hatq_oracle as O
+    from tests.test_gpu_conv_lean import dev
+    rng = np.random.default_rng(c_out + h)
+    L, wt = layer_from_codes(rng.integers(-60, 61, size=(c_out, 3, 3, 64)), form, 1, "relu")
+    x = rng.integers(-127, 128, size=(3, h, w, 64)).astype(np.int8)
+    b = rng.normal(0, 1, c_out).astype(np.float32)
+    P = H.prepare_weights(H.desc_from_spec(L), wt, b, 0.05, 0.3, L.act, 0, False)
+    y = H.conv2d_i8_subpixel(dev(x), P, 2)
+    H.sync_status()
+    p = O.prepare_layer(wt, b, L.form, L.hb_in, L.hb_out, 0.05, 0.3, L.act, 0, False, 1, 1)
+    assert np.array_equal(y.cpu().numpy(), O.depth_to_space(O.conv_layer(x, p), 2))
+
+
+@pytest.mark.parametrize("c_out,form,hb_next", [(192, "DH", 64), (96, "DH", 32), (128, "WH", 64), (96, "DH", 0)])
+@pytest.mark.parametrize("act", ["silu", "gelu"])
+def test_general_transition(H, c_out, form, hb_next, act):
+    """SiLU / GELU through the table, both group widths, several tiles with ragged edges."""
+    from oracle import hatq_oracle as O
+    from tests.test_gpu_conv_lean import dev
+    rng = np.random.default_rng(c_out + hb_next)
+    L, wt = layer_from_codes(rng.integers(-60, 61, size=(c_out, 3, 3, 64)), form, 1, act)
+    x = rng.integers(-127, 128, size=(3, 33, 26, 64)).astype(np.int8)
+    s_z, s_u, s_y = (float(np.float32(v)) for v in (0.2, 0.15, 0.3))
+    P = H.prepare_weights(H.desc_from_spec(L), wt, None, 0.05, s_y, act, hb_next, s_z=s_z, s_u=s_u)
+    y = H.conv2d_i8(dev(x), P)
+    H.sync_status()
+    p = O.prepare_layer(wt, None, L.form, L.hb_in, L.hb_out, 0.05, s_y, act, hb_next, False, 1, 1, s_z=s_z, s_u=s_u)
+    ref = O.conv_layer(x, p)
+    assert np.array_equal(y.cpu().numpy(), ref)
+    assert len(np.unique(ref)) > 20

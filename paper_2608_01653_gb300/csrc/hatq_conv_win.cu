@@ -227,20 +227,23 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t alo0 = ((smem_addr(smem + a.w16_off) >> 4) & 0x3FFFu) | (1u << 16);
             const uint32_t b_step = (uint32_t)a.b_bytes >> 4, w_step = (uint32_t)a.w16_bytes >> 4;
             const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
-            int s = 0, ws = 0, g = 0;
+            int ws = 0, g = 0;
             uint32_t ph = 0, wph = 0, acc = 0, d = tm;
-            uint32_t bl = blo0;                              // weight stage s
+            uint32_t bl = blo0;                              // the weight stage's descriptor
             // one weight block: K steps 0-1 read the window at o0, 2-3 at o1 (nk of them)
+            uint32_t bar = b_full(0);                        // b_full of the stage; its b_empty is 64 bytes on
+            const uint32_t bar_end = b_full(S);
             auto step = [&](uint32_t o0, uint32_t o1, int nk) {
-                mbar_wait_issue(b_full(s), ph, abort_flag, a.err, tm, true);
+                mbar_wait_issue(bar, ph, abort_flag, a.err, tm, true);
                 umma_f16_ss_if(lead, d, o0, ahi, bl, bhi, idesc, acc);
                 if (nk > 1) umma_f16_ss_if(lead, d, o0 + 2, ahi, bl + 2, bhi, idesc, 1u);
                 if (nk > 2) umma_f16_ss_if(lead, d, o1, ahi, bl + 4, bhi, idesc, 1u);
                 if (nk > 3) umma_f16_ss_if(lead, d, o1 + 2, ahi, bl + 6, bhi, idesc, 1u);
-                umma_commit_if(lead, b_empty(s));
+                umma_commit_if(lead, bar + 64u);
                 acc = 1u;
                 bl += b_step;
-                if (++s == S) { s = 0; ph ^= 1u; bl = blo0; }
+                bar += 8u;
+                if (bar == bar_end) { bar = b_full(0); ph ^= 1u; bl = blo0; }
             };
             for (int j = 0; j < my_tiles; ++j) {
                 int left = a.cin_kb * a.par;                 // units left in the tile

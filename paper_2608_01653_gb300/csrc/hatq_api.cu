@@ -11,6 +11,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <algorithm>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -910,8 +911,15 @@ int win_plan(const hatq_conv_desc &d, const Geometry &g, const hatq_prepared &L,
     if ((long long)a.tiles_w * a.tiles_h * 128 * 4 > area * 5) return 0;
     a.n_t = g.n_t;
     a.n_tiles_n = d.c_out / g.n_t;
-    const long long nt = (long long)n * a.tiles_w * a.tiles_h * a.n_tiles_n;
-    if (nt >= (1LL << 31)) return 0;
+    const long long mt = (long long)n * a.tiles_w * a.tiles_h;
+    // CTA pairs halve the weight bytes a CTA loads and the issue work per MMA, but couple two CTAs
+    // (and cost about 1 us of launch): measured better from about 40 weight blocks per tile on (75: ga2
+    // 4.04 -> 3.79 ms, 45 and 90: h1 707 -> 683 and h2 1345 -> 1290 us), worse below (36: 159 -> 176,
+    // 18: 45 -> 48, 27 with 192 columns: 1557 -> 1580 us)
+    a.pair = g.k_pad / 64 >= 40;
+    const long long nt = (a.pair ? (mt + 1) / 2 : mt) * a.n_tiles_n;
+    if (nt >= (1LL << 30)) return 0;
+    a.n = n;
     a.num_tiles = (int)nt;
     a.kh = d.kh;
     a.kw = d.kw;
@@ -943,17 +951,32 @@ int win_plan(const hatq_conv_desc &d, const Geometry &g, const hatq_prepared &L,
     } else {
         epi = g.G;
     }
-    a.b_bytes = g.n_t * 128;
+    a.b_bytes = (a.pair ? g.n_t / 2 : g.n_t) * 128;  // this CTA's columns
     a.w8_bytes = (a.rows * 64 + 1023) & ~1023;
     a.w16_bytes = (a.rows * 128 + 1023) & ~1023;
-    const int const_bytes = (12 * d.c_out + (general ? 256 : 0) + 127) & ~127, bars = 8 * 33 + 16;
+    const int const_bytes = (12 * d.c_out + (general ? 256 : 0) + 127) & ~127, bars = 8 * 32 + 16;
     const int budget = 227 * 1024 - 1024 /* static */ - 1024 /* alignment */ - 8 * 4096 - 512 - const_bytes - 2 * a.w16_bytes;
-    // two INT8 buffers unless they cost weight stages below four
-    a.n8 = (budget - 2 * a.w8_bytes) / a.b_bytes >= 4 ? 2 : 1;
-    a.stages = (budget - a.n8 * a.w8_bytes) / a.b_bytes;
-    if (a.stages > 8) a.stages = 8;
-    if (a.stages < 2) return 0;
-    a.w16_off = a.stages * a.b_bytes;
+    // A weight stage holds the taps of one kernel row (a wait, a commit and the counters per row
+    // instead of per tap) where at least six blocks fit in two stages or more, preferably beside two
+    // INT8 window buffers; else single blocks, with the second window buffer where four stages remain.
+    const int row_taps = a.pairs ? 4 : (d.kw + a.par - 1) / a.par;
+    a.stages = 0;
+    for (int n8 = 2; n8 >= 1 && !a.stages; --n8)
+        for (int seg = row_taps; seg >= 1 && !a.stages; --seg) {
+            const int st = std::min(8, (budget - n8 * a.w8_bytes) / (seg * a.b_bytes));
+            if (st >= 2 && st * seg >= 6) {
+                a.stages = st;
+                a.seg = seg;
+                a.n8 = n8;
+            }
+        }
+    if (!a.stages) {
+        a.seg = 1;
+        a.n8 = (budget - 2 * a.w8_bytes) / a.b_bytes >= 4 ? 2 : 1;
+        a.stages = std::min(8, (budget - a.n8 * a.w8_bytes) / a.b_bytes);
+        if (a.stages < 2) return 0;
+    }
+    a.w16_off = a.stages * a.seg * a.b_bytes;
     a.w8_off = a.w16_off + 2 * a.w16_bytes;
     a.stg_off = a.w8_off + a.n8 * a.w8_bytes;
     a.bar_off = a.stg_off + 8 * 4096;
@@ -1065,12 +1088,12 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     // warpgroups, one half each (nbuf = 1).
     const bool drains = a.num_kb > a.chunk_kb;
     a.buf_cols = a.n_t;
-    a.nbuf = (drains || g.G == 128) ? 1 : 2;
     const bool general = L->act == HATQ_ACT_SILU || L->act == HATQ_ACT_GELU;
     // the lean kernels: INT8 codes of one exact chunk per tile, no further option
     const bool plain = !general && !L->out_f32 && !a.affine && !a.a_f16 && !a.out_f16 && !a.d2s;
     a.lean = !drains && plain;
     a.group = g.G;
+    a.nbuf = (drains || g.G == 128) ? 1 : 2;
     a.tmem_cols = 512;
     a.a_col = 2 * a.n_t;
     a.seg = g.seg;
@@ -1159,7 +1182,7 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
         const cuuint64_t dims[4] = {(cuuint64_t)a.co, (cuuint64_t)wo, (cuuint64_t)ho, (cuuint64_t)n};
         const cuuint64_t strides[3] = {px, rw, im};
         const int bx = win_smem ? 8 : (a.tw < 32 ? a.tw : 32);
-        const bool narrow = g.G == 32 || (win_smem && epi == 2064);
+        const bool narrow = win_smem ? epi == 32 || epi == 2064 || epi == 4032 : g.G == 32;
         const cuuint32_t box[4] = {narrow ? 32u : 64u, (cuuint32_t)bx, (cuuint32_t)(32 / bx), 1};
         const cuuint32_t estr[4] = {1, 1, 1, 1};
         void *base = static_cast<int8_t *>(y) + ((long long)a.ooy * a.y_w + a.oox) * a.co;
@@ -1180,6 +1203,12 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return fail(HATQ_ERR_CUDA, "input window tensor map encoding failed (%d)", (int)r);
+        // weights: as the prepared map, for a pair boxes of half the tile's columns
+        const cuuint64_t bdims[2] = {(cuuint64_t)L->k_pad, (cuuint64_t)d->c_out}, bstr[1] = {(cuuint64_t)L->k_pad * 2};
+        const cuuint32_t bbox[2] = {64, (cuuint32_t)(wa.pair ? wa.n_t / 2 : wa.n_t)}, bone[2] = {1, 1};
+        r = enc(&tmB, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, L->w_f16, bdims, bstr, bbox, bone, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return fail(HATQ_ERR_CUDA, "weight tensor map encoding failed (%d)", (int)r);
         wa.err = a.err;
         wa.y = y;
         cudaError_t e = hatq::launch_conv_win(tmA, tmB, tmY, wa, epi, win_smem, reinterpret_cast<cudaStream_t>(stream));

@@ -366,20 +366,13 @@ __device__ __forceinline__ void epi_split128(const EpiCtx &e, const ConvArgs &a,
 //
 // Layers that emit INT8 codes with no further option (no general transition,
 // float or fp16 output, affine operand or sub-pixel rearrangement) whose
-// reduction is one exact chunk. Each warp finishes its 32 pixel rows by itself:
-// the accumulator columns of a group are read with two tensor-memory loads in
-// flight, the region is released as soon as the last ones arrived, and the
-// codes leave as one TMA store per warp and 64 (32) columns from a swizzled
-// 32-row staging buffer (two per warp). Nothing waits for another warp, except
-// the pair of warps that shares the rows of a 128-wide group.
+// reduction is one exact chunk. Each warp finishes its 32 pixel rows by itself
+// (groups of 128 columns with the warp of the same rows in the other
+// warpgroup): the region is released as soon as the last columns arrived, and the
+// codes leave as one TMA store per warp and group from a swizzled staging buffer.
 // Bound: integer issue (38 integer operations per value of a WH(64) -> ReLU ->
-// DH(64) transition, the 64-bit adds on the integer pipe at half rate).
-// Against the epilogue with every option (named barriers and a copy loop per
-// tile, 16 columns per tensor-memory load, the shared register budget): the
-// analysis chain on 8 x 2160 x 3840 16.32 -> 15.35 ms (ga1 is half of it), the
-// entropy chains on 8 x 135 x 240 7.52 -> 7.24 ms, 512 x 768 analysis 215 -> 204 us.
-
-// (lean_scale, lean_codes and lean_store are in hatq_lean.h.)
+// DH(64) transition, the 64-bit adds on the integer pipe).
+// (The pieces are in hatq_lean.h.)
 
 // ------------------------------------------------------------------ kernel
 
@@ -903,7 +896,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             const bool inside = oy < a.ho && ox < a.wo;
             if constexpr (LEAN != 128) {
                 if (!ok) break;
+#pragma unroll 1
                 for (int col = 0; col < a.n_t; col += LEAN) {
+                    uint32_t w[LEAN / 4];
                     long long t[LEAN];
                     {
                         uint32_t r[LEAN];
@@ -917,85 +912,35 @@ __global__ void __launch_bounds__(kThreads, 1)
                         }
                         lean_scale<LEAN>(r, mbs + n0 + col, mults + n0 + col, t);
                     }
-                    if (a.hb_out) fwht_stages<LEAN>(t, a.hb_out);
-                    if (a.act) {
-#pragma unroll
-                        for (int i = 0; i < LEAN; ++i) t[i] = relu_mad(t[i]);
-                    }
-                    if (a.hb_next) fwht_stages<LEAN>(t, a.hb_next);
-                    uint32_t w[LEAN / 4];
+                    whole_transition<LEAN>(t, a.hb_out, a.hb_next, a.act);
                     lean_codes<LEAN>(a.shift, t, w);
                     lean_store<LEAN>(wstage + buf * (kWarpStage / 2), w, &tmY, lane, inside, n0 + col, ox, oy, img);
                     buf ^= 1;
                 }
             } else {
-                // A 128-column group shared by the two warps of a quadrant, warpgroup wg producing
-                // outputs 64 wg .. 64 wg + 63 (see epi_split128): both halves of the accumulator are
-                // read for hb_out = 128, and for hb_next = 128 the halves of phi are exchanged through
-                // the warps' first staging buffers, eight values per thread and round, at a barrier of
-                // the pair. Every warp runs the exchange barriers, also after an abort.
-                const int half = 64 * wg;
-                long long p[64];
-                {
-                    uint32_t r0[32], r1[32];
+                // groups shared by the two warps of a quadrant, H columns each; every warp runs the
+                // exchange barriers, also after an abort
+                constexpr int H = LEAN / 2;
+                const uint8_t *theirs = staging + (wg ? warp - 8 : warp) * kWarpStage;
+                const int ng = a.n_t / LEAN;
+#pragma unroll 1
+                for (int gr = 0; gr < ng; ++gr) {
+                    const int col = gr * LEAN + wg * H;
+                    long long t[H];
 #pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        if (a.hb_out == 128) {
-                            long long x[32];
-                            tmem_ld32(t_acc + 32 * q, r0);
-                            tmem_ld32(t_acc + 64 + 32 * q, r1);
-                            tmem_wait_ld();
-                            lean_scale<32>(r0, mbs + n0 + 32 * q, mults + n0 + 32 * q, p + 32 * q);
-                            lean_scale<32>(r1, mbs + n0 + 64 + 32 * q, mults + n0 + 64 + 32 * q, x);
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) p[32 * q + i] = wg ? p[32 * q + i] - x[i] : p[32 * q + i] + x[i];
-                        } else {
-                            tmem_ld32(t_acc + half + 32 * q, r0);
-                            tmem_wait_ld();
-                            lean_scale<32>(r0, mbs + n0 + half + 32 * q, mults + n0 + half + 32 * q, p + 32 * q);
+                    for (int q = 0; q < H / 32; ++q) {
+                        uint32_t r[32];
+                        tmem_ld32(t_acc + col + 32 * q, r);
+                        tmem_wait_ld();
+                        if (q == H / 32 - 1 && gr == ng - 1) {
+                            tc_fence_before();
+                            mbar_arrive(acc_empty(reg));
                         }
+                        lean_scale<32>(r, mbs + n0 + col + 32 * q, mults + n0 + col + 32 * q, t + 32 * q);
                     }
+                    split_finish<LEAN>(t, a.shift, a.hb_out, a.hb_next, a.act, wstage, theirs, wg, quad, lane, &tmY,
+                                       inside && ok, n0 + col, ox, oy, img);
                 }
-                tc_fence_before();
-                mbar_arrive(acc_empty(reg));
-                if (a.hb_out) fwht_stages<64>(p, min(a.hb_out, 64));
-                if (a.act) {
-#pragma unroll
-                    for (int i = 0; i < 64; ++i) p[i] = relu_mad(p[i]);
-                }
-                if (a.hb_next == 128) {
-                    // [pair k][row] in 16-byte units: a warp's accesses are 512 contiguous bytes
-                    int4 *mine = reinterpret_cast<int4 *>(wstage) + lane;
-                    const int4 *theirs =
-                        reinterpret_cast<const int4 *>(staging + (wg ? warp - 8 : warp) * kWarpStage) + lane;
-#pragma unroll
-                    for (int rd = 0; rd < 8; ++rd) {
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const long long u0 = p[8 * rd + 2 * k], u1 = p[8 * rd + 2 * k + 1];
-                            mine[k * 32] = make_int4((int)u0, (int)(u0 >> 32), (int)u1, (int)(u1 >> 32));
-                        }
-                        asm volatile("bar.sync %0, 64;" ::"r"(4 + quad) : "memory");
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int4 v = theirs[k * 32];
-                            const long long o0 = (long long)(((unsigned long long)(uint32_t)v.y << 32) | (uint32_t)v.x);
-                            const long long o1 = (long long)(((unsigned long long)(uint32_t)v.w << 32) | (uint32_t)v.z);
-                            const int i0 = 8 * rd + 2 * k;
-                            p[i0] = wg ? o0 - p[i0] : p[i0] + o0;           // u_0 - u_1 on the upper half, u_0 + u_1 on the lower
-                            p[i0 + 1] = wg ? o1 - p[i0 + 1] : p[i0 + 1] + o1;
-                        }
-                        asm volatile("bar.sync %0, 64;" ::"r"(4 + quad) : "memory");
-                    }
-                    fwht_fixed<64, 64>(p);
-                } else if (a.hb_next) {
-                    fwht_stages<64>(p, a.hb_next);
-                }
-                uint32_t w[16];
-                lean_codes<64>(a.shift, p, w);
-                // the second buffer holds every tile's codes (the exchange has the first): its last store is long read
-                if (lane == 0) bulk_wait_read<0>();
-                lean_store<64>(wstage + kWarpStage / 2, w, &tmY, lane, inside && ok, n0 + half, ox, oy, img);
             }
         }
         if (lane == 0) bulk_wait_all();

@@ -18,12 +18,23 @@
 // Exactness as in conv_kernel: chunks of whole units whose fp32 sums stay below
 // 2^24 for the layer's weight codes, chunk g in accumulator region g & 1.
 //
+// CTA pairs (PAIR; clusters of two, cta_group::2; taken for long reductions): the
+// pair takes two neighbouring M tiles of one N tile, each CTA its own window and
+// accumulator rows and half of the weight columns, and the leader's MMA warp issues
+// M = 256 instructions for both, so that a CTA loads and stores half the weight
+// bytes.
+//
+// The issue is what bounds the loop over weight blocks: a wait, four MMAs, a commit
+// and the counters take 240 cycles alone but 560-780 beside two epilogue warps per
+// scheduler, which keep the issue slots. So a weight stage holds the taps of a
+// kernel row (of one parity) where they fit, with one wait and commit for all.
+//
 // Persistent, one CTA per SM, 512 threads:
-//   warp 0       TMA of the weight blocks (64 x n_t fp16, one per tap and unit)
-//   warp 1       TMEM allocation, MMA issue
+//   warp 0       TMA of the weight blocks (64 x n_t / 2 fp16, one per tap and unit)
+//   warp 1       TMEM allocation; in the leader: MMA issue
 //   warp 2       TMA of the INT8 windows
-//   warps 4-11   epilogue (hatq_lean.h): with one chunk per tile the warpgroups
-//                take the tiles in turn; with 128-wide groups (EPI 1128) or drains
+//   warps 4-11   epilogue (hatq_lean.h): with one chunk per tile the warpgroups take
+//                the tiles in turn; with 128-wide groups (EPI 1128) or drains
 //                (EPI 2064, 2128) both share each tile, half of every group each
 //   warps 12-15  converters: INT8 window row -> fp16 window row
 // Every wait is bounded, as in conv_kernel.
@@ -41,8 +52,9 @@ using namespace tc;
 constexpr int kThreads = 512;
 
 // barriers from bar_off: b_full[8], b_empty[8], w8_full[2], w8_empty[2], w16_full[2],
-// w16_empty[2], acc_full[4], acc_empty[4], done; then the TMEM address and the abort flag
-constexpr int kBars = 33;
+// w16_empty[2], acc_full[4], acc_empty[4]; then the TMEM address and the abort flag.
+// The leader's b_full, w16_full and acc_empty count for the pair.
+constexpr int kBars = 32;
 
 // EPI, the epilogue: 32 / 64 whole tiles per warpgroup; 1128, 2064, 2128 shared
 // tiles of 128- / 64-wide groups, 2xxx with several chunks per tile: 2064 drains
@@ -50,41 +62,12 @@ constexpr int kBars = 33;
 // 3064 whole tiles with the sub-pixel rearrangement (factor 2); 4032 / 4064 whole
 // tiles with the general transition (SiLU / GELU).
 
-// Exchange of this warp's values with the warp of the same pixel rows in the
-// other warpgroup and the top butterfly of the group: the lower half keeps the
-// sums, the upper half the differences. Eight values per thread and round
-// through 2 KB per warp; every warp runs the barriers, also after an abort.
-template <int H>
-__device__ __forceinline__ void exchange_top(long long (&p)[H], uint8_t *mine_b, const uint8_t *theirs_b, int wg, int quad,
-                                             int lane) {
-    int4 *mine = reinterpret_cast<int4 *>(mine_b) + lane;
-    const int4 *theirs = reinterpret_cast<const int4 *>(theirs_b) + lane;
-#pragma unroll
-    for (int rd = 0; rd < H / 8; ++rd) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const long long u0 = p[8 * rd + 2 * k], u1 = p[8 * rd + 2 * k + 1];
-            mine[k * 32] = make_int4((int)u0, (int)(u0 >> 32), (int)u1, (int)(u1 >> 32));
-        }
-        asm volatile("bar.sync %0, 64;" ::"r"(4 + quad) : "memory");
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int4 v = theirs[k * 32];
-            const long long o0 = (long long)(((unsigned long long)(uint32_t)v.y << 32) | (uint32_t)v.x);
-            const long long o1 = (long long)(((unsigned long long)(uint32_t)v.w << 32) | (uint32_t)v.z);
-            const int i0 = 8 * rd + 2 * k;
-            p[i0] = wg ? o0 - p[i0] : p[i0] + o0;
-            p[i0 + 1] = wg ? o1 - p[i0 + 1] : p[i0 + 1] + o1;
-        }
-        asm volatile("bar.sync %0, 64;" ::"r"(4 + quad) : "memory");
-    }
-}
-
-template <int EPI>
+template <int EPI, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
     conv_win_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmY, const __grid_constant__ WinArgs a) {
     constexpr bool kSplit = EPI / 1000 == 1 || EPI / 1000 == 2, kDrain = EPI == 2064, kTwo = EPI == 2128;
+    static_assert(EPI == 32 || EPI == 64 || EPI == 1128 || kDrain || kTwo || EPI == 3064 || EPI / 1000 == 4, "epilogue");
     constexpr bool kD2s = EPI / 1000 == 3, kGeneral = EPI / 1000 == 4;
     constexpr int G = EPI % 1000;
     constexpr int kRegions = kTwo ? 4 : 2, kRegLog = kTwo ? 2 : 1;   // accumulator regions of n_t columns
@@ -100,16 +83,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto w16_empty = [&](int s) { return bar0 + 8u * (22 + s); };
     auto acc_full = [&](int s) { return bar0 + 8u * (24 + s); };
     auto acc_empty = [&](int s) { return bar0 + 8u * (28 + s); };
-    const uint32_t mma_done = bar0 + 8u * 32;
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(bar_area + 8 * kBars);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bar_area + 8 * kBars + 4);
 
-    // a failure already recorded ends every CTA that has not started
+    // a failure already recorded ends every pair that has not started (both CTAs alike: the leader's
+    // reading decides)
     __shared__ int s_skip;
+    const uint32_t rank = PAIR ? blockIdx.x & 1u : 0u;   // in the pair, 0 the leader
     if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile int *>(a.err);
-    __syncthreads();
-    if (s_skip != 0) return;
-
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int S = a.stages;
     if (threadIdx.x == 0) {
@@ -120,22 +101,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int s = 0; s < 2; ++s) {
             mbar_init(w8_full(s), 1);
             mbar_init(w8_empty(s), 128);
-            mbar_init(w16_full(s), 128);
+            mbar_init(w16_full(s), PAIR ? 8 : 4);    // converter warps
             mbar_init(w16_empty(s), 1);
         }
         for (int s = 0; s < kRegions; ++s) {
             mbar_init(acc_full(s), 1);
-            mbar_init(acc_empty(s), kSplit ? 256 : 128);
+            mbar_init(acc_empty(s), (kSplit ? 8 : 4) * (PAIR ? 2 : 1));   // epilogue warps
         }
-        mbar_init(mma_done, 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_holder)),
-                     "r"(512)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        tmem_alloc512<PAIR>(smem_addr(tmem_holder));
     }
     // bias products M b (64 bits) and multipliers of all output channels
     long long *mbs = reinterpret_cast<long long *>(bar_area + a.const_off);
@@ -149,16 +126,27 @@ __global__ void __launch_bounds__(kThreads, 1)
     if constexpr (kGeneral)
         for (int i = threadIdx.x; i < 256; i += kThreads) lut_s[i] = a.lut[i];
     tc_fence_before();
-    __syncthreads();
+    group_sync<PAIR>();                              // both CTAs' barriers are initialized
     tc_fence_after();
     const uint32_t tmem = *tmem_holder;
+    int skip = s_skip;
+    if constexpr (PAIR)
+        asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(skip) : "r"(leader_addr(smem_addr(&s_skip))) : "memory");
+    if (skip != 0) {
+        group_sync<PAIR>();                          // the leader's word has been read
+        if (warp == 1) tmem_dealloc512<PAIR>(tmem);
+        return;
+    }
 
-    const int my_tiles = a.num_tiles > (int)blockIdx.x ? (a.num_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    // pair tile t: M tiles 2 (t / n_tiles_n) + rank (the last may lie past the last image: its
+    // window reads zeros and nothing of it is stored), N tile t % n_tiles_n
+    const int pair = (int)blockIdx.x >> (PAIR ? 1 : 0), pairs = (int)gridDim.x >> (PAIR ? 1 : 0);
+    const int my_tiles = a.num_tiles > pair ? (a.num_tiles - 1 - pair) / pairs + 1 : 0;
     const int tiles_per_img = a.tiles_w * a.tiles_h;
     auto tile_coords = [&](int j, int &img, int &ho0, int &wo0, int &n0) {
-        const int t = (int)blockIdx.x + j * (int)gridDim.x;
-        const int mt = t / a.n_tiles_n;
-        n0 = (t - mt * a.n_tiles_n) * a.n_t;
+        const int t = pair + j * pairs;
+        const int pt = t / a.n_tiles_n, mt = PAIR ? 2 * pt + (int)rank : pt;
+        n0 = (t - pt * a.n_tiles_n) * a.n_t;
         img = mt / tiles_per_img;
         const int rem = mt - img * tiles_per_img;
         const int ty = rem / a.tiles_w;
@@ -177,27 +165,44 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t lead = elect_one() ? 1u : 0u;
         if (warp == 0) {
             // ------------------------------------------------------ weight producer
+            // each CTA loads its half of the columns; both halves count on the leader's barrier
             const uint32_t st0 = smem_addr(smem), bytes = (uint32_t)a.b_bytes;
-            int s = 0;
-            uint32_t ph = 1, st = st0;
-            auto load = [&](int k, int n0) {
-                mbar_wait_issue(b_empty(s), ph, abort_flag, a.err, tmem, false);
-                mbar_expect_tx_if(lead, b_full(s), bytes);
-                tma_load_2d_if(lead, st, &tmB, b_full(s), k, n0);
-                st += bytes;
-                if (++s == S) { s = 0; ph ^= 1u; st = st0; }
+            const uint32_t bars = b_empty(0), bars_end = b_empty(S);
+            const uint32_t to_full = (PAIR ? leader_addr(b_full(0)) : b_full(0)) - b_empty(0);   // b_empty here -> the leader's b_full
+            const uint32_t expect = rank == 0 ? lead : 0u;
+            const int half = (int)rank * (a.n_t / 2);
+            const uint32_t st_step = bytes * (uint32_t)a.seg;
+            uint32_t ph = 1, st = st0, bar = bars;
+            // one stage: m blocks whose weight columns start at k, k + dk, ...
+            auto load = [&](int k, int dk, int m, int n0) {
+                mbar_wait_issue<PAIR>(bar, ph, abort_flag, a.err, tmem, false);
+                mbar_expect_tx_if(expect, bar - 64u, (PAIR ? 2u : 1u) * bytes * (uint32_t)m);
+                uint32_t dst = st;
+#pragma unroll 1
+                for (int i = 0; i < m; ++i, k += dk, dst += bytes)
+                    if constexpr (PAIR) tma_load_2d_pair_if(lead, dst, &tmB, bar + to_full, k, n0 + half);
+                    else tma_load_2d_if(lead, dst, &tmB, bar - 64u, k, n0);
+                st += st_step;
+                bar += 8u;
+                if (bar == bars_end) { bar = bars; ph ^= 1u; st = st0; }
             };
+            const int dk = a.par * a.k_tap;                  // weight columns between a row's taps
             for (int j = 0; j < my_tiles; ++j) {
                 int img, ho0, wo0, n0;
                 tile_coords(j, img, ho0, wo0, n0);
                 if (a.pairs) {
-                    for (int i = 0; i < a.kblocks; ++i) load(i * 64, n0);
+                    for (int i = 0; i < a.kblocks; i += a.seg) load(i * 64, 64, min(a.seg, a.kblocks - i), n0);
                     continue;
                 }
                 for (int cb = 0; cb < a.cin_kb; ++cb)
                     for (int p = 0; p < a.par; ++p)
-                        for (int ky = 0; ky < a.kh; ++ky)
-                            for (int kx = p; kx < a.kw; kx += a.par) load((ky * a.kw + kx) * a.k_tap + cb * 64, n0);
+                    {
+                        const int taps = a.par == 2 ? (a.kw - p + 1) >> 1 : a.kw;        // of a kernel row
+                        int k = p * a.k_tap + cb * 64;
+                        for (int ky = 0; ky < a.kh; ++ky, k += a.kw * a.k_tap)
+                            for (int t = 0; t < taps; t += a.seg)
+                                load(k + t * dk, dk, min(a.seg, taps - t), n0);
+                    }
             }
         } else if (warp == 2) {
             // ------------------------------------------------------ window producer
@@ -209,16 +214,16 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int x0 = wo0 * a.stride - a.pad_x, y0 = ho0 * a.stride - a.pad_y;
                 for (int cb = 0; cb < a.cin_kb; ++cb)
                     for (int p = 0; p < a.par; ++p) {
-                        mbar_wait_issue(w8_empty(s), ph, abort_flag, a.err, tmem, false);
+                        mbar_wait_issue<PAIR>(w8_empty(s), ph, abort_flag, a.err, tmem, false);
                         mbar_expect_tx_if(lead, w8_full(s), (uint32_t)(a.rows * 64));
                         tma_load_4d_if(lead, smem_addr(smem) + (uint32_t)(a.w8_off + s * a.w8_bytes), &tmA, w8_full(s), cb * 64,
                                        x0 + p, y0, img);
                         if (++s == a.n8) { s = 0; ph ^= 1u; }
                     }
             }
-        } else if (warp == 1) {
+        } else if (warp == 1 && rank == 0) {
             // ------------------------------------------------------ MMA issuer
-            const uint32_t idesc = idesc_f16(a.n_t);
+            const uint32_t idesc = idesc_f16(a.n_t, PAIR ? 256 : 128);
             // descriptor halves: start address (and the unused leading offset) in the low word; group
             // stride, version and 128-byte swizzle in the high word
             const uint32_t bhi = (1024u >> 4) | (1u << 14) | (2u << 29);
@@ -230,20 +235,30 @@ __global__ void __launch_bounds__(kThreads, 1)
             int ws = 0, g = 0;
             uint32_t ph = 0, wph = 0, acc = 0, d = tm;
             uint32_t bl = blo0;                              // the weight stage's descriptor
-            // one weight block: K steps 0-1 read the window at o0, 2-3 at o1 (nk of them)
+            const uint32_t st_step = b_step * (uint32_t)a.seg, row_step = (uint32_t)(a.pitch * 8);
             uint32_t bar = b_full(0);                        // b_full of the stage; its b_empty is 64 bytes on
             const uint32_t bar_end = b_full(S);
-            auto step = [&](uint32_t o0, uint32_t o1, int nk) {
-                mbar_wait_issue(bar, ph, abort_flag, a.err, tm, true);
-                umma_f16_ss_if(lead, d, o0, ahi, bl, bhi, idesc, acc);
-                if (nk > 1) umma_f16_ss_if(lead, d, o0 + 2, ahi, bl + 2, bhi, idesc, 1u);
-                if (nk > 2) umma_f16_ss_if(lead, d, o1, ahi, bl + 4, bhi, idesc, 1u);
-                if (nk > 3) umma_f16_ss_if(lead, d, o1 + 2, ahi, bl + 6, bhi, idesc, 1u);
-                umma_commit_if(lead, bar + 64u);
+            // one weight block: K steps 0-1 read the window at o0, 2-3 at o1 (nk of them)
+            auto block = [&](uint32_t o0, uint32_t o1, uint32_t b, int nk) {
+                umma_f16_ss_if<PAIR>(lead, d, o0, ahi, b, bhi, idesc, acc);
+                if (nk > 1) umma_f16_ss_if<PAIR>(lead, d, o0 + 2, ahi, b + 2, bhi, idesc, 1u);
+                if (nk > 2) umma_f16_ss_if<PAIR>(lead, d, o1, ahi, b + 4, bhi, idesc, 1u);
+                if (nk > 3) umma_f16_ss_if<PAIR>(lead, d, o1 + 2, ahi, b + 6, bhi, idesc, 1u);
                 acc = 1u;
-                bl += b_step;
+            };
+            auto stage_done = [&]() {
+                umma_commit_if<PAIR>(lead, bar + 64u);
+                bl += st_step;
                 bar += 8u;
                 if (bar == bar_end) { bar = b_full(0); ph ^= 1u; bl = blo0; }
+            };
+            // one stage of a kernel row: m taps from window offset o on
+            auto row = [&](uint32_t o, int m, int nk) {
+                mbar_wait_issue<PAIR>(bar, ph, abort_flag, a.err, tm, true);
+                uint32_t b = bl;
+#pragma unroll 1
+                for (int i = 0; i < m; ++i, o += 8, b += b_step) block(o, o + 4, b, nk);
+                stage_done();
             };
             for (int j = 0; j < my_tiles; ++j) {
                 int left = a.cin_kb * a.par;                 // units left in the tile
@@ -255,52 +270,53 @@ __global__ void __launch_bounds__(kThreads, 1)
                             d = tm + (uint32_t)(reg * a.n_t);
                             acc = 0u;
                             if (g >= kRegions)
-                                mbar_wait_issue(acc_empty(reg), ((g >> kRegLog) - 1) & 1, abort_flag, a.err, tm, true);
+                                mbar_wait_issue<PAIR>(acc_empty(reg), ((g >> kRegLog) - 1) & 1, abort_flag, a.err, tm, true);
                         }
-                        mbar_wait_issue(w16_full(ws), wph, abort_flag, a.err, tm, true);
+                        mbar_wait_issue<PAIR>(w16_full(ws), wph, abort_flag, a.err, tm, true);
                         tc_fence_after();
                         const uint32_t w0 = alo0 + (uint32_t)ws * w_step;
                         if (a.pairs) {
                             // two 32-channel taps per weight block (64 bytes of each window row are zero)
                             int ky = 0, kx = 0;
-                            for (int i = 0; i < a.kblocks; ++i) {
-                                const uint32_t o0 = w0 + (uint32_t)((ky * a.pitch + kx) * 8);
-                                if (++kx == a.kw) { kx = 0; ++ky; }
-                                const int nk = ky < a.kh ? 4 : 2;
-                                const uint32_t o1 = w0 + (uint32_t)((ky * a.pitch + kx) * 8);
-                                if (++kx == a.kw) { kx = 0; ++ky; }
-                                step(o0, o1, nk);
-                            }
-                        } else if (cb == a.cin_kb - 1 && a.nk_last < 4) {
-                            for (int ky = 0; ky < a.kh; ++ky) {
-                                uint32_t o = w0 + (uint32_t)(ky * a.pitch * 8);
-                                for (int kx = p; kx < a.kw; kx += a.par, o += 8) step(o, o + 4, a.nk_last);
+                            for (int i0 = 0; i0 < a.kblocks; i0 += a.seg) {
+                                mbar_wait_issue<PAIR>(bar, ph, abort_flag, a.err, tm, true);
+                                uint32_t b = bl;
+                                const int m = min(a.seg, a.kblocks - i0);
+#pragma unroll 1
+                                for (int i = 0; i < m; ++i, b += b_step) {
+                                    const uint32_t o0 = w0 + (uint32_t)((ky * a.pitch + kx) * 8);
+                                    if (++kx == a.kw) { kx = 0; ++ky; }
+                                    const int nk = ky < a.kh ? 4 : 2;
+                                    const uint32_t o1 = w0 + (uint32_t)((ky * a.pitch + kx) * 8);
+                                    if (++kx == a.kw) { kx = 0; ++ky; }
+                                    block(o0, o1, b, nk);
+                                }
+                                stage_done();
                             }
                         } else {
-                            for (int ky = 0; ky < a.kh; ++ky) {
-                                uint32_t o = w0 + (uint32_t)(ky * a.pitch * 8);
-                                for (int kx = p; kx < a.kw; kx += a.par, o += 8) step(o, o + 4, 4);
-                            }
+                            const int taps = a.par == 2 ? (a.kw - p + 1) >> 1 : a.kw;    // of a kernel row
+                            const int nk = cb == a.cin_kb - 1 ? a.nk_last : 4;
+                            uint32_t orow = w0;
+                            for (int ky = 0; ky < a.kh; ++ky, orow += row_step)
+                                for (int t = 0; t < taps; t += a.seg)
+                                    row(orow + (uint32_t)(8 * t), min(a.seg, taps - t), nk);
                         }
-                        umma_commit_if(lead, w16_empty(ws));
+                        umma_commit_if<PAIR>(lead, w16_empty(ws));
                         if (++ws == 2) { ws = 0; wph ^= 1u; }
                         --left;
                         if (++cu == a.chunk_units || left == 0) {
-                            umma_commit_if(lead, acc_full(g & (kRegions - 1)));
+                            umma_commit_if<PAIR>(lead, acc_full(g & (kRegions - 1)));
                             ++g;
                             cu = 0;
                         }
                     }
             }
-            umma_commit_if(lead, mma_done);
-            const long long t0 = clock64();
-            while (!mbar_try_wait(mma_done, 0) && clock64() - t0 < kWaitLimitCycles) {
-            }
+            // (the epilogues end after the last chunk's commit, which covers every MMA)
         }
     } else if (warp >= 12) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;" ::: "memory");
         // ---------------------------------------------------------- converters
-        const int t = (int)threadIdx.x - 384;
+        const int row0 = ((int)threadIdx.x - 384) >> 2, q4 = (int)threadIdx.x & 3;
         bool ok = true;
         int s8 = 0, s16 = 0;
         uint32_t p8 = 0, p16 = 0;
@@ -311,24 +327,37 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!ok) break;
             const uint8_t *src = smem + a.w8_off + s8 * a.w8_bytes;
             uint8_t *dst = smem + a.w16_off + s16 * a.w16_bytes;
-#pragma unroll 2
-            for (int r = t; r < a.rows; r += 128) {
-                // 64 codes (64-byte swizzle) -> 64 fp16 values (128-byte swizzle)
-                const int sw8 = (r >> 1) & 3, sw16 = r & 7;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const uint4 v = *reinterpret_cast<const uint4 *>(src + r * 64 + ((q ^ sw8) << 4));
-                    uint4 lo, hi;
-                    i8x4_to_f16x4(v.x, lo.x, lo.y);
-                    i8x4_to_f16x4(v.y, lo.z, lo.w);
-                    i8x4_to_f16x4(v.z, hi.x, hi.y);
-                    i8x4_to_f16x4(v.w, hi.z, hi.w);
-                    *reinterpret_cast<uint4 *>(dst + r * 128 + (((2 * q) ^ sw16) << 4)) = lo;
-                    *reinterpret_cast<uint4 *>(dst + r * 128 + (((2 * q + 1) ^ sw16) << 4)) = hi;
-                }
+            // 16 codes (64-byte swizzle) -> 16 fp16 values (128-byte swizzle) per step; a thread keeps
+            // its quarter of the row and moves on by 32 rows, so its swizzle terms stay the same
+            const uint8_t *sp = src + row0 * 64 + ((q4 ^ ((row0 >> 1) & 3)) << 4);
+            uint8_t *dp = dst + row0 * 128;
+            const int d0 = ((2 * q4) ^ (row0 & 7)) << 4, d1 = ((2 * q4 + 1) ^ (row0 & 7)) << 4;
+            auto convert = [&](const uint4 &v, uint8_t *out) {
+                uint4 lo, hi;
+                i8x4_to_f16x4(v.x, lo.x, lo.y);
+                i8x4_to_f16x4(v.y, lo.z, lo.w);
+                i8x4_to_f16x4(v.z, hi.x, hi.y);
+                i8x4_to_f16x4(v.w, hi.z, hi.w);
+                *reinterpret_cast<uint4 *>(out + d0) = lo;
+                *reinterpret_cast<uint4 *>(out + d1) = hi;
+            };
+            int r = row0;
+#pragma unroll 1
+            for (; r + 64 < a.rows; r += 96, sp += 96 * 64, dp += 96 * 128) {
+                const uint4 v0 = *reinterpret_cast<const uint4 *>(sp), v1 = *reinterpret_cast<const uint4 *>(sp + 32 * 64);
+                const uint4 v2 = *reinterpret_cast<const uint4 *>(sp + 64 * 64);
+                convert(v0, dp);
+                convert(v1, dp + 32 * 128);
+                convert(v2, dp + 64 * 128);
             }
+#pragma unroll 1
+            for (; r < a.rows; r += 32, sp += 32 * 64, dp += 32 * 128) convert(*reinterpret_cast<const uint4 *>(sp), dp);
             fence_async_shared();                    // the MMAs read the window through the async proxy
-            mbar_arrive(w16_full(s16));
+            __syncwarp();
+            if (lane == 0) {
+                if constexpr (PAIR) mbar_arrive_cluster(leader_addr(w16_full(s16)));
+                else mbar_arrive(w16_full(s16));
+            }
             mbar_arrive(w8_empty(s8));
             if (++s8 == a.n8) { s8 = 0; p8 ^= 1u; }
             if (++s16 == 2) { s16 = 0; p16 ^= 1u; }
@@ -343,37 +372,45 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint8_t *wstage = staging + (warp - 4) * kWarpStage;
         bool ok = true;
         int buf = 0;
+        // this warp's tensor-memory reads of a region are done (fenced by every lane)
+        auto release = [&](int r) {
+            __syncwarp();
+            if (lane == 0) {
+                if constexpr (PAIR) mbar_arrive_cluster(leader_addr(acc_empty(r)));
+                else mbar_arrive(acc_empty(r));
+            }
+        };
         for (int j = 0; j < my_tiles; ++j) {
             if (!kSplit && (j & 1) != wg) continue;
             int img, ho0, wo0, n0;
             tile_coords(j, img, ho0, wo0, n0);
             const int oy = ho0 + 4 * quad, ox = wo0;       // this warp's 32 rows: 4 x 8 pixels
-            const bool inside = oy < a.ho && ox < a.wo;
+            const bool inside = oy < a.ho && ox < a.wo && img < a.n;
             if constexpr (!kSplit) {
                 const int reg = j & 1;
                 const uint32_t t_acc = t_lane + (uint32_t)(reg * a.n_t);
                 ok = __all_sync(0xffffffffu, mbar_wait(acc_full(reg), (j >> 1) & 1, abort_flag, a.err));
                 tc_fence_after();
                 if (!ok) break;
+#pragma unroll 1
                 for (int col = 0; col < a.n_t; col += G) {
                     long long t[G];
-                    {
-                        uint32_t r[G];
 #pragma unroll
-                        for (int q = 0; q < G / 32; ++q)
-                            tmem_ld32(t_acc + col + 32 * q, reinterpret_cast<uint32_t(&)[32]>(r[32 * q]));
+                    for (int q = 0; q < G / 32; ++q) {
+                        uint32_t r[32];
+                        tmem_ld32(t_acc + col + 32 * q, r);
                         tmem_wait_ld();
-                        if (col + G >= a.n_t) {            // TMEM reads of this region are complete
+                        if (q == G / 32 - 1 && col + G >= a.n_t) {         // TMEM reads of this region are complete
                             tc_fence_before();
-                            mbar_arrive(acc_empty(reg));
+                            release(reg);
                         }
-                        lean_scale<G>(r, mbs + n0 + col, mults + n0 + col, t);
+                        lean_scale<32>(r, mbs + n0 + col + 32 * q, mults + n0 + col + 32 * q, t + 32 * q);
                     }
-                    if (a.hb_out) fwht_stages<G>(t, a.hb_out);
                     uint32_t w[G / 4];
                     if constexpr (kGeneral) {
                         // z = clamp(round(H~_out (M_out (.) a) / 2^n_out)), u = phi_int(z), then the next
                         // layer's transform on u itself (|H~ u| <= 127 * 64) and its requantization
+                        if (a.hb_out) fwht_stages<G>(t, a.hb_out);
                         int u[G];
 #pragma unroll
                         for (int i = 0; i < G; ++i) u[i] = (int)lut_s[requant8_any(t[i], a.shift) + 127];
@@ -386,11 +423,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                             w[i] = pack4(q[0], q[1], q[2], q[3]);
                         }
                     } else {
-                        if (a.act) {
-#pragma unroll
-                            for (int i = 0; i < G; ++i) t[i] = relu_mad(t[i]);
-                        }
-                        if (a.hb_next) fwht_stages<G>(t, a.hb_next);
+                        whole_transition<G>(t, a.hb_out, a.hb_next, a.act);
                         lean_codes<G>(a.shift, t, w);
                     }
                     if constexpr (kD2s) {
@@ -410,7 +443,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                             o[3][q] = __byte_perm(t2, t3, 0x7632);
                         }
                         const int py = oy + (lane >> 3), px = ox + (lane & 7);
-                        if (py < a.ho && px < a.wo) {
+                        if (py < a.ho && px < a.wo && img < a.n) {
                             uint8_t *y = static_cast<uint8_t *>(a.y) + (n0 + col) / 4 +
                                          (((long long)img * a.ho + py) * 4 * a.wo + 2 * px) * (a.co / 4);
 #pragma unroll
@@ -452,11 +485,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                         }
                     }
                     tc_fence_before();
-                    mbar_arrive(acc_empty(reg));
+                    release(reg);
                 }
                 if (ng == 0) {                             // n_t = 32: the other warpgroup has the tile
                     tc_fence_before();
-                    mbar_arrive(acc_empty((j * a.nch + a.nch - 1) & (kRegions - 1)));
+                    release((j * a.nch + a.nch - 1) & (kRegions - 1));
                     continue;
                 }
                 // the last chunk's region; with 2128 both chunks of the tile still sit in regions of their own
@@ -465,9 +498,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (ok) ok = __all_sync(0xffffffffu, mbar_wait(acc_full(reg0), ((gc - 1) >> kRegLog) & 1, abort_flag, a.err));
                 if (ok) ok = __all_sync(0xffffffffu, mbar_wait(acc_full(reg), (gc >> kRegLog) & 1, abort_flag, a.err));
                 tc_fence_after();
-#pragma unroll
-                for (int gr = 0; gr < NP; ++gr) {
-                    if (gr >= ng) break;
+                // one copy of this code for all groups: unrolled it would not fit the instruction cache
+#pragma unroll 1
+                for (int gr = 0; gr < ng; ++gr) {
                     const int col = gr * G + wg * H;
                     long long t[H];
 #pragma unroll
@@ -478,8 +511,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                         tmem_wait_ld();
                         if (q == H / 32 - 1 && gr == ng - 1) {
                             tc_fence_before();
-                            mbar_arrive(acc_empty(reg));
-                            if constexpr (kTwo) mbar_arrive(acc_empty(reg0));
+                            release(reg);
+                            if constexpr (kTwo) release(reg0);
                         }
                         const long long *mb = mbs + n0 + col + 32 * q;
                         const int *mu = mults + n0 + col + 32 * q;
@@ -492,7 +525,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                             for (int k = 0; k < 4; ++k) {
                                 v[k] = __float2int_rn(__uint_as_float(r[i + k]));
-                                if constexpr (kDrain) v[k] += (int)part[gr][32 * q + i + k];
+                                if constexpr (kDrain)     // (selected, as registers have no index)
+                                    v[k] += (int)(gr == 0 ? part[0][i + k] : (gr == 1 ? part[1][i + k] : part[2][i + k]));
                                 if constexpr (kTwo) v[k] += __float2int_rn(__uint_as_float(r0[i + k]));
                             }
                             t[32 * q + i] = (long long)m.x * v[0] + b0.x;
@@ -501,24 +535,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                             t[32 * q + i + 3] = (long long)m.w * v[3] + b1.y;
                         }
                     }
-                    if (a.hb_out == G) exchange_top<H>(t, wstage, theirs, wg, quad, lane);
-                    if (a.hb_out) fwht_stages<H>(t, min(a.hb_out, H));
-                    if (a.act) {
-#pragma unroll
-                        for (int i = 0; i < H; ++i) t[i] = relu_mad(t[i]);
-                    }
-                    if (a.hb_next == G) exchange_top<H>(t, wstage, theirs, wg, quad, lane);
-                    if (a.hb_next) fwht_stages<H>(t, min(a.hb_next, H));
-                    uint32_t w[H / 4];
-                    lean_codes<H>(a.shift, t, w);
-                    uint8_t *out = wstage + kWarpStage / 2;
-                    if constexpr (H == 32) {
-                        out += buf * 1024;                 // two 1 KB buffers
-                        buf ^= 1;
-                    } else if (lane == 0) {
-                        bulk_wait_read<0>();               // one 2 KB buffer
-                    }
-                    lean_store<H>(out, w, &tmY, lane, inside && ok, n0 + col, ox, oy, img);
+                    split_finish<G>(t, a.shift, a.hb_out, a.hb_next, a.act, wstage, theirs, wg, quad, lane, &tmY,
+                                    inside && ok, n0 + col, ox, oy, img);
                 }
             }
         }
@@ -526,10 +544,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 
     tc_fence_before();
-    __syncthreads();
+    group_sync<PAIR>();                              // nothing of the other CTA reaches this one any more
     tc_fence_after();
-    if (warp == 1)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    if (warp == 1) tmem_dealloc512<PAIR>(tmem);
 }
 
 }  // namespace
@@ -537,35 +554,46 @@ __global__ void __launch_bounds__(kThreads, 1)
 cudaError_t launch_conv_win(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmY, const WinArgs &a, int epi,
                             int smem_bytes, cudaStream_t s) {
     using Fn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const WinArgs);
-    static const struct { int epi; Fn fn; } kerns[] = {
-        {32, conv_win_kernel<32>},     {64, conv_win_kernel<64>},     {1128, conv_win_kernel<1128>},
-        {2064, conv_win_kernel<2064>}, {2128, conv_win_kernel<2128>}, {3064, conv_win_kernel<3064>},
-        {4032, conv_win_kernel<4032>}, {4064, conv_win_kernel<4064>}};
+#define HATQ_WIN(e) {e, {conv_win_kernel<e, false>, conv_win_kernel<e, true>}}
+    static const struct { int epi; Fn fn[2]; } kerns[] = {HATQ_WIN(32),   HATQ_WIN(64),   HATQ_WIN(1128), HATQ_WIN(2064),
+                                                          HATQ_WIN(2128), HATQ_WIN(3064), HATQ_WIN(4032), HATQ_WIN(4064)};
+#undef HATQ_WIN
     constexpr int kKerns = sizeof(kerns) / sizeof(kerns[0]);
     int v = 0;
     while (v < kKerns && kerns[v].epi != epi) ++v;
     if (v == kKerns) return cudaErrorInvalidValue;
-    const Fn kern = kerns[v].fn;
+    const int pr = a.pair ? 1 : 0;
+    const Fn kern = kerns[v].fn[pr];
     // the shared-memory opt-in and the SM count are per device
     constexpr int kMaxDev = 64;
-    static int configured[kMaxDev][kKerns] = {};
+    static int configured[kMaxDev][kKerns][2] = {};
     static int sms_of[kMaxDev] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDev) return cudaErrorInvalidDevice;
-    if (smem_bytes > configured[dev][v]) {
+    if (smem_bytes > configured[dev][v][pr]) {
         if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes)) != cudaSuccess) return e;
-        configured[dev][v] = smem_bytes;
+        configured[dev][v][pr] = smem_bytes;
     }
     if (!sms_of[dev]) {
         int sms = 0;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         sms_of[dev] = sms > 0 ? sms : 1;
     }
-    const int grid = a.num_tiles < sms_of[dev] ? a.num_tiles : sms_of[dev];
-    kern<<<grid, kThreads, smem_bytes, s>>>(tmA, tmB, tmY, a);
-    return cudaGetLastError();
+    const int groups = pr ? (sms_of[dev] / 2 < 1 ? 1 : sms_of[dev] / 2) : sms_of[dev];
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((pr ? 2 : 1) * (a.num_tiles < groups ? a.num_tiles : groups));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem_bytes;
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 2;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = pr;
+    return cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmY, a);
 }
 
 }  // namespace hatq

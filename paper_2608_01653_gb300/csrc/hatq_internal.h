@@ -152,8 +152,9 @@ cudaError_t launch_conv(const CUtensorMap &tmA, const CUtensorMap &tmB, const CU
 // once in shared memory and every kernel tap's MMAs read it through a shifted
 // descriptor.
 struct WinArgs {
-    int ho, wo, co;                  // output grid of the launch
-    int tiles_w, tiles_h, num_tiles, n_tiles_n, n_t;   // 8 x 16-pixel M tiles, n_t-channel N tiles
+    int n, ho, wo, co;               // images, output grid of the launch
+    int pair;                        // CTA pairs: two M tiles of one N tile each
+    int tiles_w, tiles_h, num_tiles, n_tiles_n, n_t;   // 8 x 16-pixel M tiles; (pairs of) them x n_t-channel N tiles
     int kh, kw, stride, pad_y, pad_x;
     int par;                         // column parities with taps (stride 2, kw > 1: 2, else 1)
     int cin_kb;                      // 64-channel blocks; units per tile = cin_kb * par
@@ -163,7 +164,7 @@ struct WinArgs {
     int kblocks;                     // pairs: weight blocks
     int pitch, rows;                 // window columns (of one parity) and rows * columns
     int chunk_units, nch;            // units per exact chunk, chunks per tile
-    int stages, n8;                  // weight stages, INT8 window buffers (1 or 2)
+    int stages, seg, n8;             // weight stages, blocks per stage (taps of one kernel row), INT8 window buffers
     int b_bytes, w8_bytes, w16_bytes;
     int w8_off, w16_off, stg_off, bar_off, const_off;   // shared-memory offsets (weight stages at 0)
     const int32_t *b_int, *mult;

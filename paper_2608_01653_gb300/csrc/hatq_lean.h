@@ -94,5 +94,87 @@ __device__ __forceinline__ void lean_store(uint8_t *buf, const uint32_t (&w)[G /
     }
 }
 
+// ------------------------------------------------------------------ transitions
+//
+// Code size: 64 values per thread with each transform written out are 46 KB of
+// straight-line code. Beyond about 32 KB the instruction cache misses: a warp
+// then issues every 3.1 cycles instead of every 1.1 (measured on the 64-point
+// transform alone), and the short loops of the other roles are evicted all the
+// time. So both transforms of a transition are one copy of code in a loop of two
+// passes, and loops over groups stay rolled.
+
+// H~_out, phi, H~_next of G columns held by one thread.
+template <int G>
+__device__ __forceinline__ void whole_transition(long long (&t)[G], int hb_out, int hb_next, int act) {
+    if (hb_out) fwht_stages<G>(t, hb_out);
+    if (act) {
+#pragma unroll
+        for (int i = 0; i < G; ++i) t[i] = relu_mad(t[i]);
+    }
+    if (hb_next) fwht_stages<G>(t, hb_next);
+}
+
+// Groups shared by the two warps of a quadrant, one of each epilogue warpgroup: a
+// thread finishes H = G / 2 of a row's columns, and the halves meet in the group's
+// top butterfly: the lower half keeps the sums, the upper half the differences
+// (lower - upper). Eight values per thread and round through the warps' staging, one
+// barrier of the pair per round: rounds alternate between the two 2 KB halves, and a
+// half is written again only after the next round's barrier, which the partner
+// reaches after reading it. Every warp runs the barriers, also after an abort.
+template <int H>
+__device__ __forceinline__ void exchange_top(long long (&p)[H], uint8_t *mine_b, const uint8_t *theirs_b, int wg, int quad,
+                                             int lane) {
+#pragma unroll
+    for (int rd = 0; rd < H / 8; ++rd) {
+        int4 *mine = reinterpret_cast<int4 *>(mine_b + (rd & 1) * (kWarpStage / 2)) + lane;
+        const int4 *theirs = reinterpret_cast<const int4 *>(theirs_b + (rd & 1) * (kWarpStage / 2)) + lane;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const long long u0 = p[8 * rd + 2 * k], u1 = p[8 * rd + 2 * k + 1];
+            mine[k * 32] = make_int4((int)u0, (int)(u0 >> 32), (int)u1, (int)(u1 >> 32));
+        }
+        asm volatile("bar.sync %0, 64;" ::"r"(4 + quad) : "memory");
+        if (wg) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) p[8 * rd + k] = -p[8 * rd + k];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int4 v = theirs[k * 32];
+            p[8 * rd + 2 * k] += (long long)(((unsigned long long)(uint32_t)v.y << 32) | (uint32_t)v.x);
+            p[8 * rd + 2 * k + 1] += (long long)(((unsigned long long)(uint32_t)v.w << 32) | (uint32_t)v.z);
+        }
+    }
+}
+
+// From t = M a + M b to the stored codes of this warp's half group (channels ch ..
+// ch + H - 1 of the box at (ox, oy) of image img). The codes take the staging half
+// that the exchange's last round did not use.
+template <int G>
+__device__ __forceinline__ void split_finish(long long (&t)[G / 2], int shift, int hb_out, int hb_next, int act, uint8_t *wstage,
+                                             const uint8_t *theirs, int wg, int quad, int lane, const CUtensorMap *tmY,
+                                             bool inside, int ch, int ox, int oy, int img) {
+    constexpr int H = G / 2;
+    if (lane == 0) bulk_wait_read<0>();                  // the previous group's store has left the staging
+    __syncwarp();
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+        const int hb = pass ? hb_next : hb_out;
+        if (hb == G) {
+            if (pass && hb_out == G)                     // the partner has read the first exchange's last round
+                asm volatile("bar.sync %0, 64;" ::"r"(4 + quad) : "memory");
+            exchange_top<H>(t, wstage, theirs, wg, quad, lane);
+        }
+        if (hb) fwht_stages<H>(t, min(hb, H));
+        if (!pass && act) {
+#pragma unroll
+            for (int i = 0; i < H; ++i) t[i] = relu_mad(t[i]);
+        }
+    }
+    uint32_t w[H / 4];
+    lean_codes<H>(shift, t, w);
+    lean_store<H>(wstage, w, tmY, lane, inside, ch, ox, oy, img);
+}
+
 }  // namespace tc
 }  // namespace hatq

@@ -85,41 +85,105 @@ __device__ __forceinline__ void tma_load_4d_if(uint32_t pr, uint32_t dst, const 
         "l"(tm), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(pr)
         : "memory");
 }
+// ------------------------------------------------------------------ CTA pairs
+// Two CTAs of a cluster on neighbouring SMs, the even one the leader: its MMA warp
+// issues for both (cta_group::2), barriers it waits on are reached from the other
+// CTA by their cluster addresses.
+// the address of this CTA's shared-memory location in the leader CTA
+__device__ __forceinline__ uint32_t leader_addr(uint32_t addr) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
+    return r;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+// The CTA group's barrier over all threads: the pair's, or the CTA's own.
+template <bool PAIR>
+__device__ __forceinline__ void group_sync() {
+    if constexpr (PAIR) cluster_sync();
+    else asm volatile("barrier.sync 0;" ::: "memory");
+}
+// Tensor memory: all 512 columns, by one warp (of each CTA of a pair).
+template <bool PAIR>
+__device__ __forceinline__ void tmem_alloc512(uint32_t holder) {
+    if constexpr (PAIR) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(holder), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(holder), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+}
+template <bool PAIR>
+__device__ __forceinline__ void tmem_dealloc512(uint32_t tmem) {
+    if constexpr (PAIR)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    else
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
 // The end of an issuing warp after a failure, away from its loops: gives this
-// CTA's copies and MMAs in flight `limit` cycles to land, meets the other warps at
-// the kernel's last barrier, frees the tensor memory if asked to and exits.
+// CTA's copies and MMAs in flight `limit` cycles to land, meets the other warps of
+// the CTA group at the kernel's last barrier, frees the tensor memory if asked to
+// and exits.
+template <bool PAIR>
 __device__ __noinline__ __attribute__((noreturn)) inline void issue_unwind(uint32_t tmem, bool dealloc, long long limit) {
     const long long t0 = clock64();
     while (clock64() - t0 < limit) {
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    asm volatile("barrier.sync 0;" ::: "memory");
+    group_sync<PAIR>();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (dealloc)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    if (dealloc) tmem_dealloc512<PAIR>(tmem);
     asm volatile("exit;");
     __builtin_unreachable();
 }
 constexpr long long kUnwindCycles = 20000000LL;        // about 10 ms: far beyond any copy or MMA of a CTA
 // A converged warp's bounded wait without a result: a failure leaves through
 // issue_unwind, so the caller's loops keep uniform trip counts (and their
-// counters, addresses and descriptors uniform registers).
+// counters, addresses and descriptors uniform registers). In a pair the barrier
+// may be reached from both CTAs.
+template <bool PAIR>
 __device__ __forceinline__ void mbar_wait_issue(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *err,
                                                 uint32_t tmem, bool dealloc) {
-    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return;
+    auto done = [&]() { return PAIR ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
+    if (__all_sync(0xffffffffu, done())) return;
     const long long t0 = clock64();
     for (uint32_t spin = 1;; ++spin) {
-        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return;
+        if (__all_sync(0xffffffffu, done())) return;
         if ((spin & 63) == 0) {
             const bool other = *abort_flag != 0 || *reinterpret_cast<volatile int *>(err) != 0;
             const bool late = clock64() - t0 > kWaitLimitCycles;
             if (__any_sync(0xffffffffu, other || late)) {
                 *abort_flag = 1;
                 if (__all_sync(0xffffffffu, !other)) atomicExch(err, kErrWaitTimeout);
-                issue_unwind(tmem, dealloc, kUnwindCycles);
+                issue_unwind<PAIR>(tmem, dealloc, kUnwindCycles);
             }
         }
     }
+}
+// The pair's copies: the bytes count on the leader's barrier (cluster address).
+__device__ __forceinline__ void tma_load_2d_pair_if(uint32_t pr, uint32_t dst, const CUtensorMap *tm, uint32_t leader_bar, int x,
+                                                    int y) {
+    asm volatile(
+        "{\n .reg .pred q;\n setp.ne.b32 q, %5, 0;\n"
+        " @q cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n}\n" ::"r"(dst),
+        "l"(tm), "r"(leader_bar), "r"(x), "r"(y), "r"(pr)
+        : "memory");
 }
 
 // One lane of a converged warp.
@@ -187,9 +251,9 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
     return d;
 }
 
-// Instruction descriptor, kind::f16: D = f32, A = B = f16, both K-major, M = 128.
-__device__ __forceinline__ uint32_t idesc_f16(int n) {
-    return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
+// Instruction descriptor, kind::f16: D = f32, A = B = f16, both K-major, M = 128 (256 for a CTA pair).
+__device__ __forceinline__ uint32_t idesc_f16(int n, int m = kTileM) {
+    return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
 // D (+)= A * B^T with the A operand in TMEM (lane = row, two fp16 per 32-bit
@@ -209,20 +273,38 @@ __device__ __forceinline__ void umma_f16_ss(uint32_t d_tmem, uint64_t a, uint64_
         "l"(a), "l"(b), "r"(idesc), "r"(acc)
         : "memory");
 }
-// The same, predicated, with the descriptors as 32-bit halves: only the low words
-// (start addresses) change between instructions.
+// Both operands in shared memory, for a CTA or a pair (M = 256: 128 rows in each
+// CTA, N / 2 columns of B in each), predicated, with the descriptors as 32-bit
+// halves: only the low words (start addresses) change between instructions.
+template <bool PAIR>
 __device__ __forceinline__ void umma_f16_ss_if(uint32_t pr, uint32_t d_tmem, uint32_t alo, uint32_t ahi, uint32_t blo,
-                                               uint32_t bhi, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n .reg .pred p, q;\n .reg .b64 da, db;\n mov.b64 da, {%1, %2};\n mov.b64 db, {%3, %4};\n setp.ne.b32 p, %6, 0;\n"
-        " setp.ne.b32 q, %7, 0;\n @q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n" ::"r"(d_tmem),
-        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc), "r"(pr)
-        : "memory");
+                                                    uint32_t bhi, uint32_t idesc, uint32_t acc) {
+    if constexpr (PAIR)
+        asm volatile(
+            "{\n .reg .pred p, q;\n .reg .b64 da, db;\n mov.b64 da, {%1, %2};\n mov.b64 db, {%3, %4};\n setp.ne.b32 p, %6, 0;\n"
+            " setp.ne.b32 q, %7, 0;\n @q tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p;\n}\n" ::"r"(d_tmem),
+            "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc), "r"(pr)
+            : "memory");
+    else
+        asm volatile(
+            "{\n .reg .pred p, q;\n .reg .b64 da, db;\n mov.b64 da, {%1, %2};\n mov.b64 db, {%3, %4};\n setp.ne.b32 p, %6, 0;\n"
+            " setp.ne.b32 q, %7, 0;\n @q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n" ::"r"(d_tmem),
+            "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc), "r"(pr)
+            : "memory");
 }
+// one arrival on the barrier (at this offset in both CTAs of a pair)
+template <bool PAIR>
 __device__ __forceinline__ void umma_commit_if(uint32_t pr, uint32_t bar) {
-    asm volatile(
-        "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
-        " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+    if constexpr (!PAIR)
+        asm volatile(
+            "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+            " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+            "r"(pr)
+            : "memory");
+    else
+        asm volatile(
+        "{\n .reg .pred q;\n .reg .b16 m;\n setp.ne.b32 q, %1, 0;\n mov.b16 m, 3;\n"
+        " @q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], m;\n}\n" ::"r"(bar),
         "r"(pr)
         : "memory");
 }

@@ -85,3 +85,13 @@ def test_general_transition(H, c_out, form, hb_next, act):
     ref = O.conv_layer(x, p)
     assert np.array_equal(y.cpu().numpy(), ref)
     assert len(np.unique(ref)) > 20
+
+
+@pytest.mark.parametrize("n,h,w", [(1, 9, 7), (1, 16, 24), (3, 16, 8), (5, 33, 17)])
+@pytest.mark.parametrize("c_out,hb_next", [(192, 64), (128, 128), (32, 0)])
+def test_pairs_with_odd_tiles(H, n, h, w, c_out, hb_next):
+    """45 weight blocks (CTA pairs), with one M tile and other odd numbers of them: the last pair's
+    second tile lies past the last image. Small codes, so that one chunk holds the reduction, and
+    uniform ones, so that it takes two."""
+    case(H, 320, c_out, 3, 1, hb_next, n, h, w, lim=40)
+    case(H, 320, c_out, 3, 1, hb_next, n, h, w, chunks=2)

@@ -1687,8 +1687,6 @@ hatq_status hatq_gdn(const int8_t *z, int n, int h, int w, const hatq_prepared_g
         (e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
         return cuda_fail(e, "device query");
     hatq::GdnArgs a{};
-    a.z = z;
-    a.y = y;
     a.pixels = pixels;
     a.c = c;
     a.inverse = g->inverse;
@@ -1696,30 +1694,31 @@ hatq_status hatq_gdn(const int8_t *z, int n, int h, int w, const hatq_prepared_g
     a.t = g->t;
     a.shift_in = g->shift_in;
     a.P = (unsigned long long)g->P;
-    a.sr = (float)std::sqrt(std::ldexp((double)g->P, -g->t));
+    a.factor = g->inverse ? std::ldexp((double)g->P, -g->t) : std::ldexp(1.0, g->t) / (double)g->P;
+    a.k256 = (float)(256.0 * a.factor);
     a.mult_in = g->mult_in;
     a.b_pool = g->b_pool;
     a.err = err_word();
     if (!a.err) return fail(HATQ_ERR_CUDA, "no CUDA device");
     a.num_tiles = (int)((pixels + 127) / 128);
-    // shared memory: G, nz z tiles, the u rows, B, barriers (plus the 1024-byte alignment slack)
-    const int g_bytes = c * c * 2, z_bytes = 128 * c, u_bytes = 128 * (c + 16);
+    // shared memory: G, nz z tiles, the pool warps' output rows (2 KB each), B, table, barriers
+    // (plus the 1024-byte alignment slack); as many z tiles ahead as fit
+    const int g_bytes = c * c * 2, z_bytes = 128 * c;
     auto layout = [&](int nz) {
         a.nz = nz;
         a.z_off = g_bytes;
         a.u_off = a.z_off + nz * z_bytes;
-        a.b_off = (a.u_off + u_bytes + 127) & ~127;
-        a.lut_off = a.b_off + 8 * c;
+        a.b_off = a.u_off + 12 * 2048;
+        a.lut_off = a.b_off + 4 * c;
         a.bar_off = (a.lut_off + 255 * (g->hb_next > 1 ? g->hb_next : 1) + 1 + 63) & ~63;
-        return a.bar_off + 64 + 1024;
+        return a.bar_off + 192 + 1024;
     };
-    int smem = layout(2);
-    if (smem > smem_max) smem = layout(1);
-    if (smem > smem_max) return fail(HATQ_ERR_UNSUPPORTED, "the GDN tile does not fit shared memory");
-    a.tmem_cols = 512;                   // A limbs (c columns) and two 128-column accumulator buffers
+    int smem = 0, nz = 4;
+    while (nz > 0 && (smem = layout(nz)) > smem_max - 1024 /* static */) --nz;
+    if (!nz) return fail(HATQ_ERR_UNSUPPORTED, "the GDN tile does not fit shared memory");
     EncodeTiledFn enc = encode_fn();
     if (!enc) return fail(HATQ_ERR_CUDA, "cuTensorMapEncodeTiled is unavailable");
-    CUtensorMap tmZ, tmG;
+    CUtensorMap tmZ, tmG, tmY;
     std::memcpy(&tmG, g->opaque, sizeof tmG);
     const cuuint64_t dims[2] = {(cuuint64_t)c, (cuuint64_t)pixels};
     const cuuint64_t strides[1] = {(cuuint64_t)c};
@@ -1729,7 +1728,11 @@ hatq_status hatq_gdn(const int8_t *z, int n, int h, int w, const hatq_prepared_g
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(HATQ_ERR_CUDA, "preactivation tensor map encoding failed (%d)", (int)r);
-    if ((e = hatq::launch_gdn(tmZ, tmG, a, smem, reinterpret_cast<cudaStream_t>(stream))) != cudaSuccess)
+    const cuuint32_t ybox[2] = {64, 32};                 // one pool warp's rows of a pass
+    r = enc(&tmY, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, y, dims, strides, ybox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(HATQ_ERR_CUDA, "output tensor map encoding failed (%d)", (int)r);
+    if ((e = hatq::launch_gdn(tmZ, tmG, tmY, a, smem, reinterpret_cast<cudaStream_t>(stream))) != cudaSuccess)
         return cuda_fail(e, "GDN launch");
     return HATQ_OK;
 }

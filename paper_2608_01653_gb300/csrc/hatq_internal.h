@@ -181,21 +181,19 @@ cudaError_t launch_conv_win(const CUtensorMap &tmA, const CUtensorMap &tmB, cons
 
 // GDN / IGDN transition kernel (hatq_gdn.cu).
 struct GdnArgs {
-    const int8_t *z;                 // [pixels][c] preactivation codes (read through the tensor map)
-    int8_t *y;                       // [pixels][c] next-layer codes
-    long long pixels;
+    long long pixels;                // [pixels][c] codes in and out, through the tensor maps
     int c, inverse, hb_next, t, shift_in;
     unsigned long long P;            // R^2 ~ P / 2^t
-    float sr;                        // sqrt(P / 2^t) (estimate only)
+    double factor;                   // 2^t / P, IGDN P / 2^t (estimate only)
+    float k256;                      // 256 factor
     long long mult_in;               // M_in
     const int32_t *b_pool;           // [c] B_i
     int *err;
-    int num_tiles, nz;               // 128-pixel tiles, z tile buffers (1 or 2)
+    int num_tiles, nz;               // 128-pixel tiles, z tile buffers (1 to 4)
     int z_off, u_off, b_off, lut_off, bar_off;  // shared-memory offsets from the 1024-aligned base
-    int tmem_cols;
 };
 
-cudaError_t launch_gdn(const CUtensorMap &tmZ, const CUtensorMap &tmG, const GdnArgs &a, int smem_bytes,
+cudaError_t launch_gdn(const CUtensorMap &tmZ, const CUtensorMap &tmG, const CUtensorMap &tmY, const GdnArgs &a, int smem_bytes,
                        cudaStream_t s);
 
 }  // namespace hatq

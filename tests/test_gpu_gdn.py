@@ -82,6 +82,29 @@ def test_gdn_transition_bit_exact(H, case):
     assert len(np.unique(u)) > 40 and (np.abs(u) == 127).any()
 
 
+@pytest.mark.parametrize("c, inverse, hb_next, pixels", [
+    (64, False, 64, 152 * 128 * 13 + 1),              # one pass a tile, buffers reused, one-pixel tail
+    (128, True, 16, 152 * 128 * 3 + 33),              # tail of one full and one partial 32-row store
+    (192, False, 32, 152 * 128 * 5 - 95),
+    (256, True, 2, 152 * 128 * 4 + 127),              # a single z buffer
+])
+def test_gdn_several_tiles_per_block(H, c, inverse, hb_next, pixels):
+    """More 128-pixel tiles than a device has SMs: every barrier passes
+    through both parities and the three pool groups take tiles and passes in
+    turn. The pixels repeat a base set in random order, so the oracle runs on
+    the base set alone."""
+    beta, gamma = _params(c, 7 * c)
+    base = _codes((1, 1, 1024, c), seed=c + hb_next)
+    pick = np.random.default_rng(c).integers(0, 1024, pixels)
+    s_z, s_y = 0.04, 0.05
+    s_u = float(np.float32(np.abs(O.gdn(s_z * base.astype(np.float64), beta, gamma, inverse)).max() / 135.0))
+    ref, _ = _oracle(base, beta, gamma, s_z, s_u, inverse, s_y, hb_next)
+    G = H.prepare_gdn(c, beta, gamma, s_z, s_u, inverse, s_y, hb_next)
+    y = H.gdn(dev(base.reshape(1024, c)[pick].reshape(1, 1, pixels, c)), G)
+    H.sync_status()
+    assert np.array_equal(y.cpu().numpy().reshape(pixels, c), ref.reshape(1024, c)[pick])
+
+
 def test_gdn_gamma_zero_and_all_saturated(H):
     """gamma = 0 (the pool is B alone) and an activation scale so small that
     every nonzero code saturates."""

@@ -954,8 +954,10 @@ int win_plan(const hatq_conv_desc &d, const Geometry &g, const hatq_prepared &L,
     a.b_bytes = (a.pair ? g.n_t / 2 : g.n_t) * 128;  // this CTA's columns
     a.w8_bytes = (a.rows * 64 + 1023) & ~1023;
     a.w16_bytes = (a.rows * 128 + 1023) & ~1023;
-    const int const_bytes = (12 * d.c_out + (general ? 256 : 0) + 127) & ~127, bars = 8 * 32 + 16;
-    const int budget = 227 * 1024 - 1024 /* static */ - 1024 /* alignment */ - 8 * 4096 - 512 - const_bytes - 2 * a.w16_bytes;
+    // per epilogue warp two 32-row buffers of 64 columns and two rows for the exact codes
+    const int stg_bytes = 8 * (4096 + 512);
+    const int const_bytes = (16 * d.c_out + (general ? 256 : 0) + 127) & ~127, bars = 8 * 32 + 16;
+    const int budget = 227 * 1024 - 1024 /* static */ - 1024 /* alignment */ - stg_bytes - 512 - const_bytes - 2 * a.w16_bytes;
     // A weight stage holds the taps of one kernel row (a wait, a commit and the counters per row
     // instead of per tap) where at least six blocks fit in two stages or more, preferably beside two
     // INT8 window buffers; else single blocks, with the second window buffer where four stages remain.
@@ -979,7 +981,7 @@ int win_plan(const hatq_conv_desc &d, const Geometry &g, const hatq_prepared &L,
     a.w16_off = a.stages * a.seg * a.b_bytes;
     a.w8_off = a.w16_off + 2 * a.w16_bytes;
     a.stg_off = a.w8_off + a.n8 * a.w8_bytes;
-    a.bar_off = a.stg_off + 8 * 4096;
+    a.bar_off = a.stg_off + stg_bytes;
     a.const_off = (bars + 127) & ~127;
     a.b_int = L.b_int;
     a.mult = L.mult;
@@ -1101,7 +1103,7 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     const int esz = L->out_f32 ? 4 : 1;
     a.row_stride = a.n_t * esz + 16;                 // padded rows: 8 consecutive rows hit 8 bank groups
     a.staging_bytes = L->out_f32 ? 0 : a.nbuf * kTileRows * a.row_stride;   // float32 output is stored directly
-    if (a.lean) a.staging_bytes = 8 * 4096;          // two 32-row buffers of 64 columns per epilogue warp
+    if (a.lean) a.staging_bytes = 8 * (4096 + 512);  // per epilogue warp two 32-row buffers of 64 columns and two exact rows
     a.win_h = (a.th - 1) * d->stride + d->kh;
     a.win_w = (a.tw - 1) * d->stride + d->kw;
     a.win_pitch = a.win_tma ? window_box_bytes(a.tw, d->stride, d->kw, d->c_in) : (a.win_w * d->c_in + 15) & ~15;

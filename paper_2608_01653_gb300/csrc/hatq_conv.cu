@@ -370,8 +370,9 @@ __device__ __forceinline__ void epi_split128(const EpiCtx &e, const ConvArgs &a,
 // (groups of 128 columns with the warp of the same rows in the other
 // warpgroup): the region is released as soon as the last columns arrived, and the
 // codes leave as one TMA store per warp and group from a swizzled staging buffer.
-// Bound: integer issue (38 integer operations per value of a WH(64) -> ReLU ->
-// DH(64) transition, the 64-bit adds on the integer pipe).
+// Bound: instruction issue. Groups of 32 and 64 columns take the fp32 estimate with exact
+// rows where it is not certain (12 operations per value of a WH(64) -> ReLU -> DH(64)
+// transition, 38 in 64-bit integers), groups of 128 the integers.
 // (The pieces are in hatq_lean.h.)
 
 // ------------------------------------------------------------------ kernel
@@ -455,12 +456,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     // bias codes, multipliers and dequant factors of all output channels,
     // staged once per CTA (128-byte aligned, read with 16-byte vector loads);
-    // the lean epilogue takes the bias products M b (64 bits) and the multipliers
+    // the lean epilogues take the bias products M b (64 bits) and the multipliers, or for
+    // their fp32 estimate multipliers and bias products times 2^-n
     int *cb = reinterpret_cast<int *>(bar_area + a.const_off);
     long long *mbs = reinterpret_cast<long long *>(bar_area + a.const_off);
     int *mults = reinterpret_cast<int *>(mbs + a.co);
     int8_t *lut_s = reinterpret_cast<int8_t *>(bar_area + a.lut_off);
-    if constexpr (LEAN != 0) {
+    if constexpr (LEAN == 32 || LEAN == 64) {
+        stage_quick(reinterpret_cast<float *>(cb), a.mult, a.b_int, a.co, a.shift);
+    } else if constexpr (LEAN != 0) {
         for (int c = threadIdx.x; c < a.co; c += kThreads) {
             const int m = a.mult[c];
             mbs[c] = (long long)m * a.b_int[c];
@@ -880,6 +884,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int quad = warp & 3;                 // TMEM lane quadrant this warp may access
         const uint32_t t_lane = tmem + ((uint32_t)(quad * 32) << 16);
         uint8_t *wstage = staging + (warp - 4) * kWarpStage;
+        [[maybe_unused]] uint8_t *scratch = staging + 8 * kWarpStage + (warp - 4) * kWarpScratch;
+        [[maybe_unused]] const Quick opt = quick_setup<LEAN>(a.hb_out, a.hb_next, a.act, a.shift);
         const int row0 = quad * 32;                // first tile row of this warp; its 32 rows are one output box
         const int box_y = row0 >> a.tw_log2, box_x = row0 & (a.tw - 1);
         bool ok = true;
@@ -898,22 +904,21 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!ok) break;
 #pragma unroll 1
                 for (int col = 0; col < a.n_t; col += LEAN) {
-                    uint32_t w[LEAN / 4];
-                    long long t[LEAN];
-                    {
-                        uint32_t r[LEAN];
+                    uint32_t w[LEAN / 4], r[LEAN];
 #pragma unroll
-                        for (int q = 0; q < LEAN / 32; ++q)
-                            tmem_ld32(t_acc + col + 32 * q, reinterpret_cast<uint32_t(&)[32]>(r[32 * q]));
-                        tmem_wait_ld();
-                        if (col + LEAN >= a.n_t) {       // TMEM reads of this region are complete
-                            tc_fence_before();
-                            mbar_arrive(acc_empty(reg));
-                        }
-                        lean_scale<LEAN>(r, mbs + n0 + col, mults + n0 + col, t);
+                    for (int q = 0; q < LEAN / 32; ++q)
+                        tmem_ld32(t_acc + col + 32 * q, reinterpret_cast<uint32_t(&)[32]>(r[32 * q]));
+                    tmem_wait_ld();
+                    if (col + LEAN >= a.n_t) {           // TMEM reads of this region are complete
+                        tc_fence_before();
+                        mbar_arrive(acc_empty(reg));
                     }
-                    whole_transition<LEAN>(t, a.hb_out, a.hb_next, a.act);
-                    lean_codes<LEAN>(a.shift, t, w);
+                    const float *ms = reinterpret_cast<const float *>(cb) + n0 + col;
+                    const bool sure = quick_codes<LEAN>(r, ms, ms + a.co, opt, lane, w);
+                    const uint32_t rows = __ballot_sync(0xffffffffu, !sure);
+                    if (rows)
+                        exact_rows<LEAN>(rows, r, reinterpret_cast<const int *>(ms) + 2 * a.co,
+                                         reinterpret_cast<const int *>(ms) + 3 * a.co, opt, scratch, lane, w);
                     lean_store<LEAN>(wstage + buf * (kWarpStage / 2), w, &tmY, lane, inside, n0 + col, ox, oy, img);
                     buf ^= 1;
                 }

@@ -69,6 +69,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr bool kSplit = EPI / 1000 == 1 || EPI / 1000 == 2, kDrain = EPI == 2064, kTwo = EPI == 2128;
     static_assert(EPI == 32 || EPI == 64 || EPI == 1128 || kDrain || kTwo || EPI == 3064 || EPI / 1000 == 4, "epilogue");
     constexpr bool kD2s = EPI / 1000 == 3, kGeneral = EPI / 1000 == 4;
+    constexpr bool kQuick = !kSplit && !kGeneral;                     // fp32 estimate, exact rows where it is not certain
     constexpr int G = EPI % 1000;
     constexpr int kRegions = kTwo ? 4 : 2, kRegLog = kTwo ? 2 : 1;   // accumulator regions of n_t columns
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -114,13 +115,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 1) {
         tmem_alloc512<PAIR>(smem_addr(tmem_holder));
     }
-    // bias products M b (64 bits) and multipliers of all output channels
+    // bias products M b (64 bits) and multipliers of all output channels, or for the fp32
+    // estimate multipliers and bias products times 2^-n
     long long *mbs = reinterpret_cast<long long *>(bar_area + a.const_off);
     int *mults = reinterpret_cast<int *>(mbs + a.co);
-    for (int c = threadIdx.x; c < a.co; c += kThreads) {
-        const int m = a.mult[c];
-        mbs[c] = (long long)m * a.b_int[c];
-        mults[c] = m;
+    float *quick = reinterpret_cast<float *>(bar_area + a.const_off);
+    if constexpr (kQuick) {
+        stage_quick(quick, a.mult, a.b_int, a.co, a.shift);
+    } else {
+        for (int c = threadIdx.x; c < a.co; c += kThreads) {
+            const int m = a.mult[c];
+            mbs[c] = (long long)m * a.b_int[c];
+            mults[c] = m;
+        }
     }
     int8_t *lut_s = reinterpret_cast<int8_t *>(mults + a.co);
     if constexpr (kGeneral)
@@ -372,6 +379,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint8_t *wstage = staging + (warp - 4) * kWarpStage;
         bool ok = true;
         int buf = 0;
+        [[maybe_unused]] const Quick opt = quick_setup<G>(a.hb_out, a.hb_next, a.act, a.shift);
         // this warp's tensor-memory reads of a region are done (fenced by every lane)
         auto release = [&](int r) {
             __syncwarp();
@@ -394,22 +402,20 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!ok) break;
 #pragma unroll 1
                 for (int col = 0; col < a.n_t; col += G) {
-                    long long t[G];
+                    uint32_t r[G], w[G / 4];
 #pragma unroll
-                    for (int q = 0; q < G / 32; ++q) {
-                        uint32_t r[32];
-                        tmem_ld32(t_acc + col + 32 * q, r);
-                        tmem_wait_ld();
-                        if (q == G / 32 - 1 && col + G >= a.n_t) {         // TMEM reads of this region are complete
-                            tc_fence_before();
-                            release(reg);
-                        }
-                        lean_scale<32>(r, mbs + n0 + col + 32 * q, mults + n0 + col + 32 * q, t + 32 * q);
+                    for (int q = 0; q < G / 32; ++q)
+                        tmem_ld32(t_acc + col + 32 * q, reinterpret_cast<uint32_t(&)[32]>(r[32 * q]));
+                    tmem_wait_ld();
+                    if (col + G >= a.n_t) {                                // TMEM reads of this region are complete
+                        tc_fence_before();
+                        release(reg);
                     }
-                    uint32_t w[G / 4];
                     if constexpr (kGeneral) {
                         // z = clamp(round(H~_out (M_out (.) a) / 2^n_out)), u = phi_int(z), then the next
                         // layer's transform on u itself (|H~ u| <= 127 * 64) and its requantization
+                        long long t[G];
+                        lean_scale<G>(r, mbs + n0 + col, mults + n0 + col, t);
                         if (a.hb_out) fwht_stages<G>(t, a.hb_out);
                         int u[G];
 #pragma unroll
@@ -423,8 +429,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                             w[i] = pack4(q[0], q[1], q[2], q[3]);
                         }
                     } else {
-                        whole_transition<G>(t, a.hb_out, a.hb_next, a.act);
-                        lean_codes<G>(a.shift, t, w);
+                        const float *ms = quick + n0 + col;
+                        const bool sure = quick_codes<G>(r, ms, ms + a.co, opt, lane, w);
+                        const uint32_t rows = __ballot_sync(0xffffffffu, !sure);
+                        if (rows)
+                            exact_rows<G>(rows, r, reinterpret_cast<const int *>(ms) + 2 * a.co,
+                                          reinterpret_cast<const int *>(ms) + 3 * a.co, opt,
+                                          staging + 8 * kWarpStage + (warp - 4) * kWarpScratch, lane, w);
                     }
                     if constexpr (kD2s) {
                         // channel 4 cd + 2 i + j of this lane's pixel -> channel cd of pixel (2 oy + i, 2 ox + j):

@@ -103,7 +103,7 @@ __device__ __forceinline__ void umma_f16_ts_if(uint32_t pr, uint32_t d_tmem, uin
         "r"(a_tmem), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc), "r"(pr)
         : "memory");
 }
-__device__ __forceinline__ int lds_u8(int addr) {
+__device__ __forceinline__ int lds_u8(uint32_t addr) {
     uint32_t r;
     asm("ld.shared.u8 %0, [%1];" : "=r"(r) : "r"(addr));
     return (int)r;
@@ -120,7 +120,7 @@ __device__ __forceinline__ void tma_store_2d(uint32_t src, const CUtensorMap *tm
 // 5 x 2^-24 (k256 3, two fmas 2), half of that after the square root; with rsqrt.approx
 // (2^-22.9) and at most two products X is off by less than 127.5 x 4.0e-7 < 2^-14: it decides
 // every code whose |X| lies more than 2^-14 from a half-integer.
-constexpr int kCodeBias = 0x4B400000;           // bits of 1.5 2^23
+constexpr uint32_t kCodeBias = 0x4B400000u;           // bits of 1.5 2^23
 constexpr float kSure = 0.5f - 0.00006103515625f;
 template <bool INV>
 __device__ __forceinline__ float gdn_estimate(float zf, uint32_t dh, uint32_t dl, float bf, float k256) {
@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(kGdnThreads, 1)
             const uint32_t t_acc = t_lane + (uint32_t)(c + 128 * db);
             // Codes as the bits of 1.5 2^23 + u; the bias leaves in the first butterflies. An estimate
             // too close to a rounding boundary sets its bit of `unsure`.
-            int v[64];
+            uint32_t v[64];
             uint32_t unsure[2] = {0u, 0u};
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kGdnThreads, 1)
                         const float x = gdn_estimate<INV>(zf, dh[4 * i + k], dl[4 * i + k], b[k], a.k256);
                         const float t = x + 12582912.0f;
                         if (fabsf(x - (t - 12582912.0f)) >= kSure) unsure[e >> 5] |= 1u << (e & 31);
-                        v[e] = __float_as_int(t);
+                        v[e] = __float_as_uint(t);
                     }
                 }
             }
@@ -344,14 +344,14 @@ __global__ void __launch_bounds__(kGdnThreads, 1)
                 tmem_ld1(t_acc + (uint32_t)e, dh);
                 tmem_ld1(t_acc + 64 + (uint32_t)e, dl);
                 tmem_wait_ld();
-                int k = 0;
+                uint32_t k = 0;
                 if (mine) {
                     const int zi = reinterpret_cast<const int8_t *>(zt)[(((e >> 4) ^ sw) << 4) + (e & 15)];
                     const float x = gdn_estimate<INV>((float)zi, dh, dl, bf_s[64 * p + e], a.k256);
                     const uint32_t D = (uint32_t)__float2int_rn(__uint_as_float(dh) * 2.0f) * 128u +
                                        (uint32_t)__float2int_rn(__uint_as_float(dl) * 256.0f) + (uint32_t)a.b_pool[64 * p + e];
-                    k = gdn_code_exact((uint32_t)abs(zi), D, (int)(fabsf(x) + 0.5f), a);
-                    k = (zi < 0 ? -k : k) + kCodeBias;
+                    const int u8 = gdn_code_exact((uint32_t)abs(zi), D, (int)(fabsf(x) + 0.5f), a);
+                    k = (uint32_t)(zi < 0 ? -u8 : u8) + kCodeBias;
                 }
                 const uint32_t bit = mine ? 1u << (e & 31) : 0u, b0 = e < 32 ? bit : 0u, b1 = e < 32 ? 0u : bit;
 #pragma unroll
@@ -363,28 +363,38 @@ __global__ void __launch_bounds__(kGdnThreads, 1)
             if (lane == 0) mbar_arrive(z_empty(zb));
             // v - bias of the first butterflies, exact (|H~ u| <= 127 hb), plus the table's address: added to
             // a full block's first value it reaches every sum, as the block's first column is all ones
-            if (a.hb_next > 1) {
-                if (a.hb_next == 64) v[0] += (int)lut;
+            auto first = [&]() {
 #pragma unroll
                 for (int i = 0; i < 64; i += 2) {
-                    const int s0 = v[i], s1 = v[i + 1];
-                    v[i] = s0 + s1 - 2 * kCodeBias;
+                    const uint32_t s0 = v[i], s1 = v[i + 1];
+                    v[i] = s0 + s1 - 2u * kCodeBias;
                     v[i + 1] = s0 - s1;
                 }
+            };
+            auto butterflies = [&](int m2) {
 #pragma unroll
-                for (int m2 = 2; m2 < 64; m2 <<= 1) {
-                    if (m2 >= a.hb_next) break;
+                for (int i = 0; i < 64; ++i)
+                    if (!(i & m2)) {
+                        const uint32_t s0 = v[i], s1 = v[i | m2];
+                        v[i] = s0 + s1;
+                        v[i | m2] = s0 - s1;
+                    }
+            };
+            if (a.hb_next == 64) {                                 // straight through: a stage that may be the last costs moves
+                v[0] += lut;
+                first();
 #pragma unroll
-                    for (int i = 0; i < 64; ++i)
-                        if (!(i & m2)) {
-                            const int s0 = v[i], s1 = v[i | m2];
-                            v[i] = s0 + s1;
-                            v[i | m2] = s0 - s1;
-                        }
+                for (int m2 = 2; m2 < 64; m2 <<= 1) butterflies(m2);
+            } else {
+                if (a.hb_next > 1) {
+                    first();
+#pragma unroll
+                    for (int m2 = 2; m2 < 32; m2 <<= 1) {
+                        if (m2 >= a.hb_next) break;
+                        butterflies(m2);
+                    }
                 }
-            }
-            if (a.hb_next != 64) {
-                const int base = (int)lut - (a.hb_next > 1 ? 0 : kCodeBias);
+                const uint32_t base = lut - (a.hb_next > 1 ? 0u : kCodeBias);
 #pragma unroll
                 for (int i = 0; i < 64; ++i) v[i] += base;
             }

@@ -96,22 +96,242 @@ __device__ __forceinline__ void lean_store(uint8_t *buf, const uint32_t (&w)[G /
 
 // ------------------------------------------------------------------ transitions
 //
-// Code size: 64 values per thread with each transform written out are 46 KB of
-// straight-line code. Beyond about 32 KB the instruction cache misses: a warp
-// then issues every 3.1 cycles instead of every 1.1 (measured on the 64-point
-// transform alone), and the short loops of the other roles are evicted all the
-// time. So both transforms of a transition are one copy of code in a loop of two
-// passes, and loops over groups stay rolled.
+// Code size: beyond about 32 KB of straight-line code the instruction cache misses: a
+// warp then issues every 3.1 cycles instead of every 1.1 (measured on the 64-point
+// transform alone), and the short loops of the other roles are evicted all the time.
+// 64 int64 values per thread with both transforms written out are 46 KB. So groups
+// that one thread holds whole take the fp32 estimate below, and shared groups run both
+// transforms as one copy of code in a loop of two passes.
 
-// H~_out, phi, H~_next of G columns held by one thread.
+// Pairs of floats, one instruction for both.
+__device__ __forceinline__ uint64_t f2_pack(float x, float y) {
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+    return d;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t v, float &x, float &y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v)); }
+__device__ __forceinline__ uint64_t f2_add(uint64_t x, uint64_t y) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(x), "l"(y));
+    return d;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t x, uint64_t y, uint64_t z) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(x), "l"(y), "l"(z));
+    return d;
+}
+
+// Unnormalized Sylvester transform of every hb-block of G floats (pairs of neighbours).
+// Whole groups (the usual case) run straight through: where a stage may be the last,
+// every value has to be moved to the register that the others leave it in.
 template <int G>
-__device__ __forceinline__ void whole_transition(long long (&t)[G], int hb_out, int hb_next, int act) {
-    if (hb_out) fwht_stages<G>(t, hb_out);
-    if (act) {
+__device__ __forceinline__ void f2_fwht(uint64_t (&p)[G / 2], int hb) {
+    const uint64_t neg = f2_pack(-1.0f, -1.0f);
+    auto first = [&]() {
 #pragma unroll
-        for (int i = 0; i < G; ++i) t[i] = relu_mad(t[i]);
+        for (int i = 0; i < G / 2; ++i) {
+            float x, y;
+            f2_unpack(p[i], x, y);
+            p[i] = f2_pack(x + y, x - y);
+        }
+    };
+    auto stage = [&](int h) {
+#pragma unroll
+        for (int i = 0; i < G / 2; ++i)
+            if (!(i & h)) {
+                const uint64_t x = p[i], y = p[i + h];
+                p[i] = f2_add(x, y);
+                p[i + h] = f2_fma(y, neg, x);
+            }
+    };
+    if (hb == G) {
+        first();
+#pragma unroll
+        for (int h = 1; h < G / 2; h <<= 1) stage(h);
+    } else if (hb > 1) {
+        first();
+#pragma unroll
+        for (int h = 1; h < G / 4; h <<= 1) {
+            if (2 * h >= hb) break;
+            stage(h);
+        }
     }
-    if (hb_next) fwht_stages<G>(t, hb_next);
+}
+
+// Constants of the estimate in shared memory, 16 bytes a channel: multipliers and bias
+// products times 2^-n in fp32, each rounded once, then multipliers and bias codes.
+__device__ __forceinline__ void stage_quick(float *s, const int32_t *mult, const int32_t *b_int, int co, int shift) {
+    const float sc = __int_as_float((127 - max(shift, 0)) << 23);
+    for (int c = threadIdx.x; c < co; c += blockDim.x) {
+        const int m = mult[c], b = b_int[c];
+        s[c] = (float)m * sc;
+        s[co + c] = (float)((long long)m * b) * sc;
+        reinterpret_cast<int *>(s)[2 * co + c] = m;
+        reinterpret_cast<int *>(s)[3 * co + c] = b;
+    }
+}
+
+// The transition's options and the factors of the estimate's error bound (quick_codes).
+struct Quick {
+    int hb_out, hb_next, act, shift;
+    float kf, kb, kz;
+};
+template <int G>
+__device__ __forceinline__ Quick quick_setup(int hb_out, int hb_next, int act, int shift) {
+    const int h1 = hb_out > 1 ? hb_out : 1, h2 = hb_next > 1 ? hb_next : 1;
+    const float u = 1.02f / 16777216.0f, g = sqrtf((float)h1 * (float)h2) * u;
+    const float l1 = (float)(31 - __clz(h1)), l2 = (float)(31 - __clz(h2));
+    const bool dc = act && hb_next == G;                     // the first output is the sum of phi's values
+    return Quick{hb_out, hb_next, act, shift, g * (2.0f + l1 + (dc ? 0.0f : l2)), g * 2.0f, dc ? u * l2 : 0.0f};
+}
+
+// Codes of one row's G columns, a[] the exact sums: t = M a + M b, H~_out, phi, H~_next
+// and round(t / 2^n), estimated in fp32 with every factor already times 2^-n. Returns
+// whether each code is certain. u = 2^-24:
+//   Factor, bias and multiply-add are each rounded, so a value f with bias term b is off by
+//   at most 2u (|f| + |b|), the row by 2u (F + B) in norm (F, B the norms of f and b).
+//   A stage of a transform of size h rounds its sums, u of their norm; the transform
+//   scales a vector's norm by sqrt(h), phi never lengthens a difference, and one output
+//   of the last transform is at most sqrt(h) times the norm of its input: an output is off
+//   by at most sqrt(h_out h_next) u (2 (F + B) + (log2 h_out + log2 h_next) F). After a
+//   ReLU the last transform's own rounding is at most u log2 h_next times the sum of its
+//   inputs, which is its first output.
+// A value farther than that from every half-integer has the exact value's rounding; the
+// others take exact_rows (one row in a hundred of a 5x5 3 -> 192 layer with a 64-wide
+// output and input transform). That layer on 8 x 2160 x 3840: 4256 us, of 6480 with 64
+// int64 values per thread; with a loop exit after each butterfly stage 5811 (20
+// instructions on the multiply-add pipe per value instead of 12, mostly moves), with
+// both transforms written out as well 7156 (instruction cache).
+template <int G>
+__device__ __forceinline__ bool quick_codes(const uint32_t (&a)[G], const float *ms, const float *bs, const Quick &o, int lane,
+                                            uint32_t (&w)[G / 4]) {
+    uint64_t p[G / 2], n0 = 0, n1 = 0;
+#pragma unroll
+    for (int i = 0; i < G; i += 4) {
+        const float4 m = *reinterpret_cast<const float4 *>(ms + i), b = *reinterpret_cast<const float4 *>(bs + i);
+        p[i / 2] = f2_fma(f2_pack(__uint_as_float(a[i]), __uint_as_float(a[i + 1])), f2_pack(m.x, m.y), f2_pack(b.x, b.y));
+        p[i / 2 + 1] = f2_fma(f2_pack(__uint_as_float(a[i + 2]), __uint_as_float(a[i + 3])), f2_pack(m.z, m.w), f2_pack(b.z, b.w));
+        n0 = f2_fma(p[i / 2], p[i / 2], n0);
+        n1 = f2_fma(p[i / 2 + 1], p[i / 2 + 1], n1);
+    }
+    float x, y, bb = bs[lane] * bs[lane];
+    if (G == 64) bb = fmaf(bs[lane + 32], bs[lane + 32], bb);
+#pragma unroll
+    for (int d = 16; d; d >>= 1) bb += __shfl_xor_sync(0xffffffffu, bb, d);
+    f2_unpack(f2_add(n0, n1), x, y);
+    float sure = 0.4999998f - fmaf(o.kf, sqrtf(x + y), o.kb * sqrtf(bb));
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+        f2_fwht<G>(p, pass ? o.hb_next : o.hb_out);
+        if (!pass && o.act) {
+#pragma unroll
+            for (int i = 0; i < G / 2; ++i) {
+                f2_unpack(p[i], x, y);
+                p[i] = f2_pack(fmaxf(x, 0.f), fmaxf(y, 0.f));
+            }
+        }
+    }
+    f2_unpack(p[0], x, y);
+    sure = fmaf(-o.kz, x, sure);
+    const uint64_t bias = f2_pack(12582912.0f, 12582912.0f), back = f2_pack(-12582912.0f, -12582912.0f),
+                   neg = f2_pack(-1.0f, -1.0f);
+    float worst = 0.f;
+#pragma unroll
+    for (int i = 0; i < G / 4; ++i) {
+        float t[4];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            f2_unpack(p[2 * i + k], x, y);
+            asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(x) : "f"(x), "f"(127.0f));      // sign(x) min(|x|, 127)
+            asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(y) : "f"(y), "f"(127.0f));
+            const uint64_t v = f2_pack(x, y), r = f2_add(v, bias);
+            f2_unpack(r, t[2 * k], t[2 * k + 1]);                                        // low byte: the code
+            f2_unpack(f2_fma(f2_add(r, back), neg, v), x, y);                            // exact
+            asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(worst) : "f"(worst), "f"(x), "f"(y));
+        }
+        w[i] = pack4(__float_as_int(t[0]), __float_as_int(t[1]), __float_as_int(t[2]), __float_as_int(t[3]));
+    }
+    return worst < sure;
+}
+
+constexpr int kWarpScratch = 512;
+
+// round(v / 2^n) half to even, clamped to [-127, 127], in few instructions of code.
+__device__ __forceinline__ int exact_code(long long v, int n) {
+    if (n > 0) v = (v + ((1LL << (n - 1)) - 1) + ((v >> n) & 1)) >> n;
+    return (int)(v > 127 ? 127 : (v < -127 ? -127 : v));
+}
+
+// The codes of the rows (lanes) in `rows`, exactly: the warp takes two rows at a time, half
+// a warp each and C neighbouring columns per lane, in int64 with shuffles. mult / b_int:
+// the group's channels in shared memory.
+template <int G>
+__device__ __forceinline__ void exact_rows(uint32_t rows, const uint32_t (&a)[G], const int *mult, const int *b_int,
+                                           const Quick &o, uint8_t *scratch, int lane, uint32_t (&w)[G / 4]) {
+    constexpr int C = G / 16;
+    const int col = C * (lane & 15);
+    uint8_t *half = scratch + (lane >> 4) * 256;
+    while (rows) {
+        const int r0 = __ffs((int)rows) - 1;
+        rows &= rows - 1u;
+        const int r1 = rows ? __ffs((int)rows) - 1 : r0;
+        rows &= rows - 1u;
+        const bool owner = lane == r0 || lane == r1;
+        uint8_t *own = scratch + (lane == r0 ? 0 : 256);
+        if (owner) {
+#pragma unroll
+            for (int i = 0; i < G; i += 4)
+                *reinterpret_cast<uint4 *>(own + 4 * i) = make_uint4(a[i], a[i + 1], a[i + 2], a[i + 3]);
+        }
+        __syncwarp();
+        long long t[C];
+#pragma unroll
+        for (int k = 0; k < C; ++k)
+            t[k] = (long long)mult[col + k] * (__float2int_rn(reinterpret_cast<const float *>(half)[col + k]) + (long long)b_int[col + k]);
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
+            const int hb = pass ? o.hb_next : o.hb_out;
+#pragma unroll
+            for (int h = 1; h < C; h <<= 1) {
+                if (h >= hb) break;
+#pragma unroll
+                for (int k = 0; k < C; ++k)
+                    if (!(k & h)) {
+                        const long long x = t[k], y = t[k + h];
+                        t[k] = x + y;
+                        t[k + h] = x - y;
+                    }
+            }
+#pragma unroll 1
+            for (int d = 1; d * C < hb; d <<= 1) {
+                const bool upper = (lane & d) != 0;
+#pragma unroll
+                for (int k = 0; k < C; ++k) {
+                    const long long x = __shfl_xor_sync(0xffffffffu, t[k], d);
+                    t[k] = x + (upper ? -t[k] : t[k]);
+                }
+            }
+            if (!pass && o.act) {
+#pragma unroll
+                for (int k = 0; k < C; ++k) t[k] = t[k] > 0 ? t[k] : 0;
+            }
+        }
+        __syncwarp();                                        // the values have been read
+#pragma unroll
+        for (int k = 0; k < C; ++k) half[col + k] = (uint8_t)exact_code(t[k], o.shift);
+        __syncwarp();
+        if (owner) {
+#pragma unroll
+            for (int i = 0; i < G / 16; ++i) {
+                const uint4 v = reinterpret_cast<const uint4 *>(own)[i];
+                w[4 * i] = v.x;
+                w[4 * i + 1] = v.y;
+                w[4 * i + 2] = v.z;
+                w[4 * i + 3] = v.w;
+            }
+        }
+        __syncwarp();                                        // before the next rows' values
+    }
 }
 
 // Groups shared by the two warps of a quadrant, one of each epilogue warpgroup: a

@@ -68,6 +68,26 @@ def test_power_of_two_scales_round_ties_to_even(H, c_out, form, hb_next, act, sh
     assert len(np.unique(ref)) > 3
 
 
+@pytest.mark.parametrize("c_in,k", [(64, 3), (64, 1), (3, 5)])        # window, general and small-channel kernels
+@pytest.mark.parametrize("c_out,hb_next,act", [(64, 64, "none"), (192, 64, "relu"), (32, 32, "none"), (96, 16, "relu")])
+def test_biases_that_leave_every_code_uncertain(H, c_in, k, c_out, hb_next, act):
+    """Biases along one Walsh function, some ten thousand codes in norm: they meet in one output of
+    each block, and the bound of the fp32 estimate, which grows with the norm, sends nearly every
+    row to the exact evaluation."""
+    rng = np.random.default_rng(c_in + c_out + k)
+    form = "WH" if c_in == 3 else "DH"
+    hb = 64 if c_out % 64 == 0 else 32
+    L = C.layer("t", c_in, c_out, k, 1, k // 2, form, act, hb_in=64 if form == "DH" else None, hb_out=hb if form == "WH" else None)
+    w = rng.standard_normal((c_out, k, k, c_in)).astype(np.float32) * 0.05
+    x = rng.integers(-60, 61, size=(2, 19, 23, c_in)).astype(np.int8)
+    s_y = 0.05 * np.sqrt(c_in * k * k) * 35 * 0.02 * 8 / 40
+    sign = 1 - 2 * (np.arange(c_out) & 1)                             # a Walsh function of every block size
+    b = (1500 * 8 * s_y * sign).astype(np.float32)
+    got, ref, P = run_both(H, L, w, b, 0.02, float(np.float32(s_y)), hb_next, x)
+    assert np.array_equal(got, ref)
+    assert len(np.unique(ref)) > 20
+
+
 @pytest.mark.parametrize("h,w", [(1, 1), (1, 129), (5, 31), (17, 33), (130, 3), (16, 64)])
 @pytest.mark.parametrize("c_out,hb_next", [(192, 64), (96, 32), (128, 128)])
 def test_ragged_output_boxes(H, h, w, c_out, hb_next):

@@ -166,8 +166,16 @@ def _stream(stream):
     return ctypes.c_void_p(s.cuda_stream)
 
 
+def _launch_stream(stream):
+    """The stream handle of a call whose tensors have been checked to be CUDA
+    tensors: the device is there, so its presence is not asked for again. (With
+    plain integer handles: 16.4 us a call of a 16x16 layer, 18.3 before.)"""
+    import torch
+    return (stream if stream is not None else torch.cuda.current_stream()).cuda_stream
+
+
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def make_desc(c_in, c_out, k, stride, pad, form, hb_in=0, hb_out=0, kw=None) -> ConvDesc:
@@ -468,10 +476,10 @@ def prepare_weights_transposed(desc: ConvDesc, out_pad, w_ohwi, bias, s_x, s_y, 
 def conv_transpose2d_i8(x, T: PreparedTransposed, y=None, stream=None):
     """hatq_conv_transpose2d_i8 on the INT8 operand x (NHWC)."""
     n, h, w, c = _check_layer_io(x, IN_OPERAND, T, y)
-    torch = _torch()
+    import torch
     if y is None:
         y = torch.empty(T.out_shape(n, h, w), dtype=torch.float32 if T.out_f32 else torch.int8, device=x.device)
-    _check(load().hatq_conv_transpose2d_i8(_ptr(x), n, h, w, ctypes.byref(T.struct), _ptr(y), _stream(stream)))
+    _check(load().hatq_conv_transpose2d_i8(_ptr(x), n, h, w, ctypes.byref(T.struct), _ptr(y), _launch_stream(stream)))
     return y
 
 
@@ -543,11 +551,11 @@ def gdn(z, g: PreparedGdn, y=None, stream=None):
     if y is not None:
         _check_tensor(y, "y", "int8", tuple(z.shape))
     _check_cuda(("z", z), ("y", y))
-    torch = _torch()
+    import torch
     if y is None:
         y = torch.empty_like(z)
     n, h, w, _ = z.shape
-    _check(load().hatq_gdn(_ptr(z), n, h, w, ctypes.byref(g.struct), _ptr(y), _stream(stream)))
+    _check(load().hatq_gdn(_ptr(z), n, h, w, ctypes.byref(g.struct), _ptr(y), _launch_stream(stream)))
     return y
 
 
@@ -559,10 +567,10 @@ def conv2d_i8_subpixel(x, L: "PreparedLayer", r: int, y=None, stream=None):
     shape = (n, ho * r, wo * r, co // (r * r))
     if y is not None:
         _check_tensor(y, "y", "int8", shape)
-    torch = _torch()
+    import torch
     if y is None:
         y = torch.empty(shape, dtype=torch.int8, device=x.device)
-    _check(load().hatq_conv2d_i8_subpixel(_ptr(x), n, h, w, ctypes.byref(L.struct), int(r), _ptr(y), _stream(stream)))
+    _check(load().hatq_conv2d_i8_subpixel(_ptr(x), n, h, w, ctypes.byref(L.struct), int(r), _ptr(y), _launch_stream(stream)))
     return y
 
 
@@ -672,26 +680,26 @@ def conv2d_i8(x, L: PreparedLayer, y=None, stream=None):
     """hatq_conv2d_i8: convolution + fused requantize epilogue on the INT8 operand x (NHWC; fp16 codes
     for a layer with in_f16)."""
     n, h, w, c = _check_layer_io(x, IN_OPERAND, L, y)
-    torch = _torch()
+    import torch
     if y is None:
         y = torch.empty(L.out_shape(n, h, w), dtype=getattr(torch, L.out_dtype), device=x.device)
-    _check(load().hatq_conv2d_i8(_ptr(x), n, h, w, ctypes.byref(L.struct), _ptr(y), _stream(stream)))
+    _check(load().hatq_conv2d_i8(_ptr(x), n, h, w, ctypes.byref(L.struct), _ptr(y), _launch_stream(stream)))
     return y
 
 
 def layer(x, x_kind, s_in, L: PreparedLayer, y=None, scratch=None, stream=None):
     """hatq_layer: input transform/quantize (when needed) + conv in one call."""
     n, h, w, c = _check_layer_io(x, x_kind, L, y, scratch)
-    torch = _torch()
+    import torch
     if y is None:
         y = torch.empty(L.out_shape(n, h, w), dtype=getattr(torch, L.out_dtype), device=x.device)
     nbytes = 0
-    if layer_launches(x_kind, s_in, L) > 1:
+    if x_kind != IN_OPERAND and layer_launches(x_kind, s_in, L) > 1:
         if scratch is None:
             scratch = torch.empty(n * h * w * c, dtype=torch.int8, device=x.device)
         nbytes = scratch.numel() * scratch.element_size()
     _check(load().hatq_layer(_ptr(x), int(x_kind), float(s_in), n, h, w, ctypes.byref(L.struct), _ptr(y),
-                             _ptr(scratch), nbytes, _stream(stream)))
+                             _ptr(scratch), nbytes, _launch_stream(stream)))
     return y
 
 
@@ -744,11 +752,11 @@ def layer_noalloc(x, x_kind, s_in, L: PreparedLayer, y=None, stream=None):
     memory; the staged INT8 operand lives in the library's fixed device array
     (at most HATQ_NOALLOC_MAX_BYTES bytes, shared by all calls)."""
     n, h, w, c = _check_layer_io(x, x_kind, L, y)
-    torch = _torch()
+    import torch
     if y is None:
         y = torch.empty(L.out_shape(n, h, w), dtype=getattr(torch, L.out_dtype), device=x.device)
     _check(load().hatq_layer_noalloc(_ptr(x), int(x_kind), float(s_in), n, h, w, ctypes.byref(L.struct), _ptr(y),
-                                     _stream(stream)))
+                                     _launch_stream(stream)))
     return y
 
 

@@ -415,6 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // A failure already recorded by this launch (or an earlier, unread one)
     // ends every CTA that has not started, so a fault cannot serialize waits.
     // One thread reads the word so the whole CTA takes the same decision.
+    pdl_enter();
     __shared__ int s_skip;
     if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile int *>(a.err);
     __syncthreads();
@@ -1185,8 +1186,17 @@ cudaError_t launch_conv(const CUtensorMap &tmA, const CUtensorMap &tmB, const CU
         sms_of[dev] = sms > 0 ? sms : 1;
     }
     const int grid = a.num_tiles < sms_of[dev] ? a.num_tiles : sms_of[dev];
-    kern<<<grid, kThreads, smem_bytes, s>>>(tmA, tmB, tmY, a);
-    return cudaGetLastError();
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem_bytes;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmY, a);
 }
 
 #endif

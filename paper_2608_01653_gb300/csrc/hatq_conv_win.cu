@@ -91,6 +91,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // reading decides)
     __shared__ int s_skip;
     const uint32_t rank = PAIR ? blockIdx.x & 1u : 0u;   // in the pair, 0 the leader
+    pdl_enter();
     if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile int *>(a.err);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int S = a.stages;
@@ -598,12 +599,14 @@ cudaError_t launch_conv_win(const CUtensorMap &tmA, const CUtensorMap &tmB, cons
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = smem_bytes;
     cfg.stream = s;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 2;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = pr;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1 + pr;
     return cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmY, a);
 }
 

@@ -6,7 +6,8 @@ ragged outputs. Bit-exact against the oracle."""
 import numpy as np
 import pytest
 
-from tests.test_gpu_conv_lean import H, layer_from_codes, run_both  # noqa: F401
+from synth import configs as C
+from tests.test_gpu_conv_lean import H, dev, layer_from_codes, run_both  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
@@ -95,3 +96,52 @@ def test_pairs_with_odd_tiles(H, n, h, w, c_out, hb_next):
     uniform ones, so that it takes two."""
     case(H, 320, c_out, 3, 1, hb_next, n, h, w, lim=40)
     case(H, 320, c_out, 3, 1, hb_next, n, h, w, chunks=2)
+
+
+@pytest.mark.parametrize("h,w", [(16, 24), (67, 131)])
+def test_dependent_launches_back_to_back(H, h, w):
+    """Kernels whose CTAs may be placed before their predecessor has ended: five dependent layers
+    of the general, window and GDN kernels, queued many times without a host wait, eagerly and from
+    a captured graph; every run's codes equal the first ones, which were waited for one by one."""
+    import torch
+    rng = np.random.default_rng(h)
+    layers, s_x, std = [], 0.05, 0.05 * 35
+    for k in (3, 1, 5, 3):
+        std *= 0.05 * 8 * k * 0.7
+        s_y = float(np.float32(std * 5 / 127))
+        L = C.layer("t", 64, 64, k, 1, k // 2, "DH", "relu", hb_in=64)
+        wts = (rng.standard_normal((64, k, k, 64)) * 0.05).astype(np.float32)
+        layers.append(H.prepare_weights(H.desc_from_spec(L), wts, None, s_x, s_y, "relu", 64))
+        s_x = s_y
+    gdn = H.prepare_gdn(64, 0.5 + rng.random(64), np.abs(rng.standard_normal((64, 64))) * 0.01, 0.04, 0.02, False, 0.05, 64)
+    x = dev(rng.integers(-60, 61, size=(2, h, w, 64)).astype(np.int8))
+    bufs = [torch.empty_like(x) for _ in range(5)]
+
+    def run(wait=False):
+        cur = x
+        for P, y in zip(layers + [None], bufs):
+            H.gdn(cur, gdn, y=y) if P is None else H.conv2d_i8(cur, P, y=y)
+            if wait:
+                H.sync_status()
+            cur = y
+
+    run(wait=True)
+    ref = [b.clone() for b in bufs]
+    assert all(len(torch.unique(b)) > 10 for b in ref)
+    for _ in range(20):
+        for b in bufs:
+            b.zero_()
+        run()
+        run()
+        H.sync_status()
+        assert all(torch.equal(a, b) for a, b in zip(bufs, ref))
+    graph = torch.cuda.CUDAGraph()
+    side = torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=side):
+        run()
+    for b in bufs:
+        b.zero_()
+    for _ in range(10):
+        graph.replay()
+    H.sync_status()
+    assert all(torch.equal(a, b) for a, b in zip(bufs, ref))

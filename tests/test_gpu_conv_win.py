@@ -41,6 +41,27 @@ def test_several_exact_chunks_per_tile(H, c_in, c_out, k, stride, hb_next, chunk
     case(H, c_in, c_out, k, stride, hb_next, 9, 64 * stride, 40 * stride, chunks=chunks)
 
 
+@pytest.mark.parametrize("c_in,chunks", [(256, 2), (320, 2), (576, 3)])
+@pytest.mark.parametrize("c_out,images", [(32, 24), (352, 5)])
+def test_drained_tiles_with_columns_for_one_warpgroup(H, c_in, chunks, c_out, images):
+    """Tiles of 32 columns drained over several chunks: the second epilogue warpgroup has no
+    columns of its own and only takes part in the regions' release. Ten tiles per CTA (with and
+    without CTA pairs), so each region is handed over many times. The images repeat two base ones."""
+    rng = np.random.default_rng(c_in + c_out)
+    L, wt = layer_from_codes(rng.integers(-127, 128, size=(c_out, 3, 3, c_in)), "DH", 1, "relu")
+    base = rng.integers(-127, 128, size=(2, 64, 40, c_in)).astype(np.int8)
+    pick = rng.integers(0, 2, images * 4)
+    s_y = 0.0254 * np.sqrt(9 * c_in)
+    b = rng.normal(0, 1, c_out).astype(np.float32)
+    _, ref, P = run_both(H, L, wt, b, 0.05, s_y, 0, base)
+    units = -(-c_in // 64)
+    assert -(-units // P.struct.chunk_units) == chunks
+    for _ in range(3):
+        y = H.conv2d_i8(dev(base[pick]), P)
+        H.sync_status()
+        assert np.array_equal(y.cpu().numpy(), ref[pick])
+
+
 @pytest.mark.parametrize("hb_out,hb_next", [(64, 64), (64, 0), (64, 32)])
 def test_output_transform_with_chunks(H, hb_out, hb_next):
     """A WH layer of several chunks: the 64-wide output transform is shared by two warps."""

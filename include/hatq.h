@@ -288,6 +288,28 @@ hatq_status hatq_layer_noalloc(const void *x, int x_kind, float s_in, int n, int
  * arguments (for launch accounting), or -1 for invalid arguments. */
 int hatq_layer_launches(int x_kind, float s_in, const hatq_prepared *L);
 
+/* The kernel that hatq_conv2d_i8 (r = 0) or hatq_conv2d_i8_subpixel (factor r)
+ * launches for a layer and an input size, for tests and profiles. Host only:
+ * no device is touched and the layer's buffers are not read. The status is the
+ * one that the call's own checks of layer and size give. */
+typedef enum {
+    HATQ_KERNEL_NONE = 0,     /* empty batch */
+    HATQ_KERNEL_GENERAL = 1,  /* conv_kernel with every option */
+    HATQ_KERNEL_LEAN = 2,     /* conv_kernel for plain INT8 codes of one exact chunk */
+    HATQ_KERNEL_WINDOW = 3    /* conv_win_kernel */
+} hatq_kernel;
+typedef struct {
+    int kernel;        /* hatq_kernel */
+    int epilogue;      /* LEAN: transform group (32, 64, 128); WINDOW: epilogue number (hatq_conv_win.cu) */
+    int pair;          /* WINDOW: 1 when it runs as CTA pairs */
+    int n_t;           /* output channels per tile */
+    int chunks;        /* exact chunks of the reduction per tile */
+    int stages;        /* pipeline stages */
+    int blocks;        /* 64-wide reduction blocks per stage */
+    int smem_bytes;    /* dynamic shared memory */
+} hatq_conv_kernel_info;
+hatq_status hatq_conv_kernel(const hatq_prepared *L, int n, int h, int w, int r, hatq_conv_kernel_info *info);
+
 /* Message describing the calling thread's most recent failure ("" if none). */
 const char *hatq_last_error(void);
 

@@ -995,12 +995,20 @@ int win_plan(const hatq_conv_desc &d, const Geometry &g, const hatq_prepared &L,
     return a.bar_off + a.const_off + const_bytes + 1024;
 }
 
-hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared *L, void *y, hatq_stream stream,
-                        const OutGrid *og, const float *affine_s = nullptr) {
-    if (!L) return fail(HATQ_ERR_INVALID_ARG, "null layer");
-    if (n == 0 && h >= 1 && w >= 1) return HATQ_OK;                    // empty batch: nothing to do
-    if (!x || !y) return fail(HATQ_ERR_INVALID_ARG, "null argument");
-    if (!aligned16(x) || !aligned16(y)) return fail(HATQ_ERR_INVALID_ARG, "input and output must be 16-byte aligned");
+// What one convolution launch runs: the kernel, its arguments (but for the
+// buffers of the call) and its shared memory. Host only.
+struct ConvPlan {
+    Geometry g;
+    hatq::ConvArgs a;        // conv_kernel, lean or with every option
+    int smem_bytes;
+    hatq::WinArgs wa;        // conv_win_kernel, taken where win_smem is not 0
+    int epi, win_smem;
+    bool empty;              // no output: nothing to launch
+};
+
+hatq_status conv_plan(int n, int h, int w, const hatq_prepared *L, const OutGrid *og, bool affine, ConvPlan &p) {
+    p.empty = true;
+    p.win_smem = 0;
     const hatq_conv_desc *d = &L->d;
     hatq_status st = check_desc(d);
     if (st != HATQ_OK) return st;
@@ -1017,18 +1025,20 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     }
     if (ho < 1 || wo < 1) return HATQ_OK;
     if ((long long)n * h * w * d->c_in >= (1LL << 40)) return fail(HATQ_ERR_UNSUPPORTED, "input too large");
-    if ((L->in_affine != 0) != (affine_s != nullptr))
+    if ((L->in_affine != 0) != affine)
         return fail(HATQ_ERR_INVALID_ARG, L->in_affine ? "a layer prepared for affine activations runs through "
                                                          "hatq_conv2d_affine"
                                                        : "hatq_conv2d_affine needs a layer from "
                                                          "hatq_prepare_weights_affine");
     if (n == 0) return HATQ_OK;
-    Geometry g;
+    p.empty = false;
+    Geometry &g = p.g;
     if ((st = geometry(d, L->hb_next, &g)) != HATQ_OK) return st;
     if (g.k_pad != L->k_pad || g.gather != L->gather) return fail(HATQ_ERR_INVALID_ARG, "prepared layer is inconsistent");
     if ((long long)n * ((ho + 0) * (long long)wo) > (1LL << 31)) return fail(HATQ_ERR_UNSUPPORTED, "too many output pixels");
 
-    hatq::ConvArgs a{};
+    hatq::ConvArgs &a = p.a;
+    a = hatq::ConvArgs{};
     a.n = n; a.h = h; a.w = w; a.c = d->c_in;
     a.ho = ho; a.wo = wo; a.co = d->c_out;
     a.kh = d->kh; a.kw = d->kw; a.stride = d->stride;
@@ -1139,18 +1149,16 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     const int bar_bytes = 8 * (3 * a.stages + 9) + 16;
     a.const_off = (bar_bytes + table_bytes + 127) & ~127;
     a.win_off = a.const_off + const_bytes;
-    const int smem_bytes = a.stages * a.stage_bytes + a.staging_bytes + 1024 + a.win_off + win_bytes;
+    const int smem_bytes = p.smem_bytes = a.stages * a.stage_bytes + a.staging_bytes + 1024 + a.win_off + win_bytes;
     // the exchange of a 128-wide next-layer transform uses the output tile: 2 x 128 rows x 64 bytes
     if (!a.lean && g.G == 128 && L->hb_next == 128 && a.staging_bytes < 2 * kTileRows * 64)
         return fail(HATQ_ERR_UNSUPPORTED, "output tile too small for the 128-wide transition exchange");
     if (smem_bytes > 227 * 1024 - 1024) return fail(HATQ_ERR_UNSUPPORTED, "shared memory budget exceeded (%d bytes)", smem_bytes);
     if (a.affine && g.gather) return fail(HATQ_ERR_UNSUPPORTED, "affine activations need c_in % 16 == 0");
-    a.x = static_cast<const int8_t *>(x);
     a.b_int = L->b_int;
     a.mult = L->mult;
     a.deq = L->deq;
     a.s_w = L->s_w;
-    a.affine_s = affine_s;
     a.inv_gamma = d->form == HATQ_WH ? (float)(1.0 / std::sqrt((double)d->hb_out)) : 1.0f;
     a.shift = L->shift;
     a.hb_out = d->form == HATQ_WH ? d->hb_out : 0;
@@ -1162,6 +1170,27 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     a.lut_off = a.const_off + ((4 * d->c_out * 4 + 127) & ~127);
     std::memcpy(a.lut, L->lut, sizeof a.lut);
     a.out_f32 = L->out_f32;
+    if (!L->out_f32 && !a.affine && !a.a_f16 && !a.out_f16 && !g.gather)
+        p.win_smem = win_plan(*d, g, *L, og, n, ho, wo, (long long)a.tiles_w * a.tw * a.tiles_h * a.th, p.wa, p.epi);
+    return HATQ_OK;
+}
+
+hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared *L, void *y, hatq_stream stream,
+                        const OutGrid *og, const float *affine_s = nullptr) {
+    if (!L) return fail(HATQ_ERR_INVALID_ARG, "null layer");
+    if (n == 0 && h >= 1 && w >= 1) return HATQ_OK;                    // empty batch: nothing to do
+    if (!x || !y) return fail(HATQ_ERR_INVALID_ARG, "null argument");
+    if (!aligned16(x) || !aligned16(y)) return fail(HATQ_ERR_INVALID_ARG, "input and output must be 16-byte aligned");
+    ConvPlan p;
+    const hatq_status st = conv_plan(n, h, w, L, og, affine_s != nullptr, p);
+    if (st != HATQ_OK || p.empty) return st;
+    const hatq_conv_desc *d = &L->d;
+    const Geometry &g = p.g;
+    hatq::ConvArgs &a = p.a;
+    hatq::WinArgs &wa = p.wa;
+    const int ho = a.ho, wo = a.wo, epi = p.epi, win_smem = p.win_smem;
+    a.x = static_cast<const int8_t *>(x);
+    a.affine_s = affine_s;
     a.y = y;
     a.err = err_word();
     if (!a.err) return fail(HATQ_ERR_CUDA, "no CUDA device");
@@ -1169,12 +1198,7 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     CUtensorMap tmB, tmA, tmY;
     std::memcpy(&tmB, L->opaque, sizeof tmB);
     tmY = tmB;
-    hatq::WinArgs wa;
-    int epi = 0, win_smem = 0;
-    const bool win_ok = !L->out_f32 && !a.affine && !a.a_f16 && !a.out_f16 && !g.gather;
-    if (win_ok)
-        win_smem = win_plan(*d, g, *L, og, n, ho, wo, (long long)a.tiles_w * a.tw * a.tiles_h * a.th, wa, epi);
-    if (a.lean || (win_smem && !a.d2s)) {
+    if (win_smem ? !a.d2s : a.lean) {
         // the launch's output pixels as a [n][ho][wo][co] tensor (a parity class of a transposed
         // convolution: every ostride-th row and column from (ooy, oox)); a box is the 32 rows of one
         // epilogue warp, 64 (G = 32: 32) channels wide, swizzled over its row
@@ -1252,8 +1276,19 @@ hatq_status conv_launch(const void *x, int n, int h, int w, const hatq_prepared 
     } else {
         tmA = tmB;
     }
-    cudaError_t e = hatq::launch_conv(tmA, tmB, tmY, a, smem_bytes, reinterpret_cast<cudaStream_t>(stream));
+    cudaError_t e = hatq::launch_conv(tmA, tmB, tmY, a, p.smem_bytes, reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(e, "convolution launch");
+    return HATQ_OK;
+}
+
+// The output grid of a sub-pixel layer of factor r.
+hatq_status subpixel_grid(const hatq_prepared *L, int h, int w, int r, OutGrid *og) {
+    const hatq_conv_desc *d = &L->d;
+    if (h < 1 || w < 1) return fail(HATQ_ERR_INVALID_ARG, "bad input shape");
+    const int ho = (h + 2 * d->pad - d->kh) / d->stride + 1, wo = (w + 2 * d->pad - d->kw) / d->stride + 1;
+    if (h + 2 * d->pad < d->kh || w + 2 * d->pad < d->kw || ho < 1 || wo < 1)
+        return fail(HATQ_ERR_INVALID_ARG, "input smaller than the kernel");
+    *og = OutGrid{d->pad, d->pad, ho, wo, ho, wo, 1, 0, 0, r};
     return HATQ_OK;
 }
 
@@ -1380,16 +1415,35 @@ hatq_status hatq_conv2d_i8(const int8_t *x, int n, int h, int w, const hatq_prep
     return conv_launch(x, n, h, w, L, y, stream, nullptr);
 }
 
+hatq_status hatq_conv_kernel(const hatq_prepared *L, int n, int h, int w, int r, hatq_conv_kernel_info *info) {
+    if (!L || !info) return fail(HATQ_ERR_INVALID_ARG, "null argument");
+    if (r != 0 && (r < 2 || r > 4)) return fail(HATQ_ERR_INVALID_ARG, "sub-pixel factor must be 0 or 2..4");
+    *info = hatq_conv_kernel_info{};
+    if (n == 0 && h >= 1 && w >= 1) return HATQ_OK;
+    hatq_status st = check_desc(&L->d);
+    if (st != HATQ_OK) return st;
+    OutGrid og{};
+    if (r && (st = subpixel_grid(L, h, w, r, &og)) != HATQ_OK) return st;
+    ConvPlan p;
+    st = conv_plan(n, h, w, L, r ? &og : nullptr, L->in_affine != 0, p);
+    if (st != HATQ_OK || p.empty) return st;
+    if (p.win_smem) {
+        *info = {HATQ_KERNEL_WINDOW, p.epi, p.wa.pair, p.wa.n_t, p.wa.nch, p.wa.stages, p.wa.seg, p.win_smem};
+    } else {
+        const int chunks = (p.a.num_kb + p.a.chunk_kb - 1) / p.a.chunk_kb;
+        *info = {p.a.lean ? HATQ_KERNEL_LEAN : HATQ_KERNEL_GENERAL, p.a.lean ? p.a.group : 0, 0, p.a.n_t, chunks,
+                 p.a.stages, p.a.sub, p.smem_bytes};
+    }
+    return HATQ_OK;
+}
+
 hatq_status hatq_conv2d_i8_subpixel(const int8_t *x, int n, int h, int w, const hatq_prepared *L, int r, void *y,
                                     hatq_stream stream) {
     if (!L) return fail(HATQ_ERR_INVALID_ARG, "null layer");
     if (r < 2 || r > 4) return fail(HATQ_ERR_INVALID_ARG, "sub-pixel factor must be 2..4");
-    const hatq_conv_desc *d = &L->d;
-    if (h < 1 || w < 1) return fail(HATQ_ERR_INVALID_ARG, "bad input shape");
-    const int ho = (h + 2 * d->pad - d->kh) / d->stride + 1, wo = (w + 2 * d->pad - d->kw) / d->stride + 1;
-    if (h + 2 * d->pad < d->kh || w + 2 * d->pad < d->kw || ho < 1 || wo < 1)
-        return fail(HATQ_ERR_INVALID_ARG, "input smaller than the kernel");
-    const OutGrid og{d->pad, d->pad, ho, wo, ho, wo, 1, 0, 0, r};
+    OutGrid og{};
+    const hatq_status st = subpixel_grid(L, h, w, r, &og);
+    if (st != HATQ_OK) return st;
     return conv_launch(x, n, h, w, L, y, stream, &og);
 }
 

@@ -67,6 +67,13 @@ class PreparedGdnStruct(ctypes.Structure):
                 ("opaque", ctypes.c_uint64 * 16)]
 
 
+KERNEL_NONE, KERNEL_GENERAL, KERNEL_LEAN, KERNEL_WINDOW = range(4)
+
+
+class KernelInfo(ctypes.Structure):
+    _fields_ = [(k, ctypes.c_int) for k in ("kernel", "epilogue", "pair", "n_t", "chunks", "stages", "blocks", "smem_bytes")]
+
+
 _LIB = None
 _P = ctypes.c_void_p
 _I = ctypes.c_int
@@ -124,6 +131,7 @@ def load(build: bool = True) -> ctypes.CDLL:
                                            ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(_I)]),
             "hatq_prepare_gdn": (_I, [_I, _P, _P, _F, _F, _I, _F, _I, ctypes.POINTER(PreparedGdnStruct), _P]),
             "hatq_gdn": (_I, [_P, _I, _I, _I, ctypes.POINTER(PreparedGdnStruct), _P, _P]),
+            "hatq_conv_kernel": (_I, [ctypes.POINTER(PreparedStruct), _I, _I, _I, _I, ctypes.POINTER(KernelInfo)]),
             "hatq_set_operand_format": (_I, [ctypes.POINTER(PreparedStruct), _I, _I]),
             "hatq_version": (_I, []),
         }
@@ -705,6 +713,14 @@ def layer(x, x_kind, s_in, L: PreparedLayer, y=None, scratch=None, stream=None):
 
 def layer_launches(x_kind, s_in, L: PreparedLayer) -> int:
     return int(load().hatq_layer_launches(int(x_kind), float(s_in), ctypes.byref(L.struct)))
+
+
+def conv_kernel(L, n, h, w, r=0) -> KernelInfo:
+    """hatq_conv_kernel: the kernel a convolution call on [n, h, w, c_in] takes (r: sub-pixel factor, 0 none).
+    L: a PreparedLayer or its struct. Host only."""
+    info = KernelInfo()
+    _check(load().hatq_conv_kernel(ctypes.byref(getattr(L, "struct", L)), int(n), int(h), int(w), int(r), ctypes.byref(info)))
+    return info
 
 
 def sync_status(stream=None):

@@ -63,6 +63,7 @@ def test_power_of_two_scales_round_ties_to_even(H, c_out, form, hb_next, act, sh
     s_y = float(np.float32(2.0 ** -10 * 2.0 ** (shift - 30) / alpha))
     got, ref, P = run_both(H, L, w, np.zeros(c_out, np.float32), 1.0, s_y, hb_next, x)
     assert np.array_equal(got, ref)
+    assert H.conv_kernel(P, 2, 9, 37).kernel == H.KERNEL_WINDOW
     if hb_next != 128 and hb_next != 32:                   # alpha is a power of two
         assert P.struct.shift == shift
     assert len(np.unique(ref)) > 3
@@ -85,6 +86,7 @@ def test_biases_that_leave_every_code_uncertain(H, c_in, k, c_out, hb_next, act)
     b = (1500 * 8 * s_y * sign).astype(np.float32)
     got, ref, P = run_both(H, L, w, b, 0.02, float(np.float32(s_y)), hb_next, x)
     assert np.array_equal(got, ref)
+    assert H.conv_kernel(P, 2, 19, 23).kernel == (H.KERNEL_WINDOW if (c_in, k) == (64, 3) else H.KERNEL_LEAN)
     assert len(np.unique(ref)) > 20
 
 
@@ -95,8 +97,9 @@ def test_ragged_output_boxes(H, h, w, c_out, hb_next):
     rng = np.random.default_rng(h * 1000 + w)
     L, wt = layer_from_codes(rng.integers(-127, 128, size=(c_out, 1, 1, 64)), "DH", 1, "relu")
     x = rng.integers(-127, 128, size=(2, h, w, 64)).astype(np.int8)
-    got, ref, _ = run_both(H, L, wt, rng.normal(0, 1, c_out).astype(np.float32), 0.05, 0.11, hb_next, x)
+    got, ref, P = run_both(H, L, wt, rng.normal(0, 1, c_out).astype(np.float32), 0.05, 0.11, hb_next, x)
     assert np.array_equal(got, ref)
+    assert H.conv_kernel(P, 2, h, w).kernel == H.KERNEL_LEAN
 
 
 @pytest.mark.parametrize("avg,one_chunk", [(120, True), (122, False)])
@@ -121,4 +124,5 @@ def test_whole_reduction_in_one_exact_chunk(H, avg, one_chunk, sign):
     got, ref, P = run_both(H, L, w, b, 1.0, float(np.float32(8 * s_w)), 0, x)
     assert np.array_equal(got, ref)
     assert (P.struct.chunk_kb >= k // 64) == one_chunk
+    assert H.conv_kernel(P, 1, 5, 27).kernel == (H.KERNEL_LEAN if one_chunk else H.KERNEL_GENERAL)
     assert len(np.unique(ref)) > 3

@@ -2,7 +2,8 @@
 its units, K steps, chunks and window offsets can go wrong: channel counts that
 do not fill a 64-channel block, 32-channel layers, both strides with odd and
 even kernels, several exact chunks per tile with and without 128-wide groups,
-ragged outputs. Bit-exact against the oracle."""
+ragged outputs. Bit-exact against the oracle; every test also asserts which kernel
+and epilogue its sizes take."""
 import numpy as np
 import pytest
 
@@ -12,9 +13,20 @@ from tests.test_gpu_conv_lean import H, dev, layer_from_codes, run_both  # noqa:
 pytestmark = pytest.mark.gpu
 
 
-def case(H, c_in, c_out, k, stride, hb_next, n, h, w, act="relu", form="DH", lim=127, chunks=None):
+def takes(H, P, n, h, w, kernel=None, epilogue=None, pair=None, r=0):
+    """Asserts the kernel of the call (the window kernel if not said otherwise), its epilogue number
+    and whether it runs as CTA pairs."""
+    info = H.conv_kernel(P, n, h, w, r)
+    assert info.kernel == (H.KERNEL_WINDOW if kernel is None else kernel)
+    assert epilogue is None or info.epilogue == epilogue
+    assert pair is None or info.pair == pair
+
+
+def case(H, c_in, c_out, k, stride, hb_next, n, h, w, act="relu", form="DH", lim=127, chunks=None, **kernel):
     rng = np.random.default_rng(c_in * 31 + c_out + k)
-    L, wt = layer_from_codes(rng.integers(-lim, lim + 1, size=(c_out, k, k, c_in)), form, stride, act)
+    q = rng.integers(-lim, lim + 1, size=(c_out, k, k, c_in))
+    q[:, k // 2, k // 2, 0] = 127                            # the channel's scale: the codes stay as drawn
+    L, wt = layer_from_codes(q, form, stride, act)
     x = rng.integers(-127, 128, size=(n, h, w, c_in)).astype(np.int8)
     s_y = 0.0002 * lim * np.sqrt(k * k * c_in)
     got, ref, P = run_both(H, L, wt, rng.normal(0, 1, c_out).astype(np.float32), 0.05, s_y, hb_next, x)
@@ -23,6 +35,7 @@ def case(H, c_in, c_out, k, stride, hb_next, n, h, w, act="relu", form="DH", lim
     if chunks is not None:
         units = (c_in + 63) // 64 * (2 if stride == 2 else 1)
         assert -(-units // P.struct.chunk_units) == chunks
+    takes(H, P, n, h, w, **kernel)
 
 
 @pytest.mark.parametrize("c_in", [16, 32, 48, 64, 80, 96, 160, 224])
@@ -38,7 +51,9 @@ def test_several_exact_chunks_per_tile(H, c_in, c_out, k, stride, hb_next, chunk
     """Uniform codes (mean 64): the reduction needs several chunks, drained into registers
     (groups up to 64) or kept in two accumulator regions (128-wide groups). 20 tiles per image,
     so that CTAs of the last layers run several tiles and the regions are reused."""
-    case(H, c_in, c_out, k, stride, hb_next, 9, 64 * stride, 40 * stride, chunks=chunks)
+    epilogue = 2064 if hb_next < 128 else 2128 if chunks == 2 else 1128
+    case(H, c_in, c_out, k, stride, hb_next, 9, 64 * stride, 40 * stride, chunks=chunks, epilogue=epilogue,
+         pair=int(c_in * k * k // 64 >= 40))
 
 
 @pytest.mark.parametrize("c_in,chunks", [(256, 2), (320, 2), (576, 3)])
@@ -56,25 +71,51 @@ def test_drained_tiles_with_columns_for_one_warpgroup(H, c_in, chunks, c_out, im
     _, ref, P = run_both(H, L, wt, b, 0.05, s_y, 0, base)
     units = -(-c_in // 64)
     assert -(-units // P.struct.chunk_units) == chunks
+    takes(H, P, images * 4, 64, 40, epilogue=2064, pair=int(c_in > 256))
+    assert H.conv_kernel(P, images * 4, 64, 40).n_t == 32
     for _ in range(3):
         y = H.conv2d_i8(dev(base[pick]), P)
         H.sync_status()
         assert np.array_equal(y.cpu().numpy(), ref[pick])
 
 
+@pytest.mark.parametrize("n,h,w", [(2, 33, 17), (21, 64, 40)])     # ragged; more pairs of tiles than CTA pairs
 @pytest.mark.parametrize("hb_out,hb_next", [(64, 64), (64, 0), (64, 32)])
-def test_output_transform_with_chunks(H, hb_out, hb_next):
-    """A WH layer of several chunks: the 64-wide output transform is shared by two warps."""
-    case(H, 320, 192, 3, 1, hb_next, 1, 33, 26, form="WH", chunks=2)
+def test_output_transform_with_chunks(H, hb_out, hb_next, n, h, w):
+    """A WH layer of several chunks: the 64-wide output transform is shared by two warps. The
+    images repeat two base ones."""
+    rng = np.random.default_rng(hb_next + h)
+    L, wt = layer_from_codes(rng.integers(-127, 128, size=(192, 3, 3, 320)), "WH", 1, "relu")
+    base = rng.integers(-127, 128, size=(2, h, w, 320)).astype(np.int8)
+    pick = np.concatenate([[0, 1], rng.integers(0, 2, n - 2)])
+    _, ref, P = run_both(H, L, wt, rng.normal(0, 1, 192).astype(np.float32), 0.05, 0.0254 * np.sqrt(9 * 320), hb_next, base)
+    assert np.mean(np.abs(ref.astype(int)) == 127) < 0.2 and len(np.unique(ref)) > 20
+    takes(H, P, n, h, w, epilogue=2064, pair=1)
+    assert H.conv_kernel(P, n, h, w).chunks == 2
+    y = H.conv2d_i8(dev(base[pick]), P)
+    H.sync_status()
+    assert np.array_equal(y.cpu().numpy(), ref[pick])
 
 
-@pytest.mark.parametrize("h,w", [(16, 8), (17, 9), (15, 7), (1, 40), (48, 1)])
+@pytest.mark.parametrize("hb_next", [0, 32, 64])
+def test_output_transform_with_chunks_in_the_general_kernel(H, hb_next):
+    """The same layer on an output that fills 8 x 16 tiles badly."""
+    case(H, 320, 192, 3, 1, hb_next, 1, 33, 26, form="WH", chunks=2, kernel=H.KERNEL_GENERAL)
+
+
+@pytest.mark.parametrize("h,w", [(16, 8), (31, 15), (15, 7), (17, 23), (48, 1), (33, 17)])
 def test_ragged_windows(H, h, w):
-    case(H, 64, 192, 3, 1, 64, 3, h, w)
+    case(H, 64, 192, 3, 1, 64, 3, h, w, epilogue=64, pair=0)
+
+
+@pytest.mark.parametrize("h,w", [(17, 9), (1, 40), (33, 26)])
+def test_outputs_that_fill_the_tiles_badly(H, h, w):
+    """The other side of the rule: these take the general kernel's lean form."""
+    case(H, 64, 192, 3, 1, 64, 3, h, w, kernel=H.KERNEL_LEAN, epilogue=64)
 
 
 @pytest.mark.parametrize("c_out,form", [(256, "DH"), (192, "WH"), (768, "DH")])
-@pytest.mark.parametrize("h,w", [(33, 26), (16, 8), (17, 5)])
+@pytest.mark.parametrize("h,w", [(33, 26), (16, 8), (17, 5), (33, 17), (100, 36)])
 def test_subpixel_stores(H, c_out, form, h, w):
     """The factor-2 rearrangement in the epilogue's stores, at ragged tile edges."""
     from oracle import hatq_oracle as O
@@ -84,6 +125,10 @@ def test_subpixel_stores(H, c_out, form, h, w):
     x = rng.integers(-127, 128, size=(3, h, w, 64)).astype(np.int8)
     b = rng.normal(0, 1, c_out).astype(np.float32)
     P = H.prepare_weights(H.desc_from_spec(L), wt, b, 0.05, 0.3, L.act, 0, False)
+    if (h, w) == (33, 26):
+        takes(H, P, 3, h, w, kernel=H.KERNEL_GENERAL, r=2)
+    else:
+        takes(H, P, 3, h, w, epilogue=3064, r=2)
     y = H.conv2d_i8_subpixel(dev(x), P, 2)
     H.sync_status()
     p = O.prepare_layer(wt, b, L.form, L.hb_in, L.hb_out, 0.05, 0.3, L.act, 0, False, 1, 1)
@@ -92,15 +137,21 @@ def test_subpixel_stores(H, c_out, form, h, w):
 
 @pytest.mark.parametrize("c_out,form,hb_next", [(192, "DH", 64), (96, "DH", 32), (128, "WH", 64), (96, "DH", 0)])
 @pytest.mark.parametrize("act", ["silu", "gelu"])
-def test_general_transition(H, c_out, form, hb_next, act):
-    """SiLU / GELU through the table, both group widths, several tiles with ragged edges."""
+@pytest.mark.parametrize("n,h,w", [(3, 33, 26), (3, 33, 17), (9, 63, 39)])
+def test_general_transition(H, c_out, form, hb_next, act, n, h, w):
+    """SiLU / GELU through the table, both group widths, several tiles with ragged edges; the
+    first size takes the general kernel, the last has more tiles than CTAs."""
     from oracle import hatq_oracle as O
     from tests.test_gpu_conv_lean import dev
     rng = np.random.default_rng(c_out + hb_next)
     L, wt = layer_from_codes(rng.integers(-60, 61, size=(c_out, 3, 3, 64)), form, 1, act)
-    x = rng.integers(-127, 128, size=(3, 33, 26, 64)).astype(np.int8)
+    x = rng.integers(-127, 128, size=(n, h, w, 64)).astype(np.int8)
     s_z, s_u, s_y = (float(np.float32(v)) for v in (0.2, 0.15, 0.3))
     P = H.prepare_weights(H.desc_from_spec(L), wt, None, 0.05, s_y, act, hb_next, s_z=s_z, s_u=s_u)
+    if (h, w) == (33, 26):
+        takes(H, P, n, h, w, kernel=H.KERNEL_GENERAL)
+    else:
+        takes(H, P, n, h, w, epilogue=4064 if c_out % 64 == 0 else 4032)
     y = H.conv2d_i8(dev(x), P)
     H.sync_status()
     p = O.prepare_layer(wt, None, L.form, L.hb_in, L.hb_out, 0.05, s_y, act, hb_next, False, 1, 1, s_z=s_z, s_u=s_u)
@@ -115,8 +166,9 @@ def test_pairs_with_odd_tiles(H, n, h, w, c_out, hb_next):
     """45 weight blocks (CTA pairs), with one M tile and other odd numbers of them: the last pair's
     second tile lies past the last image. Small codes, so that one chunk holds the reduction, and
     uniform ones, so that it takes two."""
-    case(H, 320, c_out, 3, 1, hb_next, n, h, w, lim=40)
-    case(H, 320, c_out, 3, 1, hb_next, n, h, w, chunks=2)
+    one, two = {64: (64, 2064), 128: (1128, 2128), 0: (32, 2064)}[hb_next]
+    case(H, 320, c_out, 3, 1, hb_next, n, h, w, lim=40, epilogue=one, pair=1)
+    case(H, 320, c_out, 3, 1, hb_next, n, h, w, chunks=2, epilogue=two, pair=1)
 
 
 @pytest.mark.parametrize("h,w", [(16, 24), (67, 131)])

@@ -1103,7 +1103,6 @@ hatq_status conv_plan(int n, int h, int w, const hatq_prepared *L, const OutGrid
     const bool general = L->act == HATQ_ACT_SILU || L->act == HATQ_ACT_GELU;
     // the lean kernels: INT8 codes of one exact chunk per tile, no further option
     const bool plain = !general && !L->out_f32 && !a.affine && !a.a_f16 && !a.out_f16 && !a.d2s;
-    a.lean = !drains && plain;
     a.group = g.G;
     a.nbuf = (drains || g.G == 128) ? 1 : 2;
     a.tmem_cols = 512;
@@ -1113,7 +1112,6 @@ hatq_status conv_plan(int n, int h, int w, const hatq_prepared *L, const OutGrid
     const int esz = L->out_f32 ? 4 : 1;
     a.row_stride = a.n_t * esz + 16;                 // padded rows: 8 consecutive rows hit 8 bank groups
     a.staging_bytes = L->out_f32 ? 0 : a.nbuf * kTileRows * a.row_stride;   // float32 output is stored directly
-    if (a.lean) a.staging_bytes = 8 * (4096 + 512);  // per epilogue warp two 32-row buffers of 64 columns and two exact rows
     a.win_h = (a.th - 1) * d->stride + d->kh;
     a.win_w = (a.tw - 1) * d->stride + d->kw;
     a.win_pitch = a.win_tma ? window_box_bytes(a.tw, d->stride, d->kw, d->c_in) : (a.win_w * d->c_in + 15) & ~15;
@@ -1124,13 +1122,20 @@ hatq_status conv_plan(int n, int h, int w, const hatq_prepared *L, const OutGrid
     const int table_bytes = g.gather ? a.num_kb * 8 * 4 : 0;
     const int const_bytes = ((4 * d->c_out * 4 + 127) & ~127) + (general ? 256 : 0);
     const int fixed = 1024 /* align */ + 8 * (3 * 8 + 9) + 16 + 128 + table_bytes + const_bytes + win_bytes;
-    const int budget = 227 * 1024 - 1024 /* static */ - fixed - a.staging_bytes;
+    const int room = 227 * 1024 - 1024 /* static */ - fixed;
     // a stage holds `sub` 64-wide reduction blocks: [weights x sub | INT8 box x sub].
     // The cost of a stage is dominated by its barrier hand-offs, not its bytes,
     // so take the widest stage that still leaves two stages and two A slots:
     // four blocks (two 4-block stages, 2 x 128 TMEM columns), else two (three
     // stages, 2 x 64 columns), else one.
     const int one = a.b_bytes + a.raw_bytes;
+    // The lean staging has one size (per epilogue warp two 32-row buffers of 64 columns and two exact
+    // rows), more than the output tiles of narrow N tiles: where two stages do not fit beside it, as in
+    // layers of some 9,000 output channels and more, the layer stays with the other epilogue.
+    constexpr int kLeanStaging = 8 * (4096 + 512);
+    a.lean = !drains && plain && (room - kLeanStaging) / one >= 2;
+    if (a.lean) a.staging_bytes = kLeanStaging;
+    const int budget = room - a.staging_bytes;
     const int free_cols = 512 - a.a_col;
     a.sub = 1;
     if (!g.gather && a.num_kb >= 4 && budget / (4 * one) >= 2 && free_cols >= 256) a.sub = 4;

@@ -108,3 +108,25 @@ def test_plans_stay_within_the_documented_limits():
         else:
             assert i.blocks in (1, 2, 4) and (i.kernel == G or i.chunks == 1)
     assert {k for k, _, _ in seen} == {G, LEAN, WIN} and {e for k, e, _ in seen if k == WIN} >= {32, 64, 1128, 2064, 2128}
+
+
+@pytest.mark.parametrize("k", [1, 3])
+@pytest.mark.parametrize("hb_next", [0, 64, 128])
+def test_wide_layers_are_taken_wherever_a_tile_fits(hb_next, k):
+    """The constants of a wide layer (16 bytes per output channel) leave little shared memory. Every
+    layer for which two single-block stages fit beside the general epilogue's output tile is accepted,
+    whether or not the lean kernel's fixed staging fits there."""
+    G_ = max(32, hb_next)
+    lean = general = 0
+    for c_out in range(8192, 12288 + 1, 128 if hb_next == 128 else 64):
+        n_t = next(t for t in range(224, 0, -16) if t % G_ == 0 and c_out % t == 0)
+        budget = 226 * 1024 - (1024 + 8 * 37 + 16 + 128 + 16 * c_out) - (1 if G_ == 128 else 2) * 128 * (n_t + 16)
+        fits = budget // (n_t * 128 + 8192) >= 2
+        try:
+            i = H.conv_kernel(struct(64, c_out, k, hb_next=hb_next), 1, 16, 8)
+        except H.HatqError as e:
+            assert not fits and e.status == H.ERR_UNSUPPORTED, c_out
+            continue
+        lean, general = lean + (i.kernel == LEAN), general + (i.kernel == G)
+        assert i.stages >= 2 and i.smem_bytes <= 227 * 1024 - 1024
+    assert lean and general

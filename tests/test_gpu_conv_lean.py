@@ -126,3 +126,16 @@ def test_whole_reduction_in_one_exact_chunk(H, avg, one_chunk, sign):
     assert (P.struct.chunk_kb >= k // 64) == one_chunk
     assert H.conv_kernel(P, 1, 5, 27).kernel == (H.KERNEL_LEAN if one_chunk else H.KERNEL_GENERAL)
     assert len(np.unique(ref)) > 3
+
+
+@pytest.mark.parametrize("c_out,hb_next", [(9216, 128), (10048, 64), (9696, 32)])
+def test_wide_layers_without_room_for_the_lean_staging(H, c_out, hb_next):
+    """Their constants leave shared memory for two stages beside the general epilogue's output tile
+    only."""
+    rng = np.random.default_rng(c_out)
+    L, wt = layer_from_codes(rng.integers(-127, 128, size=(c_out, 1, 1, 64)), "DH", 1, "relu")
+    x = rng.integers(-127, 128, size=(1, 5, 31, 64)).astype(np.int8)
+    got, ref, P = run_both(H, L, wt, rng.normal(0, 1, c_out).astype(np.float32), 0.05, 0.11, hb_next, x)
+    assert H.conv_kernel(P, 1, 5, 31).kernel == H.KERNEL_GENERAL
+    assert np.array_equal(got, ref)
+    assert len(np.unique(ref)) > 20

@@ -22,7 +22,7 @@ LIB = os.path.join(BUILD, "libhatq.so")
 SOURCES = ["hatq_conv_win.cu", "hatq_conv_lean.cu", "hatq_conv_lean_pieces.cu", "hatq_conv.cu", "hatq_conv_pieces.cu", "hatq_api.cu",
            "hatq_fwht.cu", "hatq_gdn.cu", "hatq_noalloc.cu", "hatq_profile.cu"]
 HEADERS = [os.path.join(CSRC, "hatq_internal.h"), os.path.join(CSRC, "hatq_tc.h"),
-           os.path.join(CSRC, "hatq_lean.h"), os.path.join(INCLUDE, "hatq.h")]
+           os.path.join(CSRC, "hatq_launch.h"), os.path.join(CSRC, "hatq_lean.h"), os.path.join(INCLUDE, "hatq.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -18,6 +18,7 @@
 
 #include "hatq.h"
 #include "hatq_internal.h"
+#include "hatq_launch.h"
 
 namespace {
 
@@ -957,7 +958,7 @@ int win_plan(const hatq_conv_desc &d, const Geometry &g, const hatq_prepared &L,
     // per epilogue warp two 32-row buffers of 64 columns and two rows for the exact codes
     const int stg_bytes = 8 * (4096 + 512);
     const int const_bytes = (16 * d.c_out + (general ? 256 : 0) + 127) & ~127, bars = 8 * 32 + 16;
-    const int budget = 227 * 1024 - 1024 /* static */ - 1024 /* alignment */ - stg_bytes - 512 - const_bytes - 2 * a.w16_bytes;
+    const int budget = hatq::kMaxDynamicSmem - 1024 /* alignment */ - stg_bytes - 512 - const_bytes - 2 * a.w16_bytes;
     // A weight stage holds the taps of one kernel row (a wait, a commit and the counters per row
     // instead of per tap) where at least six blocks fit in two stages or more, preferably beside two
     // INT8 window buffers; else single blocks, with the second window buffer where four stages remain.
@@ -1122,7 +1123,7 @@ hatq_status conv_plan(int n, int h, int w, const hatq_prepared *L, const OutGrid
     const int table_bytes = g.gather ? a.num_kb * 8 * 4 : 0;
     const int const_bytes = ((4 * d->c_out * 4 + 127) & ~127) + (general ? 256 : 0);
     const int fixed = 1024 /* align */ + 8 * (3 * 8 + 9) + 16 + 128 + table_bytes + const_bytes + win_bytes;
-    const int room = 227 * 1024 - 1024 /* static */ - fixed;
+    const int room = hatq::kMaxDynamicSmem - fixed;
     // a stage holds `sub` 64-wide reduction blocks: [weights x sub | INT8 box x sub].
     // The cost of a stage is dominated by its barrier hand-offs, not its bytes,
     // so take the widest stage that still leaves two stages and two A slots:
@@ -1158,7 +1159,7 @@ hatq_status conv_plan(int n, int h, int w, const hatq_prepared *L, const OutGrid
     // the exchange of a 128-wide next-layer transform uses the output tile: 2 x 128 rows x 64 bytes
     if (!a.lean && g.G == 128 && L->hb_next == 128 && a.staging_bytes < 2 * kTileRows * 64)
         return fail(HATQ_ERR_UNSUPPORTED, "output tile too small for the 128-wide transition exchange");
-    if (smem_bytes > 227 * 1024 - 1024) return fail(HATQ_ERR_UNSUPPORTED, "shared memory budget exceeded (%d bytes)", smem_bytes);
+    if (smem_bytes > hatq::kMaxDynamicSmem) return fail(HATQ_ERR_UNSUPPORTED, "shared memory budget exceeded (%d bytes)", smem_bytes);
     if (a.affine && g.gather) return fail(HATQ_ERR_UNSUPPORTED, "affine activations need c_in % 16 == 0");
     a.b_int = L->b_int;
     a.mult = L->mult;
@@ -1742,11 +1743,7 @@ hatq_status hatq_gdn(const int8_t *z, int n, int h, int w, const hatq_prepared_g
     if (pixels > (1LL << 31) - 256) return fail(HATQ_ERR_UNSUPPORTED, "at most 2^31 - 256 pixels per call");
     const int8_t *zl = z, *zh = z + pixels * c, *yl = y, *yh = y + pixels * c;
     if (zl < yh && yl < zh) return fail(HATQ_ERR_INVALID_ARG, "z and y overlap");
-    int dev = 0, smem_max = 0;
     cudaError_t e;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
-        (e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
-        return cuda_fail(e, "device query");
     hatq::GdnArgs a{};
     a.pixels = pixels;
     a.c = c;
@@ -1775,7 +1772,7 @@ hatq_status hatq_gdn(const int8_t *z, int n, int h, int w, const hatq_prepared_g
         return a.bar_off + 192 + 1024;
     };
     int smem = 0, nz = 4;
-    while (nz > 0 && (smem = layout(nz)) > smem_max - 1024 /* static */) --nz;
+    while (nz > 0 && (smem = layout(nz)) > hatq::kMaxDynamicSmem) --nz;
     if (!nz) return fail(HATQ_ERR_UNSUPPORTED, "the GDN tile does not fit shared memory");
     EncodeTiledFn enc = encode_fn();
     if (!enc) return fail(HATQ_ERR_CUDA, "cuTensorMapEncodeTiled is unavailable");

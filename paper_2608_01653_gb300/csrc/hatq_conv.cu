@@ -54,6 +54,7 @@
 #include <cuda_fp16.h>
 
 #include "hatq_internal.h"
+#include "hatq_launch.h"
 #include "hatq_lean.h"
 #include "hatq_tc.h"
 
@@ -1159,14 +1160,6 @@ cudaError_t launch_wait_selftest(int *err, long long limit_cycles, cudaStream_t 
 
 cudaError_t launch_conv(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmY, const ConvArgs &a,
                         int smem_bytes, cudaStream_t s) {
-    // the shared-memory opt-in and the SM count are per device
-    constexpr int kMaxDev = 64;
-    static int configured_smem[kMaxDev][24] = {};
-    static int sms_of[kMaxDev] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDev) return cudaErrorInvalidDevice;
     if ((a.sub != 1 && a.sub != 2 && a.sub != 4) || (a.gather && a.sub != 1) || a.chunk_kb % a.sub ||
         (a.half && (a.gather || a.a_f16 || a.cin_h < 1)) || (a.lean && a.num_kb > a.chunk_kb))
         return cudaErrorInvalidValue;   // gathered tiles: one block per stage
@@ -1174,18 +1167,13 @@ cudaError_t launch_conv(const CUtensorMap &tmA, const CUtensorMap &tmB, const CU
     const int v = (a.sub == 4 ? 2 : (a.sub == 2 ? 1 : 0)) + (a.half ? 3 : 0) + 6 * fam;
     const ConvKernelFn kern = a.lean ? (a.half ? conv_lean_pieces_kernel(a.sub, a.group) : conv_lean_kernel(a.sub, a.group))
                                      : (a.half ? conv_pieces_kernel(a.sub) : conv_full_kernel(a.sub));
-    if (smem_bytes > configured_smem[dev][v]) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-        if (e != cudaSuccess) return e;
-        configured_smem[dev][v] = smem_bytes;
-    }
-    if (!sms_of[dev]) {
-        int sms = 0;
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        sms_of[dev] = sms > 0 ? sms : 1;
-    }
-    const int grid = a.num_tiles < sms_of[dev] ? a.num_tiles : sms_of[dev];
+    static SmemOptIn opt_in[24];
+    int dev = 0, sms = 0;
+    cudaError_t e;
+    if ((e = current_device(&dev)) != cudaSuccess || (e = opt_in[v].set(dev, reinterpret_cast<const void *>(kern))) != cudaSuccess ||
+        (e = device_sms(dev, &sms)) != cudaSuccess)
+        return e;
+    const int grid = a.num_tiles < sms ? a.num_tiles : sms;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;

@@ -41,6 +41,7 @@
 #include <cuda_fp16.h>
 
 #include "hatq_internal.h"
+#include "hatq_launch.h"
 #include "hatq_lean.h"
 #include "hatq_tc.h"
 
@@ -578,24 +579,13 @@ cudaError_t launch_conv_win(const CUtensorMap &tmA, const CUtensorMap &tmB, cons
     if (v == kKerns) return cudaErrorInvalidValue;
     const int pr = a.pair ? 1 : 0;
     const Fn kern = kerns[v].fn[pr];
-    // the shared-memory opt-in and the SM count are per device
-    constexpr int kMaxDev = 64;
-    static int configured[kMaxDev][kKerns][2] = {};
-    static int sms_of[kMaxDev] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDev) return cudaErrorInvalidDevice;
-    if (smem_bytes > configured[dev][v][pr]) {
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes)) != cudaSuccess) return e;
-        configured[dev][v][pr] = smem_bytes;
-    }
-    if (!sms_of[dev]) {
-        int sms = 0;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        sms_of[dev] = sms > 0 ? sms : 1;
-    }
-    const int groups = pr ? (sms_of[dev] / 2 < 1 ? 1 : sms_of[dev] / 2) : sms_of[dev];
+    static SmemOptIn opt_in[kKerns][2];
+    int dev = 0, sms = 0;
+    cudaError_t e;
+    if ((e = current_device(&dev)) != cudaSuccess || (e = opt_in[v][pr].set(dev, reinterpret_cast<const void *>(kern))) != cudaSuccess ||
+        (e = device_sms(dev, &sms)) != cudaSuccess)
+        return e;
+    const int groups = pr ? (sms / 2 < 1 ? 1 : sms / 2) : sms;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((pr ? 2 : 1) * (a.num_tiles < groups ? a.num_tiles : groups));
     cfg.blockDim = dim3(kThreads);

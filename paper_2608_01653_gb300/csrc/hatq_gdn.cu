@@ -46,6 +46,7 @@
 #include <cuda_fp16.h>
 
 #include "hatq_internal.h"
+#include "hatq_launch.h"
 #include "hatq_tc.h"
 
 namespace hatq {
@@ -432,11 +433,13 @@ __global__ void __launch_bounds__(kGdnThreads, 1)
 cudaError_t launch_gdn(const CUtensorMap &tmZ, const CUtensorMap &tmG, const CUtensorMap &tmY, const GdnArgs &a, int smem_bytes,
                        cudaStream_t s) {
     auto kern = a.inverse ? gdn_kernel<true> : gdn_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
+    static SmemOptIn opt_in[2];
     int dev = 0, sms = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    cudaError_t e;
+    if ((e = current_device(&dev)) != cudaSuccess ||
+        (e = opt_in[a.inverse ? 1 : 0].set(dev, reinterpret_cast<const void *>(kern))) != cudaSuccess ||
+        (e = device_sms(dev, &sms)) != cudaSuccess)
+        return e;
     const int grid = a.num_tiles < sms ? a.num_tiles : sms;
     kern<<<grid, kGdnThreads, smem_bytes, s>>>(tmZ, tmG, tmY, a);
     return cudaGetLastError();

@@ -88,7 +88,8 @@ typedef struct {
  * input-independent and stored after offline transformation).
  * The caller sets the six device pointers (sizes from hatq_prepared_sizes)
  * before hatq_prepare_weights fills them; every other field is written by
- * the library. opaque[] holds the library's tensor-memory-access descriptor
+ * the library. A caller that writes other codes into w_i8 / w_f16 afterwards
+ * sets chunk_kb and chunk_units to 0, or the sums may not be exact. opaque[] holds the library's tensor-memory-access descriptor
  * of w_f16 and must not be modified.
  */
 typedef struct {
@@ -102,6 +103,12 @@ typedef struct {
                              entries (kx, c_in) padded with zero weights to a multiple of 8 */
     float s_x;            /* scale of the INT8 operand this layer consumes */
     float s_y;            /* scale of the INT8 codes it emits */
+    /* Exact chunks, written by the preparation from the codes in w_i8 (they take what was padding, so
+     * that every field keeps its place): */
+    uint16_t chunk_kb;    /* 64-wide reduction blocks whose fp32 sums are exact for these codes; 0: the bound
+                             that holds for any codes */
+    uint16_t chunk_units; /* the same for the order of the window convolution: input windows (64 channels, for
+                             stride 2 of one column parity) per exact chunk; 0: that kernel is not taken */
     int8_t *w_i8;         /* [c_out][k_pad] weight codes w_int, K order (kh, kw, c_in); gather == 0: c_in
                              padded to a multiple of 64 per tap, except c_in % 64 == 32 (taps unpadded,
                              the total padded to a multiple of 64); gather == 1: kw*c_in padded to 8 per row */
@@ -121,11 +128,6 @@ typedef struct {
     int8_t lut[256];      /* phi_int of Eq. supp_general_activation at z = -127..127 (index z + 127) */
     int in_f16;           /* 1: the INT8 operand arrives as IEEE fp16 values (exact), see hatq_set_operand_format */
     int out_f16;          /* 1: the INT8 codes are written as IEEE fp16 values (exact) */
-    int chunk_kb;         /* 64-wide reduction blocks whose fp32 sums are exact for these weights (written by the
-                             preparation from w_i8); 0: the bound that holds for any codes. Set it to 0 if
-                             the weight buffers are changed afterwards */
-    int chunk_units;      /* the same for the order of the window convolution: input windows (64 channels, for
-                             stride 2 of one column parity) per exact chunk; 0: that kernel is not taken */
 } hatq_prepared;
 
 /*

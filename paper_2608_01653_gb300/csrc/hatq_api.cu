@@ -10,6 +10,7 @@
 
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <algorithm>
 #include <cstring>
@@ -673,6 +674,17 @@ int exact_units(const std::vector<int8_t> &w, const hatq_conv_desc &d, const Geo
     return 0;
 }
 
+// The chunk fields lie in what was padding behind s_y: a program compiled against the header without
+// them passes a struct of the same size and layout.
+static_assert(sizeof(hatq_prepared) == 536 && offsetof(hatq_prepared, chunk_kb) == 68 && offsetof(hatq_prepared, w_i8) == 72 &&
+                  offsetof(hatq_prepared, opaque) == 120 && offsetof(hatq_prepared, out_f16) == 532,
+              "hatq_prepared keeps its layout");
+// A longer chunk than the field holds is cut (any shorter one is exact too; a multiple of 4 as before).
+void set_chunks(hatq_prepared *L, int kb, int units) {
+    L->chunk_kb = (uint16_t)std::min(kb, 65532);
+    L->chunk_units = (uint16_t)std::min(units, 65535);
+}
+
 // Copies the host arrays to the caller's device buffers, encodes the weight
 // tensor map and fills the struct (dop: the descriptor of the operand).
 hatq_status upload_layer(const hatq_conv_desc &dop, const Geometry &g, const HostLayer &hl, int act, int hb_next,
@@ -719,8 +731,7 @@ hatq_status upload_layer(const hatq_conv_desc &dop, const Geometry &g, const Hos
     out->in_affine = 0;
     out->in_f16 = 0;
     out->out_f16 = 0;
-    out->chunk_kb = exact_chunk(hl.w_i8, co, g.k_pad, 128, kChunkAny);   // INT8 operands, -128 included
-    out->chunk_units = exact_units(hl.w_i8, dop, g, 128);
+    set_chunks(out, exact_chunk(hl.w_i8, co, g.k_pad, 128, kChunkAny), exact_units(hl.w_i8, dop, g, 128));   // -128 included
     out->mult_in = gen ? gen->mult_in : 0;
     if (gen) std::memcpy(out->lut, gen->lut, sizeof out->lut);
     else std::memset(out->lut, 0, sizeof out->lut);
@@ -1478,7 +1489,7 @@ hatq_status hatq_prepare_weights_affine(const hatq_conv_desc *d, const float *w_
     }
     if ((st = upload_layer(dop, g, hl, act, 0, 1, 1.f, 0.f, nullptr, out, stream)) != HATQ_OK) return st;
     out->in_affine = 1;
-    out->chunk_kb = exact_chunk(hl.w_i8, dop.c_out, g.k_pad, 255, kChunkAnyAffine);
+    set_chunks(out, exact_chunk(hl.w_i8, dop.c_out, g.k_pad, 255, kChunkAnyAffine), 0);   // (window kernel: INT8 operands only)
     out->s_x = 0.f;
     return HATQ_OK;
 }

@@ -41,13 +41,13 @@ class PreparedStruct(ctypes.Structure):
     _fields_ = [("d", ConvDesc), ("act", ctypes.c_int), ("hb_next", ctypes.c_int), ("out_f32", ctypes.c_int),
                 ("shift", ctypes.c_int), ("k_pad", ctypes.c_int), ("gather", ctypes.c_int),
                 ("s_x", ctypes.c_float), ("s_y", ctypes.c_float),
+                ("chunk_kb", ctypes.c_uint16), ("chunk_units", ctypes.c_uint16),
                 ("w_i8", ctypes.c_void_p), ("w_f16", ctypes.c_void_p), ("b_int", ctypes.c_void_p),
                 ("mult", ctypes.c_void_p), ("deq", ctypes.c_void_p), ("s_w", ctypes.c_void_p),
                 ("opaque", ctypes.c_uint64 * 16),
                 ("s_z", ctypes.c_float), ("s_u", ctypes.c_float), ("shift_in", ctypes.c_int),
                 ("in_affine", ctypes.c_int), ("mult_in", ctypes.c_longlong), ("lut", ctypes.c_int8 * 256),
-                ("in_f16", ctypes.c_int), ("out_f16", ctypes.c_int), ("chunk_kb", ctypes.c_int),
-                ("chunk_units", ctypes.c_int)]
+                ("in_f16", ctypes.c_int), ("out_f16", ctypes.c_int)]
 
 
 MAX_TRANSPOSED_CLASSES = 4

@@ -308,7 +308,8 @@ def test_prepared_struct_mirror_matches_the_c_layout(tmp_path):
     if cc is None:
         pytest.skip("no C compiler")
     fields = ["d", "act", "hb_next", "out_f32", "shift", "k_pad", "gather", "s_x", "s_y", "w_i8", "w_f16", "b_int",
-              "mult", "deq", "s_w", "opaque", "s_z", "s_u", "shift_in", "in_affine", "mult_in", "lut"]
+              "mult", "deq", "s_w", "opaque", "s_z", "s_u", "shift_in", "in_affine", "mult_in", "lut", "in_f16", "out_f16",
+              "chunk_kb", "chunk_units"]
     src = tmp_path / "layout.c"
     inc = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "include")
     src.write_text("#include <stdio.h>\n#include <stddef.h>\n#include \"hatq.h\"\nint main(void) {\n"
@@ -321,6 +322,19 @@ def test_prepared_struct_mirror_matches_the_c_layout(tmp_path):
     assert ctypes.sizeof(H.PreparedStruct) == out[0]
     for f, off in zip(fields, out[1:]):
         assert getattr(H.PreparedStruct, f).offset == off, f
+
+
+def test_prepared_struct_keeps_its_layout():
+    """Programs compiled against version 1's header pass this struct: 536 bytes with these offsets. The
+    chunk lengths lie in the padding behind s_y."""
+    S = H.PreparedStruct
+    assert H.version() == 1
+    assert ctypes.sizeof(S) == 536
+    expect = dict(d=0, act=36, hb_next=40, out_f32=44, shift=48, k_pad=52, gather=56, s_x=60, s_y=64, chunk_kb=68, chunk_units=70,
+                  w_i8=72, w_f16=80, b_int=88, mult=96, deq=104, s_w=112, opaque=120, s_z=248, s_u=252, shift_in=256,
+                  in_affine=260, mult_in=264, lut=272, in_f16=528, out_f16=532)
+    assert {f: getattr(S, f).offset for f, *_ in S._fields_} == expect
+    assert ctypes.sizeof(H.PreparedTransposedStruct) == H.PreparedTransposedStruct.sub.offset + 4 * 536
 
 
 @pytest.mark.parametrize("hb_out", [0, 16, 32, 64, 128])

@@ -234,7 +234,8 @@ def prepare_weights_host(desc: ConvDesc, w_ohwi, bias, s_x, s_y, act="none", hb_
 
 
 class PreparedLayer:
-    """A prepared layer: device buffers (torch tensors) plus the C struct."""
+    """A prepared layer: device buffers (torch tensors) plus the C struct. The struct's chunk lengths
+    hold for the prepared codes: after writing others into w_i8 / w_f16, call codes_changed()."""
 
     def __init__(self, desc: ConvDesc, device="cuda"):
         torch = _torch()
@@ -253,6 +254,11 @@ class PreparedLayer:
         self.struct.mult = self.mult.data_ptr()
         self.struct.deq = self.deq.data_ptr()
         self.struct.s_w = self.s_w.data_ptr()
+
+    def codes_changed(self):
+        """The layer takes the chunk length that is exact for any codes (and the general kernel, at its
+        speed) from here on: to be called after its weight codes were overwritten."""
+        self.struct.chunk_kb = self.struct.chunk_units = 0
 
     @property
     def c_in(self):
@@ -452,6 +458,11 @@ class PreparedTransposed:
             for k, t in bufs.items():
                 setattr(self.struct.sub[cls], k, t.data_ptr())
             self.buffers.append(bufs)
+
+    def codes_changed(self):
+        """As PreparedLayer.codes_changed, for every parity class."""
+        for sub in self.struct.sub:
+            sub.chunk_kb = sub.chunk_units = 0
 
     @property
     def c_in(self):

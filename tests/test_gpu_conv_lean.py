@@ -139,3 +139,30 @@ def test_wide_layers_without_room_for_the_lean_staging(H, c_out, hb_next):
     assert H.conv_kernel(P, 1, 5, 31).kernel == H.KERNEL_GENERAL
     assert np.array_equal(got, ref)
     assert len(np.unique(ref)) > 20
+
+
+@pytest.mark.parametrize("c_in,k", [(1088, 1), (128, 3)])              # general and window kernel as prepared
+def test_overwritten_weight_codes(H, c_in, k):
+    """Codes written over a prepared layer's, with sums beyond the prepared chunk: exact once the
+    layer has been told. The bias cancels the sum, so the output shows its low bits."""
+    rng = np.random.default_rng(k)
+    q = np.full((32, k, k, c_in), 100)
+    q[:, 0, 0, 0] = 127
+    L, w = layer_from_codes(q, "DH", 1, "none")
+    x = np.full((1, 16, 24, c_in), 127, np.int8)
+    dec = 1 + 40 // (k * k)
+    x[..., 1:dec] -= rng.integers(0, 2, size=(1, 16, 24, dec - 1)).astype(np.int8)
+    total, s_w = 127 * 127 * c_in * k * k, 2.0 ** -10
+    b = np.full(32, -(total - 4000) * s_w, np.float32)
+    P = H.prepare_weights(H.desc_from_spec(L), w, b, 1.0, float(np.float32(80 * s_w)), "none", 0, False)
+    assert H.conv_kernel(P, 1, 16, 24).chunks == 1 and total > 2 ** 24
+    P.w_i8[P.w_i8 != 0] = 127
+    P.w_f16[P.w_f16 != 0] = 127.0
+    P.codes_changed()
+    assert H.conv_kernel(P, 1, 16, 24).kernel == H.KERNEL_GENERAL
+    y = H.conv2d_i8(dev(x), P)
+    H.sync_status()
+    p = O.prepare_layer(w, b, L.form, L.hb_in, L.hb_out, 1.0, float(np.float32(80 * s_w)), "none", 0, False, L.stride, L.pad)
+    p.w_int = np.full_like(p.w_int, 127)
+    ref = O.conv_layer(x, p)
+    assert np.array_equal(y.cpu().numpy(), ref) and len(np.unique(ref)) > 3

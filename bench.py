@@ -278,13 +278,17 @@ def run_layer_mode(args, cfg, scales):
     raise SystemExit(f"unknown layer {args.layer}")
 
 
+CONV_SOURCES = ("hatq_api.cu", "hatq_conv.cu", "hatq_conv_lean.cu", "hatq_conv_lean_pieces.cu", "hatq_conv_pieces.cu",
+                "hatq_conv_win.cu", "hatq_internal.h", "hatq_launch.h", "hatq_lean.h", "hatq_tc.h")
+
+
 def conv_source_sha() -> str:
-    """sha256 prefix of the conv kernels' sources (kernel files and the
-    device-helper headers they include), the key of committed counter captures."""
+    """sha256 prefix of the sources that decide what a convolution runs (kernel files, the headers
+    they include, and the planning that chooses kernel, tiles, chunks and stages), the key of committed
+    counter captures."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("hatq_conv.cu", "hatq_conv_lean.cu", "hatq_conv_lean_pieces.cu", "hatq_conv_pieces.cu", "hatq_conv_win.cu", "hatq_lean.h",
-              "hatq_tc.h"):
+    for f in CONV_SOURCES:
         h.update(open(os.path.join(ROOT, "paper_2608_01653_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 

@@ -30,3 +30,20 @@ def test_reference_arm_other_ranks_exit_quietly():
     r = subprocess.run([sys.executable, "bench.py", "--impl", "reference", "--steps", "1", "--warmup", "0"],
                        cwd=ROOT, capture_output=True, text=True, timeout=600, env={**os.environ, "RANK": "1"})
     assert r.returncode == 0 and r.stdout.strip() == ""
+
+
+def test_traffic_key_covers_what_decides_the_kernels():
+    """The hash that keeps a committed DRAM capture with its sources: every convolution source, what it
+    includes, and the planning (choice of kernel, tiles, chunks and stages) in hatq_api.cu."""
+    import re
+
+    import bench
+    csrc = os.path.join(ROOT, "paper_2608_01653_gb300", "csrc")
+    need, todo = set(), {f for f in os.listdir(csrc) if f.startswith("hatq_conv")} | {"hatq_api.cu"}
+    while todo:
+        f = todo.pop()
+        need.add(f)
+        if f != "hatq_api.cu":
+            inc = re.findall(r'#include "(\w+\.\w+)"', open(os.path.join(csrc, f)).read())
+            todo |= {i for i in inc if os.path.exists(os.path.join(csrc, i))} - need
+    assert set(bench.CONV_SOURCES) == need

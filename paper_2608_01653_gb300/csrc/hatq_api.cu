@@ -909,8 +909,11 @@ struct OutGrid {
 // returns the shared memory it needs, or 0. Plain INT8 layers (the caller checks
 // the options) with at most 64 taps, whose windows and at least two weight stages
 // fit shared memory and whose output is not mostly the padding of its 8 x 16-pixel
-// tiles: `area` is the pixels of the other kernel's tiling, and up to a quarter
-// more is still the better bargain (a 64-row conversion saved per tap).
+// tiles: `area` is the pixels of the other kernel's tiling, and up to a quarter more
+// is taken. Time of this kernel over the other's for the same layer (3x3 64 -> 192,
+// 5x5 s2 192 -> 192, 3x3 320 -> 640, 224 -> 128 and 128 -> 32; 32 to 192 images of
+// 17 x 12 to 64 x 64 outputs): equal area 0.58-0.88, 1.20 of it 0.69-0.88, 1.33
+// 0.74-1.08, twice 1.02-1.29.
 int win_plan(const hatq_conv_desc &d, const Geometry &g, const hatq_prepared &L, const OutGrid *og, int n, int ho, int wo,
              long long area, hatq::WinArgs &a, int &epi) {
     if (L.chunk_units < 1 || d.kh * d.kw > 64 || d.kh * d.kw < 2) return 0;
@@ -973,6 +976,11 @@ int win_plan(const hatq_conv_desc &d, const Geometry &g, const hatq_prepared &L,
     // A weight stage holds the taps of one kernel row (a wait, a commit and the counters per row
     // instead of per tap) where at least six blocks fit in two stages or more, preferably beside two
     // INT8 window buffers; else single blocks, with the second window buffer where four stages remain.
+    // Measured with at least 4 blocks in flight / 6 / single blocks always, us: 5x5 s2 192 -> 192 on
+    // 2 x 1080 x 1920 1225 / 982 / 1012, 3x3 320 -> 640 on 8 x 135 x 240 685 / 685 / 811, 640 -> 640 on
+    // 4 x 135 x 240 612 / 612 / 743, 224 -> 128 137 / 137 / 147, 128 -> 32 51 / 51 / 67. The rule loses
+    // where only two stages of part of a row fit: 5x5 192 -> 192 stride 1 on 2 x 270 x 480 272 against
+    // 248 single, 7x7 64 -> 192 189 against 158.
     const int row_taps = a.pairs ? 4 : (d.kw + a.par - 1) / a.par;
     a.stages = 0;
     for (int n8 = 2; n8 >= 1 && !a.stages; --n8)

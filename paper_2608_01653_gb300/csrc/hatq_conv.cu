@@ -371,9 +371,11 @@ __device__ __forceinline__ void epi_split128(const EpiCtx &e, const ConvArgs &a,
 // (groups of 128 columns with the warp of the same rows in the other
 // warpgroup): the region is released as soon as the last columns arrived, and the
 // codes leave as one TMA store per warp and group from a swizzled staging buffer.
-// Bound: instruction issue. Groups of 32 and 64 columns take the fp32 estimate with exact
-// rows where it is not certain (12 operations per value of a WH(64) -> ReLU -> DH(64)
-// transition, 38 in 64-bit integers), groups of 128 the integers.
+// Groups of 32 and 64 columns take the fp32 estimate with exact rows where it is not certain
+// (12 operations per value of a WH(64) -> ReLU -> DH(64) transition, 38 in 64-bit integers),
+// groups of 128 the integers. Bound: the small-channel layer 5x5 s2 3 -> 192 issues 25
+// instructions per value in all at 48 % of the issue rate, with two epilogue warps per
+// scheduler to hide the latency of tensor memory, barriers and instruction fetch.
 // (The pieces are in hatq_lean.h.)
 
 // ------------------------------------------------------------------ kernel
@@ -502,7 +504,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
 
     // Register split by warpgroup (launch: 512 x 128 = 65536): warpgroup 0
-    // (producer, MMA issuer, two idle warps) 40, warpgroup 3 (converters) 72,
+    // (two producers, MMA issuer, an idle warp) 40, warpgroup 3 (converters) 72,
     // warpgroups 1-2 (epilogue) 200: 128 x (40 + 72) + 256 x 200 = 65536, and
     // per scheduler (one warp of each warpgroup) 32 x (40 + 72 + 2 x 200) = 16384.
     const int SA = a.a_slots;

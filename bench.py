@@ -278,7 +278,8 @@ def run_layer_mode(args, cfg, scales):
     raise SystemExit(f"unknown layer {args.layer}")
 
 
-CONV_SOURCES = ("hatq_api.cu", "hatq_conv.cu", "hatq_conv_lean.cu", "hatq_conv_lean_pieces.cu", "hatq_conv_pieces.cu",
+CONV_SOURCES = ("hatq_api.cu", "hatq_conv.cu", "hatq_conv_f32.cu", "hatq_conv_f32_pieces.cu", "hatq_conv_general.cu",
+                "hatq_conv_general_pieces.cu", "hatq_conv_lean.cu", "hatq_conv_lean_pieces.cu", "hatq_conv_pieces.cu",
                 "hatq_conv_win.cu", "hatq_internal.h", "hatq_launch.h", "hatq_lean.h", "hatq_tc.h")
 
 

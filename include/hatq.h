@@ -296,7 +296,7 @@ int hatq_layer_launches(int x_kind, float s_in, const hatq_prepared *L);
  * one that the call's own checks of layer and size give. */
 typedef enum {
     HATQ_KERNEL_NONE = 0,     /* empty batch */
-    HATQ_KERNEL_GENERAL = 1,  /* conv_kernel with every option */
+    HATQ_KERNEL_GENERAL = 1,  /* conv_kernel: float32 or fp16 output, general transitions, several chunks, ... */
     HATQ_KERNEL_LEAN = 2,     /* conv_kernel for plain INT8 codes of one exact chunk */
     HATQ_KERNEL_WINDOW = 3    /* conv_win_kernel */
 } hatq_kernel;

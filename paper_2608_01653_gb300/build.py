@@ -19,7 +19,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "libhatq.so")
-SOURCES = ["hatq_conv_win.cu", "hatq_conv_lean.cu", "hatq_conv_lean_pieces.cu", "hatq_conv.cu", "hatq_conv_pieces.cu", "hatq_api.cu",
+SOURCES = ["hatq_conv_win.cu", "hatq_conv_lean.cu", "hatq_conv_lean_pieces.cu", "hatq_conv.cu", "hatq_conv_pieces.cu", "hatq_conv_f32.cu",
+           "hatq_conv_f32_pieces.cu", "hatq_conv_general.cu", "hatq_conv_general_pieces.cu", "hatq_api.cu",
            "hatq_fwht.cu", "hatq_gdn.cu", "hatq_noalloc.cu", "hatq_profile.cu"]
 HEADERS = [os.path.join(CSRC, "hatq_internal.h"), os.path.join(CSRC, "hatq_tc.h"),
            os.path.join(CSRC, "hatq_launch.h"), os.path.join(CSRC, "hatq_lean.h"), os.path.join(INCLUDE, "hatq.h")]

@@ -36,19 +36,28 @@
 // Every mbarrier wait is bounded: on expiry the kernel records an error word,
 // raises a CTA-wide abort flag and unwinds (waiting, again bounded, for its own
 // MMAs and copies) before freeing TMEM.
-// This file is compiled four times: as itself (the kernels with every option,
-// the launcher, the self test) and through hatq_conv_pieces.cu (activation
-// blocks arriving as two 32-channel boxes), hatq_conv_lean.cu and
-// hatq_conv_lean_pieces.cu (the lean kernels: INT8 codes of one exact chunk per
-// tile without further options, one instantiation per transform group). Four
-// translation units build in parallel, and no kernel carries code that its
-// layers never run: with every option in one kernel, each change of any branch
-// changed the code generated for all of them (ga1 between 7.6 and 8.9 ms).
+// This file is compiled eight times: as itself (the kernels for INT8 codes with
+// fp16 storage, sub-pixel order or several chunks, the launcher, the self test),
+// through hatq_conv_f32.cu (float32 output), hatq_conv_general.cu (the general
+// transition) and hatq_conv_lean.cu (the lean kernels: INT8 codes of one exact
+// chunk per tile without further options, one instantiation per transform group),
+// and each through its *_pieces.cu (activation blocks arriving as two 32-channel
+// boxes). The translation units build in parallel, and no kernel carries code that
+// its layers never run: with every option in one kernel, each change of any branch
+// changed the code generated for all of them. On 2 x 270 x 480, one kernel / each
+// its own: 1x1 320 -> 320 float32 176 / 164 us, 3x3 192 -> 192 float32 222 / 211 and
+// to fp16 codes 214 / 196, 1x1 192 -> 192 SiLU 440 / 436.
 #ifndef HATQ_CONV_PIECES
 #define HATQ_CONV_PIECES 0
 #endif
 #ifndef HATQ_CONV_LEAN
 #define HATQ_CONV_LEAN 0
+#endif
+#ifndef HATQ_CONV_F32
+#define HATQ_CONV_F32 0
+#endif
+#ifndef HATQ_CONV_GENERAL
+#define HATQ_CONV_GENERAL 0
 #endif
 
 #include <cuda_fp16.h>
@@ -195,9 +204,9 @@ __device__ __forceinline__ long long relu(long long v) { return ((int)(v >> 32))
 __device__ __forceinline__ float relu(float v) { return fmaxf(v, 0.f); }
 
 // One group of G <= 64 columns held entirely in registers.
-template <int G>
+template <int G, int OUT>
 __device__ __forceinline__ void epi_group(const EpiCtx &e, const ConvArgs &a, int col) {
-    if (a.general) {
+    if constexpr (OUT == 2) {
         // Sec. general nonlinearities: z = clamp(round(H~_out (M_out (.) a) / 2^n_out)),
         // u = phi_int(z), x = clamp(round(H~_next (M_in u) / 2^n_in)); |H~_next u| <= 127 * 64
         // fits int32 and M_in is one scalar, so the next transform runs on u itself
@@ -217,9 +226,7 @@ __device__ __forceinline__ void epi_group(const EpiCtx &e, const ConvArgs &a, in
 #pragma unroll
         for (int i = 0; i < G; ++i) x[i] = requant8_any(a.mult_in * (long long)u[i], a.shift_in);
         store_codes_i32<G>(e.row, col, x);
-        return;
-    }
-    if (!a.out_f32) {
+    } else if constexpr (OUT == 0) {
         long long t[G];
 #pragma unroll
         for (int q = 0; q < G / 16; ++q) {
@@ -267,10 +274,11 @@ __device__ __forceinline__ void epi_group(const EpiCtx &e, const ConvArgs &a, in
 // abort (ok false: the values are then meaningless but stay in this CTA's
 // tensor and shared memory, and the copy-out is skipped), so the named
 // barrier always completes.
+template <bool F32>
 __device__ __forceinline__ void epi_split128(const EpiCtx &e, const ConvArgs &a, int wg, bool ok, uint8_t *xbuf,
                                              int row) {
     const int half = 64 * wg;
-    if (a.out_f32) {
+    if constexpr (F32) {
         if (!ok) return;
         float p[64];
         if (a.hb_out == 128) {
@@ -303,7 +311,7 @@ __device__ __forceinline__ void epi_split128(const EpiCtx &e, const ConvArgs &a,
         }
         store_f32<64>(e.gout, half, p);
         return;
-    }
+    } else {
     long long p[64];
     if (a.hb_out == 128) {
 #pragma unroll
@@ -361,6 +369,7 @@ __device__ __forceinline__ void epi_split128(const EpiCtx &e, const ConvArgs &a,
         fwht<64>(p, a.hb_next);
     }
     store_codes<64>(a, e.row, half, p);
+    }
 }
 
 // ------------------------------------------------------------------ lean epilogue
@@ -391,13 +400,16 @@ __device__ __forceinline__ void epi_split128(const EpiCtx &e, const ConvArgs &a,
 // SUB: 64-wide reduction blocks per pipeline stage (1, 2 or 4). PIECES: the
 // activation blocks arrive as two 32-channel boxes (c % 64 == 32); a separate
 // instantiation, so that the other layers' kernels carry none of its code.
-// LEAN: 0 the epilogue with every option, else the lean epilogue's group.
+// LEAN: 0 the epilogue for INT8 codes with their other options, 1 the one for float32 output (also of
+// affine operands), 2 the one for the general transition, else the lean epilogue's group.
 template <int SUB, bool PIECES, int LEAN>
 __global__ void __launch_bounds__(kThreads, 1)
     conv_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const __grid_constant__ CUtensorMap tmY, const __grid_constant__ ConvArgs a) {
+    constexpr bool kLean = LEAN >= 32, kF32 = LEAN == 1, kGeneral = LEAN == 2;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    const bool affine = kF32 && a.affine;            // int16 operand codes
     const int S = a.stages;
     uint8_t *staging = smem + (size_t)S * a.stage_bytes;
     uint8_t *bar_area = staging + (size_t)a.staging_bytes;
@@ -418,7 +430,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     // A failure already recorded by this launch (or an earlier, unread one)
     // ends every CTA that has not started, so a fault cannot serialize waits.
     // One thread reads the word so the whole CTA takes the same decision.
-    pdl_enter();
+    // (Float32 layers mostly follow a kernel without an early start, where its cost shows: a 1x1
+    // 128 -> 128 layer with its input transform on 32 x 48 takes 11.7 us, with it 12.6.)
+    if constexpr (!kF32) pdl_enter();
     __shared__ int s_skip;
     if (threadIdx.x == 0) s_skip = *reinterpret_cast<volatile int *>(a.err);
     __syncthreads();
@@ -468,21 +482,24 @@ __global__ void __launch_bounds__(kThreads, 1)
     int8_t *lut_s = reinterpret_cast<int8_t *>(bar_area + a.lut_off);
     if constexpr (LEAN == 32 || LEAN == 64) {
         stage_quick(reinterpret_cast<float *>(cb), a.mult, a.b_int, a.co, a.shift);
-    } else if constexpr (LEAN != 0) {
+    } else if constexpr (kLean) {
         for (int c = threadIdx.x; c < a.co; c += kThreads) {
             const int m = a.mult[c];
             mbs[c] = (long long)m * a.b_int[c];
             mults[c] = m;
         }
     } else {
-        const float s_aff = a.affine ? *a.affine_s : 0.f;
+        const float s_aff = affine ? *a.affine_s : 0.f;
         for (int c = threadIdx.x; c < a.co; c += kThreads) {
             cb[c] = a.b_int[c];
-            cb[a.co + c] = a.mult[c];
-            reinterpret_cast<float *>(cb)[2 * a.co + c] = a.affine ? s_aff * a.s_w[c] * a.inv_gamma : a.deq[c];
-            reinterpret_cast<float *>(cb)[3 * a.co + c] = a.affine ? a.deq[c] : 0.f;
+            if constexpr (!kF32) {
+                cb[a.co + c] = a.mult[c];
+            } else {
+                reinterpret_cast<float *>(cb)[2 * a.co + c] = affine ? s_aff * a.s_w[c] * a.inv_gamma : a.deq[c];
+                reinterpret_cast<float *>(cb)[3 * a.co + c] = affine ? a.deq[c] : 0.f;
+            }
         }
-        if (a.general)
+        if constexpr (kGeneral)
             for (int i = threadIdx.x; i < 256; i += kThreads) lut_s[i] = a.lut[i];
     }
     tc_fence_before();
@@ -720,7 +737,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // row m of a 64-wide INT8 box (64 bytes, 16-byte chunks permuted by the
             // 64-byte swizzle) -> 32 columns of fp16 pairs
             auto convert_row = [&](const uint8_t *raw, uint32_t (&h)[32]) {
-                if (a.affine) {
+                if (affine) {
                     // row m of a 64-wide int16 box (128 bytes, 16-byte chunks permuted by the 128-byte
                     // swizzle), or of two 32-wide boxes (64-byte rows, 64-byte swizzle)
                     const int sw = PIECES ? (m >> 1) & 3 : m & 7;
@@ -758,7 +775,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             };
             // bytes of one operand row of a 64-wide block (of one of its 32-wide boxes with a.half)
-            const int row_in = ((a.affine || a.a_f16) ? 128 : 64) >> (PIECES ? 1 : 0);
+            const int row_in = ((affine || a.a_f16) ? 128 : 64) >> (PIECES ? 1 : 0);
             for (int j = 0; j < my_tiles && ok; ++j) {
                 for (int kb0 = 0; kb0 < a.num_kb; kb0 += SUB) {
                     const int nsub = min(SUB, a.num_kb - kb0);
@@ -881,7 +898,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (a.win_tma && ok) mbar_arrive(win_empty(j & 1));   // this thread's reads of the window are done
             }
         }
-    } else if constexpr (LEAN != 0) {
+    } else if constexpr (kLean) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 200;" ::: "memory");
         // ---------------------------------------------------------- lean epilogue (warps 4-11)
         const int wg = (warp - 4) >> 2;            // 0 or 1
@@ -959,9 +976,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int wg = (warp - 4) >> 2;            // 0 or 1
         const int quad = warp & 3;                 // TMEM lane quadrant this warp may access
         const int row = quad * 32 + lane;
-        const int et = threadIdx.x - 128 - 128 * wg;   // 0..127 within the warpgroup
-        const int esz = a.out_f32 ? 4 : 1;
-        const int row_bytes = a.n_t * esz;
+        [[maybe_unused]] const int et = threadIdx.x - 128 - 128 * wg;   // 0..127 within the warpgroup
         uint8_t *stage_tile = staging + (size_t)(nbuf == 2 ? wg : 0) * kTileM * a.row_stride;
         const int G = max(32, max(a.hb_out, a.hb_next));
         uint32_t part[4][32];                      // nbuf == 1: int32 partial sums of column groups 2k + wg
@@ -1038,35 +1053,36 @@ __global__ void __launch_bounds__(kThreads, 1)
                 e.lut = lut_s;
                 e.row = stage_tile + (size_t)row * a.row_stride;
                 e.gout = nullptr;
-                if (a.out_f32) {
+                if constexpr (kF32) {
                     const int oy = ho0 + row / a.tw, ox = wo0 + row % a.tw;
                     if (oy < a.ho && ox < a.wo)
                         e.gout = static_cast<float *>(a.y) + (((long long)img * a.y_h + oy * a.ostride + a.ooy) * a.y_w +
                                                               ox * a.ostride + a.oox) * a.co + n0;
                 }
-                if (G == 128) {
+                if (!kGeneral && G == 128) {
                     // n_t == 128, nbuf == 1: the warpgroups share the group; the shared-memory
                     // output tile is free until the codes are stored and serves as the exchange buffer
-                    epi_split128(e, a, wg, ok, stage_tile, row);
+                    epi_split128<kF32>(e, a, wg, ok, stage_tile, row);
                 } else if (ok) {
                     int gi = 0;
                     for (int col = 0; col < a.n_t; col += G, ++gi) {
                         if (nbuf == 1 && (gi & 1) != wg) continue;
-                        if (G == 32) epi_group<32>(e, a, col);
-                        else epi_group<64>(e, a, col);
+                        if (G == 32) epi_group<32, LEAN>(e, a, col);
+                        else epi_group<64, LEAN>(e, a, col);
                     }
                 }
                 tc_fence_before();
                 mbar_arrive(acc_empty(reg));           // TMEM reads of this region are complete
+                if constexpr (kF32) continue;          // stored directly
                 // coalesced copy-out: consecutive threads write consecutive 16-byte chunks
                 const int nthr = nbuf == 2 ? 128 : 256;
                 const int tid = nbuf == 2 ? et : et + 128 * wg;
                 if (nbuf == 2) asm volatile("bar.sync %0, 128;" ::"r"(2 + wg) : "memory");
                 else asm volatile("bar.sync 4, 256;" ::: "memory");
                 // a half-warp per tile row (at most 14 chunks of 16 bytes), so no division per chunk
-                const int cpr = row_bytes >> 4;
+                const int cpr = a.n_t >> 4;
                 const int c = lane & 15;
-                for (int r = (tid >> 5) * 2 + (lane >> 4); ok && !a.out_f32 && r < kTileM; r += nthr >> 4) {
+                for (int r = (tid >> 5) * 2 + (lane >> 4); ok && r < kTileM; r += nthr >> 4) {
                     const int oy = ho0 + (r >> a.tw_log2), ox = wo0 + (r & (a.tw - 1));
                     if (c < cpr && oy < a.ho && ox < a.wo) {
                         const int gy = oy * a.ostride + a.ooy, gx = ox * a.ostride + a.oox;
@@ -1121,7 +1137,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
-#if !HATQ_CONV_PIECES && !HATQ_CONV_LEAN
+#if !HATQ_CONV_PIECES && !HATQ_CONV_LEAN && !HATQ_CONV_F32 && !HATQ_CONV_GENERAL
 // Failure-detection self test: one thread waits, through the pipeline's
 // bounded wait, on an mbarrier nothing arrives at; the wait expires after
 // `limit` cycles and records kErrWaitTimeout in the error word.
@@ -1150,6 +1166,14 @@ ConvKernelFn conv_lean_pieces_kernel(int sub, int g) {
 ConvKernelFn conv_lean_kernel(int sub, int g) {
     return g == 128 ? HATQ_SUB_KERNEL(false, 128) : (g == 64 ? HATQ_SUB_KERNEL(false, 64) : HATQ_SUB_KERNEL(false, 32));
 }
+#elif HATQ_CONV_F32 && HATQ_CONV_PIECES
+ConvKernelFn conv_f32_pieces_kernel(int sub) { return HATQ_SUB_KERNEL(true, 1); }
+#elif HATQ_CONV_F32
+ConvKernelFn conv_f32_kernel(int sub) { return HATQ_SUB_KERNEL(false, 1); }
+#elif HATQ_CONV_GENERAL && HATQ_CONV_PIECES
+ConvKernelFn conv_general_pieces_kernel(int sub) { return HATQ_SUB_KERNEL(true, 2); }
+#elif HATQ_CONV_GENERAL
+ConvKernelFn conv_general_kernel(int sub) { return HATQ_SUB_KERNEL(false, 2); }
 #elif HATQ_CONV_PIECES
 ConvKernelFn conv_pieces_kernel(int sub) { return HATQ_SUB_KERNEL(true, 0); }
 #else
@@ -1165,11 +1189,13 @@ cudaError_t launch_conv(const CUtensorMap &tmA, const CUtensorMap &tmB, const CU
     if ((a.sub != 1 && a.sub != 2 && a.sub != 4) || (a.gather && a.sub != 1) || a.chunk_kb % a.sub ||
         (a.half && (a.gather || a.a_f16 || a.cin_h < 1)) || (a.lean && a.num_kb > a.chunk_kb))
         return cudaErrorInvalidValue;   // gathered tiles: one block per stage
-    const int fam = a.lean ? (a.group == 128 ? 3 : (a.group == 64 ? 2 : 1)) : 0;
+    const int fam = a.lean ? (a.group == 128 ? 3 : (a.group == 64 ? 2 : 1)) : (a.out_f32 ? 4 : (a.general ? 5 : 0));
     const int v = (a.sub == 4 ? 2 : (a.sub == 2 ? 1 : 0)) + (a.half ? 3 : 0) + 6 * fam;
-    const ConvKernelFn kern = a.lean ? (a.half ? conv_lean_pieces_kernel(a.sub, a.group) : conv_lean_kernel(a.sub, a.group))
-                                     : (a.half ? conv_pieces_kernel(a.sub) : conv_full_kernel(a.sub));
-    static SmemOptIn opt_in[24];
+    const ConvKernelFn kern = a.lean      ? (a.half ? conv_lean_pieces_kernel(a.sub, a.group) : conv_lean_kernel(a.sub, a.group))
+                              : a.out_f32 ? (a.half ? conv_f32_pieces_kernel(a.sub) : conv_f32_kernel(a.sub))
+                              : a.general ? (a.half ? conv_general_pieces_kernel(a.sub) : conv_general_kernel(a.sub))
+                                          : (a.half ? conv_pieces_kernel(a.sub) : conv_full_kernel(a.sub));
+    static SmemOptIn opt_in[36];
     int dev = 0, sms = 0;
     cudaError_t e;
     if ((e = current_device(&dev)) != cudaSuccess || (e = opt_in[v].set(dev, reinterpret_cast<const void *>(kern))) != cudaSuccess ||
@@ -1185,7 +1211,7 @@ cudaError_t launch_conv(const CUtensorMap &tmA, const CUtensorMap &tmB, const CU
     cfg.dynamicSmemBytes = smem_bytes;
     cfg.stream = s;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = a.out_f32 ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmY, a);
 }
 

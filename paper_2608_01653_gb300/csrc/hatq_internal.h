@@ -135,13 +135,17 @@ struct ConvArgs {
     int8_t lut[256];
 };
 
-// The convolution kernels, by blocks per pipeline stage (sub): the one with
-// every option, and the lean ones for INT8 codes without options (a.lean, group
-// g = 32, 64 or 128); "pieces" for layers whose activation blocks arrive as two
-// 32-channel boxes (a.half). Each family is its own translation unit.
+// The convolution kernels, by blocks per pipeline stage (sub): for INT8 codes with
+// their options, for float32 output, for the general transition, and the lean ones for
+// INT8 codes without options (a.lean, group g = 32, 64 or 128); "pieces" for layers whose activation blocks
+// arrive as two 32-channel boxes (a.half). Each family is its own translation unit.
 using ConvKernelFn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const ConvArgs);
 ConvKernelFn conv_full_kernel(int sub);
 ConvKernelFn conv_pieces_kernel(int sub);
+ConvKernelFn conv_f32_kernel(int sub);
+ConvKernelFn conv_f32_pieces_kernel(int sub);
+ConvKernelFn conv_general_kernel(int sub);
+ConvKernelFn conv_general_pieces_kernel(int sub);
 ConvKernelFn conv_lean_kernel(int sub, int g);
 ConvKernelFn conv_lean_pieces_kernel(int sub, int g);
 // tmY: output box of one epilogue warp (lean kernels)

@@ -29,6 +29,8 @@ CASES = [
     ("wh3x3_gelu_next64", C.layer("a", 64, 128, 3, 1, 1, "WH", "gelu", hb_out=64), (1, 11, 17), 64),
     ("dh5x5s2_gelu_next32_drain", C.layer("a", 192, 192, 5, 2, 2, "DH", "gelu", hb_in=64), (1, 19, 37), 32),
     ("wh5x5s2_c3_silu_gather", C.layer("a", 3, 64, 5, 2, 2, "WH", "silu", hb_out=32), (2, 30, 41), 64),
+    ("dh3x3_c96_gelu_pieces", C.layer("a", 96, 64, 3, 1, 1, "DH", "gelu", hb_in=32), (2, 33, 26), 64),      # two 32-channel boxes
+    ("dh1x1_c160_silu_pieces", C.layer("a", 160, 96, 1, 1, 0, "DH", "silu", hb_in=32), (2, 9, 21), 32),
     ("dh1x1_silu_ragged", C.layer("a", 128, 224, 1, 1, 0, "DH", "silu", hb_in=128), (3, 5, 7), 32),
 ]
 

@@ -55,6 +55,7 @@ int *err_word() {
 }
 
 constexpr int kTileRows = 128;
+constexpr int kSms = 152;        // a GB300's
 
 bool pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -1118,11 +1119,19 @@ hatq_status conv_plan(int n, int h, int w, const hatq_prepared *L, const OutGrid
     // the columns, keeping int32 partials in registers (nbuf = 1). A
     // 128-column transform group (n_t = 128) is always shared by both
     // warpgroups, one half each (nbuf = 1).
-    const bool drains = a.num_kb > a.chunk_kb;
     a.buf_cols = a.n_t;
     const bool general = L->act == HATQ_ACT_SILU || L->act == HATQ_ACT_GELU;
     // the lean kernels: INT8 codes of one exact chunk per tile, no further option
     const bool plain = !general && !L->out_f32 && !a.affine && !a.a_f16 && !a.out_f16 && !a.d2s;
+    // With the int64 epilogue and few tiles per CTA, both warpgroups at each tile (as with drains) are
+    // worth more than the longer chunk, which they take in turns: with one tile, and for a cheap
+    // transition of two chunks with up to eight. Drains / one chunk, us, at 152, 156, 1080 and 2400 tiles:
+    // 3x3 192 -> 192 with fp16 codes (27 blocks) 21 / 26, 32 / 37, 106 / 111, 217 / 216, with SiLU 54 / 70,
+    // 95 / 70, 356 / 308, 725 / 668; 5x5 s2 192 -> 192 with fp16 codes (75 blocks) 35 / 34, 58 / 57,
+    // 221 / 211, 435 / 413.
+    const int few = !general && a.num_kb <= 2 * kChunkAny ? 8 * kSms : kSms;
+    if (!plain && !L->out_f32 && a.num_tiles <= few && a.chunk_kb > kChunkAny) a.chunk_kb = kChunkAny;
+    const bool drains = a.num_kb > a.chunk_kb;
     a.group = g.G;
     a.nbuf = (drains || g.G == 128) ? 1 : 2;
     a.tmem_cols = 512;

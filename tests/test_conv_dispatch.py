@@ -57,6 +57,19 @@ def test_kernel_of_a_layer(kw, size, expect):
     assert route(struct(**kw), *size) == expect
 
 
+@pytest.mark.parametrize("act,k,counts", [("silu", 3, {1: 2, 12: 2, 13: 1, 102: 1}), ("relu", 3, {1: 2, 13: 2, 101: 2, 102: 1}),
+                                          ("relu", 5, {1: 5, 12: 5, 13: 1})])
+def test_few_tiles_per_cta_keep_both_warpgroups(act, k, counts):
+    """The int64 epilogue of one long chunk is one warpgroup's; with few tiles per CTA the general chunk
+    length stays, and both warpgroups drain and finish a tile."""
+    s = struct(192, 192, k, hb_next=64, act=act, chunk_units=0)
+    s.out_f16 = int(act == "relu")
+    for n, chunks in counts.items():                                 # 12 tiles of 16 x 96 pixels per image
+        i = H.conv_kernel(s, n, 16, 96)
+        assert (i.kernel, i.chunks) == (G, chunks), n
+    assert H.conv_kernel(struct(192, 192, out_f32=True), 1, 16, 96).chunks == 1
+
+
 @pytest.mark.parametrize("c_out,r,size,expect", [(256, 2, (3, 64, 40), (WIN, 3064, 0)), (256, 2, (3, 33, 26), (G, 0, 0)),
                                                  (64, 2, (3, 64, 40), (WIN, 3064, 0)), (288, 3, (3, 64, 40), None)])
 def test_kernel_of_a_subpixel_layer(c_out, r, size, expect):

@@ -126,3 +126,20 @@ def test_chain_with_f16_operands_equals_int8_chain(H):
     assert f16[0].dtype == torch.float16 and f16[1].dtype == torch.float16
     for a, b in zip(base, f16):
         assert np.array_equal(a.cpu().numpy().astype(np.int64), b.cpu().numpy().astype(np.int64))
+
+
+@pytest.mark.parametrize("n,chunks", [(3, 2), (40, 2), (180, 1)])
+def test_fp16_codes_on_both_sides_of_the_chunk_rule(H, n, chunks):
+    """Few tiles are drained by both epilogue warpgroups, many run one chunk each in turn. The images
+    repeat two base ones."""
+    L = C.layer("a", 192, 192, 3, 1, 1, "DH", "relu", hb_in=64)
+    wts, b = I.weights(192, 3, 3, 192, seed=5), I.bias(192, seed=6)
+    base = I.activations_i8((2, 21, 40, 192), seed=7, s_in=0.05)
+    P = H.prepare_weights(H.desc_from_spec(L), wts, b, 0.05, 0.08, L.act, 64, False)
+    H.set_operand_format(P, False, True)
+    assert H.conv_kernel(P, n, 21, 40).chunks == chunks
+    pick = np.random.default_rng(n).integers(0, 2, n)
+    y = H.conv2d_i8(dev(base[pick]), P)
+    H.sync_status()
+    ref = O.conv_layer(base, O.prepare_layer(wts, b, "DH", 64, 0, 0.05, 0.08, L.act, 64, False, 1, 1))
+    assert np.array_equal(y.cpu().numpy(), ref[pick].astype(np.float16)) and len(np.unique(ref)) > 20

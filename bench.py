@@ -784,7 +784,7 @@ def main():
         "warmup": max(3, args.warmup), "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "int8",
         "arithmetic": "INT8 codes as exact fp16 tensor-core operands, fp32 chunk sums below 2^24, int32 totals, "
-                      "int64 requantization",
+                      "exact requantization (fp32 estimate with a proven error bound, int64 where it does not decide)",
         "data": "synthetic (seeded LIC-shaped inputs, random-init weights)",
         "effective_tops": world * 2 * macs_step / (ms / 1000.0) / 1e12,
         "config": {"workload": workload_name(cfg), "global_batch": world * images_step,

@@ -1020,7 +1020,7 @@ int win_plan(const hatq_conv_desc &d, const Geometry &g, const hatq_prepared &L,
 // buffers of the call) and its shared memory. Host only.
 struct ConvPlan {
     Geometry g;
-    hatq::ConvArgs a;        // conv_kernel, lean or with every option
+    hatq::ConvArgs a;        // conv_kernel, lean or with options
     int smem_bytes;
     hatq::WinArgs wa;        // conv_win_kernel, taken where win_smem is not 0
     int epi, win_smem;

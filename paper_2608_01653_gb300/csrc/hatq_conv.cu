@@ -409,7 +409,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr bool kLean = LEAN >= 32, kF32 = LEAN == 1, kGeneral = LEAN == 2;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    const bool affine = kF32 && a.affine;            // int16 operand codes
+    // int16 operand codes (never in the lean kernels, which keep the test and with it the code generated
+    // for them so far)
+    const bool affine = (kF32 || kLean) && a.affine;
     const int S = a.stages;
     uint8_t *staging = smem + (size_t)S * a.stage_bytes;
     uint8_t *bar_area = staging + (size_t)a.staging_bytes;
@@ -703,6 +705,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const long long t0 = clock64();
         while (!mbar_try_wait(mma_done, 0) && clock64() - t0 < kWaitLimitCycles) {
         }
+        __syncwarp();                                // (the barrier and the release of TMEM take the warp whole)
     }
     } else if (warp >= 12) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 72;" ::: "memory");

@@ -500,19 +500,22 @@ __global__ void __launch_bounds__(kThreads, 1)
                     tc_fence_before();
                     release(reg);
                 }
+                if (ng == 0) {                             // n_t = 32: the other warpgroup has the tile
+                    // (released only after a wait like every region: an arrival ahead of the chunk would
+                    // let two of this warp's stand for one of a warp that still reads the region)
+                    const int gl = j * a.nch + a.nch - 1, rl = gl & (kRegions - 1);
+                    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(acc_full(rl), (gl >> kRegLog) & 1, abort_flag, a.err));
+                    tc_fence_after();
+                    tc_fence_before();
+                    release(rl);
+                    continue;
+                }
                 // the last chunk's region; with 2128 both chunks of the tile still sit in regions of their own
                 const int gc = j * a.nch + a.nch - 1, reg = gc & (kRegions - 1), reg0 = (gc - 1) & (kRegions - 1);
                 if constexpr (kTwo)
                     if (ok) ok = __all_sync(0xffffffffu, mbar_wait(acc_full(reg0), ((gc - 1) >> kRegLog) & 1, abort_flag, a.err));
                 if (ok) ok = __all_sync(0xffffffffu, mbar_wait(acc_full(reg), (gc >> kRegLog) & 1, abort_flag, a.err));
                 tc_fence_after();
-                if (ng == 0) {                             // n_t = 32: the other warpgroup has the tile
-                    // (released only after its wait like any other: an arrival ahead of the chunk would
-                    // let two of this warp's stand for one of a warp that still reads the region)
-                    tc_fence_before();
-                    release(reg);
-                    continue;
-                }
                 // one copy of this code for all groups: unrolled it would not fit the instruction cache
 #pragma unroll 1
                 for (int gr = 0; gr < ng; ++gr) {

@@ -705,7 +705,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         const long long t0 = clock64();
         while (!mbar_try_wait(mma_done, 0) && clock64() - t0 < kWaitLimitCycles) {
         }
-        __syncwarp();                                // (the barrier and the release of TMEM take the warp whole)
     }
     } else if (warp >= 12) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 72;" ::: "memory");

@@ -36,7 +36,7 @@
 //                CTA), one TMA store of 64 bytes x 32 rows per warp
 // No warp waits for another but through the barriers of tiles, limbs and accumulators;
 // every wait is bounded.
-// Bound: 32 instructions per value, issued at 47 % of the rate (waits on tensor and shared
+// Bound: 32 instructions per value, issued at about 48 % of the rate (waits on tensor and shared
 // memory take the rest; the memory traffic alone would take 117 us for 4 x 540 x 960 x 192). That size takes 704 us; with quarters of a pixel row in different
 // warps, CTA-wide barriers between the phases and 59 instructions per value it took 1561.
 // Straight code beyond the instruction cache is what costs next: with the exact

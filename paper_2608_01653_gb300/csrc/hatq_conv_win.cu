@@ -109,7 +109,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         for (int s = 0; s < kRegions; ++s) {
             mbar_init(acc_full(s), 1);
-            mbar_init(acc_empty(s), (kSplit ? 8 : 4) * (PAIR ? 2 : 1));   // epilogue warps
+            // epilogue warps that read the region (a tile of 32 columns is the first warpgroup's alone)
+            mbar_init(acc_empty(s), (kSplit && a.n_t > G / 2 ? 8 : 4) * (PAIR ? 2 : 1));
         }
         *abort_flag = 0;
         fence_barrier_init();
@@ -476,6 +477,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 uint32_t part[kDrain ? NP : 1][kDrain ? H : 1];   // exact int32 sums of the drained chunks
                 // groups of this warp: columns (2 gr + wg) H .. + H - 1 (tiles of 32-wide groups may hold an odd number)
                 const int ng = (a.n_t / H - wg + 1) / 2;
+                if (ng == 0) continue;                     // n_t = 32: the other warpgroup has the tile to itself
                 for (int ch = 0; kDrain && ch + 1 < a.nch; ++ch) {
                     const int gc = j * a.nch + ch, reg = gc & 1;
                     if (ok) ok = __all_sync(0xffffffffu, mbar_wait(acc_full(reg), (gc >> 1) & 1, abort_flag, a.err));
@@ -499,16 +501,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     tc_fence_before();
                     release(reg);
-                }
-                if (ng == 0) {                             // n_t = 32: the other warpgroup has the tile
-                    // (released only after a wait like every region: an arrival ahead of the chunk would
-                    // let two of this warp's stand for one of a warp that still reads the region)
-                    const int gl = j * a.nch + a.nch - 1, rl = gl & (kRegions - 1);
-                    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(acc_full(rl), (gl >> kRegLog) & 1, abort_flag, a.err));
-                    tc_fence_after();
-                    tc_fence_before();
-                    release(rl);
-                    continue;
                 }
                 // the last chunk's region; with 2128 both chunks of the tile still sit in regions of their own
                 const int gc = j * a.nch + a.nch - 1, reg = gc & (kRegions - 1), reg0 = (gc - 1) & (kRegions - 1);
